@@ -140,10 +140,8 @@ ht_status engine_configure(Engine &E, std::string *why)
     f.HC = std::max(t.fill_HC ? t.fill_HC : 2048u, 2 * f.threads);   // hits staged per chunk
     f.pitch16 = round_up((b.n_b + 1) / 2, 32);
     f.pitch32 = round_up(b.n_b, 32);
-    f.beta_words = round_up(b.n_b + 1, 4);
     f.dyn = 1;   // the last items are handed out at run time (htk::dyn_items)
     f.vote_weight = htk::kVoteWeight;
-    const size_t beta_bytes = (size_t)f.beta_words * 4;
     if (t.fill_W && (t.fill_W & (t.fill_W - 1))) {
         *why = "fill_rows must be a power of two";
         return HT_E_INVAL;
@@ -169,7 +167,7 @@ ht_status engine_configure(Engine &E, std::string *why)
         while (W > 2 && (size_t)W * f.pitch16 * 4 > 64 * 1024)
             W >>= 1;
     }
-    while (W > 2 && (size_t)W * f.pitch16 * 4 + (size_t)f.HC * 16 + beta_bytes > kSmemMax)
+    while (W > 2 && (size_t)W * f.pitch16 * 4 + (size_t)f.HC * 8 > kSmemMax)
         W >>= 1;
     f.W = W;
     f.tile_words = W * f.pitch16;
@@ -508,6 +506,21 @@ ht_status engine_create(Engine &E, const ht_binning *b, const ht_ranges *r, uint
     g.db = htg::delta(r->b_min, r->b_max, b->n_b);
     g.nbf = (float)b->n_b;
     g.inv_db = (float)(1.0 / (double)g.db);
+    {   // the linear model of the votes (htk::vote_line)
+        const double da = g.da, db = g.db, e24 = std::ldexp(1.0, -24);
+        const double Ra = da * b->n_a, Am = std::max(std::fabs((double)r->a_min), std::fabs((double)r->a_max)) + da,
+                     Bm = std::max(std::fabs((double)r->b_min), std::fabs((double)r->b_max)) + db;
+        auto two = [](double v, float &hi, float &lo) {
+            hi = (float)v;
+            lo = (float)(v - (double)hi);
+        };
+        g.mid = (int)(b->n_a / 2);
+        two(-2.0 * da / db, g.lin_v, g.lin_vl);
+        two(-2.0 * ((double)r->a_min + (g.mid + 0.5) * da), g.lin_a, g.lin_al);
+        two(1.0 / db, g.lin_s, g.lin_sl);
+        g.err_v = std::nextafter((float)(1.5 * e24 * (5.1 * Ra + 4.0 * Am) / (2.0 * da)), INFINITY);
+        g.err_half = std::nextafter((float)(0.5 - 1.5 * e24 * (2.0 * Bm / db + 4.0 * b->n_b + 8.0)), -INFINITY);
+    }
     E.bth.resize(b->n_b + 1);
     htg::b_thresholds(g.b_min, g.db, b->n_b, E.bth.data());
 
@@ -539,6 +552,7 @@ ht_status engine_create(Engine &E, const ht_binning *b, const ht_ranges *r, uint
         (e = dalloc(&E.d_codes, hits_cap * 4, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_slice, (3 * units + 1) * 4, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_list, (size_t)list_cap * 16, &acc)) != cudaSuccess ||
+        (e = dalloc(&E.d_lines, ((size_t)list_cap + 2) * 8, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_entries, (size_t)s.entries_cap * 16, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_ctr, (size_t)ctr_words * 4, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_split, (size_t)E.split_cap * 8, &acc)) != cudaSuccess) {
@@ -617,6 +631,7 @@ void engine_destroy(Engine &E)
     cudaFree(E.d_slice);
     cudaFree(E.d_split);
     cudaFree(E.d_list);
+    cudaFree(E.d_lines);
     cudaFree(E.d_edge);
     cudaFree(E.d_entries);
     cudaFree(E.d_book);
@@ -628,6 +643,7 @@ void engine_destroy(Engine &E)
     E.d_slice = nullptr;
     E.d_split = nullptr;
     E.d_list = nullptr;
+    E.d_lines = nullptr;
     E.d_edge = nullptr;
     E.edge_pass = 0;
     E.d_entries = nullptr;
@@ -657,6 +673,7 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
     w.slice_fill = E.d_slice + units;
     w.slice_off = E.d_slice + 2 * units;
     w.list = E.d_list;
+    w.lines = E.d_lines;
     w.list_cap = E.list_cap;
     w.edge = E.d_edge;
     w.edge_pass = E.edge_pass;

@@ -108,6 +108,7 @@ struct Engine {
     uint32_t edge_pass = 0;       // passes per unit the edge buffer holds
     uint32_t *d_slice = nullptr;  // unit counts | scatter cursors | offsets (3 * units + 1)
     float4 *d_list = nullptr;     // hit records unit by unit
+    float2 *d_lines = nullptr;    // their vote lines
     uint32_t list_cap = 0;
     uint4 *d_entries = nullptr;
     void *d_book = nullptr;       // desc | cta arrays

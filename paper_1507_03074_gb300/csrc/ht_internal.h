@@ -17,11 +17,10 @@ struct FillCfg {
     uint32_t strips;      // ceil(n_a / W)
     uint32_t pitch16;     // tile words per row in u16 mode (multiple of 32)
     uint32_t pitch32;     // tile words per row in u32 mode (multiple of 32)
-    uint32_t HC;          // hits staged in shared memory per chunk (>= 2 * threads)
+    uint32_t HC;          // vote lines staged in shared memory per chunk
     uint32_t tile_words;  // W * pitch16
     uint32_t threads;     // block size
     uint32_t accumulate;  // add the tile to M_H instead of storing it
-    uint32_t beta_words;  // shared-memory copy of the B-bin thresholds (n_b + 1, rounded to 4)
     uint32_t dyn;         // 1: the last dyn_items() items are handed out at run time (see below)
     uint32_t bulk;        // fused fill: 1 = passes leave through u32 staging and bulk copies (k_fill_bulk)
     uint32_t vote_weight; // cost of one vote against one cell written, in the static split (cta_items)

@@ -249,12 +249,15 @@ __global__ void __launch_bounds__(256) k_scatter(Geom g, Work w)
         if (code == kDropped)
             continue;
         const float4 hv = w.hits4[h];
+        const float2 line = vote_line(g, hv.x, hv.y, hv.z);
         const uint32_t e = __float_as_uint(hv.w);
         for_each_slice(g, code, [&](uint32_t s) {
             const uint32_t u = e * g.n_slices + s;
             const uint32_t idx = w.slice_off[u] + atomicAdd(&w.slice_fill[u], 1u);
-            if (idx < w.list_cap)
+            if (idx < w.list_cap) {
                 w.list[idx] = hv;
+                w.lines[idx] = line;
+            }
         });
     }
     const uint32_t U = w.n_events * g.n_slices;
@@ -441,10 +444,13 @@ __global__ void __launch_bounds__(1024, 1) k_bin_cluster(Geom g, Work w)
 #pragma unroll
     for (uint32_t q = 0; q < kBinClusterHPT; ++q) {
         const uint32_t e = ev[q];
+        const float2 line = vote_line(g, hv[q].x, hv[q].y, hv[q].z);
         for_each_slice(g, code[q], [&](uint32_t s) {
             const uint32_t idx = atomicAdd(&s_pl[e * g.n_slices + s], 1u);
-            if (idx < w.list_cap)
+            if (idx < w.list_cap) {
                 w.list[idx] = hv[q];
+                w.lines[idx] = line;
+            }
         });
     }
     if (rank == 0 && w.split_mode == kSplitGiven)
@@ -490,40 +496,38 @@ __device__ __forceinline__ void note_candidate(const FlushList &L, uint32_t r, u
         L.cand[p] = key;
 }
 
-// Votes of hits hs[hl], hs[hl + hstride], .. < nc into tile row r (A bin i).
+// Votes of hits hs[hl], hs[hl + hstride], .. < nc (the vote lines of the
+// records rec[0 .. nc)) into tile row r (A bin i).
 // With LIST, a vote that lifts its cell from T - 1 to T lists the cell
 // (note_candidate): votes are +1 increments and T >= 1 (the context
 // rejects T = 0), so every cell >= T is listed exactly once.
 template <bool U16, bool LIST = false>
-__device__ __forceinline__ void vote_rows(const Geom &g, uint32_t *tile, const float4 *hs, const float *beta,
+__device__ __forceinline__ void vote_rows(const Geom &g, uint32_t *tile, const float2 *hs, const float4 *rec,
                                           uint32_t nc, uint32_t r, uint32_t i, uint32_t hl, uint32_t hstride,
                                           uint32_t pitch, const FlushList &L = FlushList{})
 {
-    const float twoA = __fmul_rn(2.0f, a_centre(g, i));
     const uint32_t rowbase = r * pitch;
     const uint32_t sw = U16 ? (row_hash(r) & 0x1Eu) : (row_hash(r) & 0x1Cu);
-    const float b_lo = beta[0], b_hi = beta[g.nb];   // the in-range test of every vote
     const uint32_t tm1 = g.threshold - 1u;
 #pragma unroll 4
     for (uint32_t h = hl; h < nc; h += hstride) {
-        const float4 hv = hs[h];
-        const int j = vote_bin_tab(g, beta, b_lo, b_hi, twoA, hv.x, hv.y, hv.z);
-        if (j >= 0) {
+        const uint32_t j = vote_bin_line(g, hs[h], i, rec + h);
+        if (j < g.nb) {
             if (U16) {
-                const uint32_t word = rowbase + ((uint32_t(j) >> 1) ^ sw);
-                const uint32_t sh = (uint32_t(j) & 1u) << 4;
+                const uint32_t word = rowbase + ((j >> 1) ^ sw);
+                const uint32_t sh = (j & 1u) << 4;
                 if (LIST) {
                     if (((atomicAdd(&tile[word], 1u << sh) >> sh) & 0xffffu) == tm1)
-                        note_candidate(L, r, r * g.nb + uint32_t(j));
+                        note_candidate(L, r, r * g.nb + j);
                 } else {
                     atomicAdd(&tile[word], 1u << sh);
                 }
             } else {
                 if (LIST) {
-                    if (atomicAdd(&tile[rowbase + (uint32_t(j) ^ sw)], 1u) == tm1)
-                        note_candidate(L, r, r * g.nb + uint32_t(j));
+                    if (atomicAdd(&tile[rowbase + (j ^ sw)], 1u) == tm1)
+                        note_candidate(L, r, r * g.nb + j);
                 } else {
-                    atomicAdd(&tile[rowbase + (uint32_t(j) ^ sw)], 1u);
+                    atomicAdd(&tile[rowbase + (j ^ sw)], 1u);
                 }
             }
         }
@@ -635,21 +639,21 @@ __device__ __forceinline__ void flush_tile(const Geom &g, uint32_t *tile, uint32
     }
 }
 
-// Copy up to cap hit records of a unit's list, from list index pos on (pos
+// Copy up to cap vote lines of a unit's list, from list index pos on (pos
 // < end), into hs; advances pos.  All threads of the group call it.
 template <class G = BlockGroup>
-__device__ __forceinline__ uint32_t stage_hits(const Work &w, float4 *hs, uint32_t cap, uint32_t &pos, uint32_t end)
+__device__ __forceinline__ uint32_t stage_hits(const Work &w, float2 *hs, uint32_t cap, uint32_t &pos, uint32_t end)
 {
     G::sync();   // the previous readers of hs are done
     const uint32_t n = min(cap, end - pos);
     constexpr uint32_t U = 4;
     for (uint32_t k0 = 0; k0 < n; k0 += U * G::size()) {
-        float4 v[U];
+        float2 v[U];
 #pragma unroll
         for (uint32_t q = 0; q < U; ++q) {
             const uint32_t k = k0 + q * G::size() + G::rank();
             if (k < n)
-                v[q] = __ldg(&w.list[pos + k]);
+                v[q] = __ldg(&w.lines[pos + k]);
         }
 #pragma unroll
         for (uint32_t q = 0; q < U; ++q) {
@@ -670,8 +674,8 @@ __device__ __forceinline__ uint32_t stage_hits(const Work &w, float4 *hs, uint32
 // (the previous pass's readers of the tile are done); without it the caller
 // orders the tile by other means.  All threads of the group call it.
 template <class G, bool SYNC, bool LIST>
-__device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t *tile, float4 *hs, const float *beta,
-                                          uint32_t HC, uint64_t es, uint32_t l0, uint32_t l1, uint64_t &cached_es,
+__device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t *tile, float2 *hs, uint32_t HC,
+                                          uint64_t es, uint32_t l0, uint32_t l1, uint64_t &cached_es,
                                           uint32_t &cached_n, bool u16, uint32_t r, uint32_t pr, uint32_t i,
                                           uint32_t hl, uint32_t hstride, uint32_t pitch, const FlushList &L)
 {
@@ -680,9 +684,9 @@ __device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t
             G::sync();
         if (r < pr) {
             if (u16)
-                vote_rows<true, LIST>(g, tile, hs, beta, cached_n, r, i, hl, hstride, pitch, L);
+                vote_rows<true, LIST>(g, tile, hs, w.list + l0, cached_n, r, i, hl, hstride, pitch, L);
             else
-                vote_rows<false, LIST>(g, tile, hs, beta, cached_n, r, i, hl, hstride, pitch, L);
+                vote_rows<false, LIST>(g, tile, hs, w.list + l0, cached_n, r, i, hl, hstride, pitch, L);
         }
         return;
     }
@@ -690,6 +694,7 @@ __device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t
     uint32_t pos = l0;
     bool first = true;
     while (first || pos < l1) {
+        const float4 *rec = w.list + pos;
         const uint32_t nsel = stage_hits<G>(w, hs, HC, pos, l1);
         if (first && pos >= l1) {
             cached_es = es;   // the whole list fits: keep it
@@ -698,9 +703,9 @@ __device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t
         first = false;
         if (r < pr) {
             if (u16)
-                vote_rows<true, LIST>(g, tile, hs, beta, nsel, r, i, hl, hstride, pitch, L);
+                vote_rows<true, LIST>(g, tile, hs, rec, nsel, r, i, hl, hstride, pitch, L);
             else
-                vote_rows<false, LIST>(g, tile, hs, beta, nsel, r, i, hl, hstride, pitch, L);
+                vote_rows<false, LIST>(g, tile, hs, rec, nsel, r, i, hl, hstride, pitch, L);
         }
     }
 }
@@ -834,14 +839,11 @@ __global__ void __launch_bounds__(1024) k_fill_priv(Geom g, Work w, FillCfg c)
 {
     extern __shared__ uint4 sm4[];
     uint32_t *tile = reinterpret_cast<uint32_t *>(sm4);
-    float4 *hs = reinterpret_cast<float4 *>(tile + c.tile_words);
-    float *beta = reinterpret_cast<float *>(hs + c.HC);
+    float2 *hs = reinterpret_cast<float2 *>(tile + c.tile_words);
 
     const uint32_t tid = threadIdx.x, bd = blockDim.x;
     for (uint32_t k = tid; k < c.tile_words / 4; k += bd)
         sm4[k] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t k = tid; k <= g.nb; k += bd)
-        beta[k] = g.bth[k];
     grid_dep_wait();   // the unit lists of k_scatter
 
     __shared__ unsigned long long s_rng[2];
@@ -871,7 +873,7 @@ __global__ void __launch_bounds__(1024) k_fill_priv(Geom g, Work w, FillCfg c)
         for (uint32_t p0 = 0; p0 < rows; p0 += rpass) {
             const uint32_t pr = min(rpass, rows - p0);
             const uint32_t i = i0 + p0 + r;
-            vote_pass<BlockGroup, true, false>(g, w, tile, hs, beta, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
+            vote_pass<BlockGroup, true, false>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
                                                i, hl, hstride, pitch, FlushList{});
             __syncthreads();
             uint32_t *dst = Mrow + (size_t)p0 * g.nb;
@@ -1494,21 +1496,18 @@ __device__ __forceinline__ void fill_scan_body(const Geom &g, const Work &w, con
 {
     extern __shared__ uint4 sm4[];
     // layout: ScanSmem (256 B) | K entries | tile | [BULK: 2 staging buffers] | HC staged hits |
-    //         B thresholds | candidate lists (keys, votes, sorted keys, sorted votes)
+    //         candidate lists (keys, votes, sorted keys, sorted votes)
     ScanSmem &ss = *reinterpret_cast<ScanSmem *>(sm4);
     uint4 *pbuf = sm4 + 16;
     uint32_t *tile = reinterpret_cast<uint32_t *>(pbuf + a.K);
     uint32_t *stg = tile + c.tile_words;
-    float4 *hs = reinterpret_cast<float4 *>(stg + (BULK ? staging_words(c, g.nb) : 0u));
-    float *beta = reinterpret_cast<float *>(hs + c.HC);
-    uint32_t *lists = reinterpret_cast<uint32_t *>(beta + c.beta_words);
+    float2 *hs = reinterpret_cast<float2 *>(stg + (BULK ? staging_words(c, g.nb) : 0u));
+    uint32_t *lists = reinterpret_cast<uint32_t *>(hs + c.HC);
     __shared__ uint32_t s_hot[2], s_nc;
 
     const uint32_t tid = threadIdx.x, bd = blockDim.x, nb = g.nb;
     for (uint32_t k = tid; k < c.tile_words / 4; k += bd)
         sm4[16 + a.K + k] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t k = tid; k <= nb; k += bd)
-        beta[k] = g.bth[k];
     grid_dep_wait();   // the unit lists of k_scatter
     const uint32_t cta = blockIdx.x;
     ChunkList inner = interior_list(a, cta);
@@ -1546,7 +1545,7 @@ __device__ __forceinline__ void fill_scan_body(const Geom &g, const Work &w, con
             // ---- vote (no barrier first: the previous pass, the previous item's
             // hand-out or the set-up ended with one) ---------------------------
             const uint32_t i = iA + r;
-            vote_pass<BlockGroup, false, false>(g, w, tile, hs, beta, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
+            vote_pass<BlockGroup, false, false>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
                                                 i, hl, hstride, pitch, FlushList{});
             // ---- write the pass, clear the tile, emit its candidates --------
             if (BULK) {
@@ -1631,7 +1630,7 @@ struct FlatMap {
     }
 };
 
-// The votes of the staged hits hs[0 .. m.nc) into tile rows 0 .. pr - 1 (A
+// The votes of the staged hits hs[0 .. m.nc) (the lines of rec[0 .. m.nc)) into tile rows 0 .. pr - 1 (A
 // bins iA ..): candidate q = r * nc + h goes to thread q % blockDim, so a
 // warp's lanes take consecutive hits of one row (their B columns, and so
 // their banks, are spread by the hits).  A vote that lifts its cell from
@@ -1640,22 +1639,19 @@ struct FlatMap {
 // cell index) and their lowest lane adds their number with one atomic; the
 // cell is listed by the add that takes it from below T to T or more.
 template <bool AGG>
-__device__ __forceinline__ void vote_flat(const Geom &g, uint32_t *tile, const float4 *hs, const float *beta,
+__device__ __forceinline__ void vote_flat(const Geom &g, uint32_t *tile, const float2 *hs, const float4 *rec,
                                           const FlatMap &m, uint32_t pr, uint32_t iA, const FlushList &L)
 {
     const uint32_t nb = g.nb, nc = m.nc;
     if (nc == 0 || m.r0 >= pr)
         return;
     const uint32_t T = g.threshold, tm1 = T - 1u, lane = threadIdx.x & 31u;
-    const float b_lo = beta[0], b_hi = beta[nb];
     uint32_t r = m.r0, h = m.h0;
 #pragma unroll 2
     while (r < pr) {
-        const float twoA = __fmul_rn(2.0f, a_centre(g, iA + r));
-        const float4 hv = hs[h];
-        const int j = vote_bin_tab(g, beta, b_lo, b_hi, twoA, hv.x, hv.y, hv.z);
-        if (j >= 0) {
-            const uint32_t key = r * nb + (uint32_t)j;
+        const uint32_t j = vote_bin_line(g, hs[h], iA + r, rec + h);
+        if (j < nb) {
+            const uint32_t key = r * nb + j;
             if (AGG) {
                 const uint32_t peers = __match_any_sync(__activemask(), key);
                 if (lane == (uint32_t)(__ffs(peers) - 1)) {
@@ -1683,20 +1679,20 @@ __device__ __forceinline__ void vote_flat(const Geom &g, uint32_t *tile, const f
 // case: the previous pass's clearing of this tile is complete.  All threads
 // call it.
 template <bool AGG>
-__device__ __forceinline__ void vote_pass_flat(const Geom &g, const Work &w, uint32_t *tile, float4 *hs,
-                                               const float *beta, uint32_t HC, uint64_t es, uint32_t l0, uint32_t l1,
-                                               uint64_t &cached_es, FlatMap &cached, uint32_t pr, uint32_t iA,
-                                               const FlushList &L)
+__device__ __forceinline__ void vote_pass_flat(const Geom &g, const Work &w, uint32_t *tile, float2 *hs, uint32_t HC,
+                                               uint64_t es, uint32_t l0, uint32_t l1, uint64_t &cached_es,
+                                               FlatMap &cached, uint32_t pr, uint32_t iA, const FlushList &L)
 {
     if (cached_es == es) {
         __syncthreads();
-        vote_flat<AGG>(g, tile, hs, beta, cached, pr, iA, L);
+        vote_flat<AGG>(g, tile, hs, w.list + l0, cached, pr, iA, L);
         return;
     }
     cached_es = ~0ull;   // hs is about to be overwritten
     uint32_t pos = l0;
     bool first = true;
     while (first || pos < l1) {
+        const float4 *rec = w.list + pos;
         const uint32_t nsel = stage_hits<BlockGroup>(w, hs, HC, pos, l1);   // starts with a barrier
         FlatMap m;
         m.set(nsel);
@@ -1705,7 +1701,7 @@ __device__ __forceinline__ void vote_pass_flat(const Geom &g, const Work &w, uin
             cached = m;
         }
         first = false;
-        vote_flat<AGG>(g, tile, hs, beta, m, pr, iA, L);
+        vote_flat<AGG>(g, tile, hs, rec, m, pr, iA, L);
     }
 }
 
@@ -1717,14 +1713,13 @@ __global__ void __launch_bounds__(1024) k_fill_tma(Geom g, Work w, FillCfg c, Sc
 {
     constexpr int NT = 2;
     extern __shared__ uint4 sm4[];
-    // layout: ScanSmem (256 B) | K entries | NT tiles | HC staged hits | B thresholds |
+    // layout: ScanSmem (256 B) | K entries | NT tiles | HC staged vote lines |
     //         candidate lists (keys, votes, sorted keys, sorted votes)
     ScanSmem &ss = *reinterpret_cast<ScanSmem *>(sm4);
     uint4 *pbuf = sm4 + 16;
     uint32_t *tiles = reinterpret_cast<uint32_t *>(pbuf + a.K);
-    float4 *hs = reinterpret_cast<float4 *>(tiles + NT * c.tile_words);
-    float *beta = reinterpret_cast<float *>(hs + c.HC);
-    uint32_t *lists = reinterpret_cast<uint32_t *>(beta + c.beta_words);
+    float2 *hs = reinterpret_cast<float2 *>(tiles + NT * c.tile_words);
+    uint32_t *lists = reinterpret_cast<uint32_t *>(hs + c.HC);
     uint32_t *cand = lists, *candv = lists + kFusedCand, *srt = lists + 2 * kFusedCand,
              *srtv = lists + 3 * kFusedCand;
     __shared__ uint32_t s_hot[2], s_nc;
@@ -1732,8 +1727,6 @@ __global__ void __launch_bounds__(1024) k_fill_tma(Geom g, Work w, FillCfg c, Sc
     const uint32_t tid = threadIdx.x, bd = blockDim.x, nb = g.nb;
     for (uint32_t k = tid; k < NT * c.tile_words / 4; k += bd)
         reinterpret_cast<uint4 *>(tiles)[k] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t k = tid; k <= nb; k += bd)
-        beta[k] = g.bth[k];
     if (tid == 0)
         s_hot[0] = s_hot[1] = s_nc = 0u;
     const uint32_t cta = blockIdx.x;
@@ -1774,7 +1767,7 @@ __global__ void __launch_bounds__(1024) k_fill_tma(Geom g, Work w, FillCfg c, Sc
         uint32_t *tile = tiles + (size_t)tsel * c.tile_words;
 
         // ---- vote (tile tsel is clear, the lists empty) ------------------------
-        vote_pass_flat<AGG>(g, w, tile, hs, beta, c.HC, es, l0, l1, cached_es, cached, pr, iA,
+        vote_pass_flat<AGG>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached, pr, iA,
                        FlushList{s_hot, cand, candv, &s_nc, kFusedCand});
         fence_proxy_async_smem();   // the tile's counts, visible to the copy engine
         __syncthreads();            // votes and lists complete
@@ -1906,9 +1899,8 @@ __global__ void __launch_bounds__(1024) k_fill_peaks(Geom g, Work w, FillCfg c, 
     ScanSmem &ss = *reinterpret_cast<ScanSmem *>(sm4);
     uint4 *pbuf = sm4 + 16;
     uint32_t *tile = reinterpret_cast<uint32_t *>(pbuf + a.K);
-    float4 *hs = reinterpret_cast<float4 *>(tile + c.tile_words);
-    float *beta = reinterpret_cast<float *>(hs + c.HC);
-    uint32_t *lists = reinterpret_cast<uint32_t *>(beta + c.beta_words);
+    float2 *hs = reinterpret_cast<float2 *>(tile + c.tile_words);
+    uint32_t *lists = reinterpret_cast<uint32_t *>(hs + c.HC);
     uint32_t *cand = lists, *srt = lists + 2 * kFusedCand, *srtv = lists + 3 * kFusedCand;
     __shared__ uint32_t s_hot[2], s_nc;
 
@@ -1917,8 +1909,6 @@ __global__ void __launch_bounds__(1024) k_fill_peaks(Geom g, Work w, FillCfg c, 
         s_hot[0] = s_hot[1] = s_nc = 0u;
     for (uint32_t k = tid; k < c.tile_words / 4; k += bd)
         sm4[16 + a.K + k] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t k = tid; k <= nb; k += bd)
-        beta[k] = g.bth[k];
     const uint32_t cta = blockIdx.x;
     ChunkList inner = interior_list(a, cta);
 
@@ -1963,7 +1953,7 @@ __global__ void __launch_bounds__(1024) k_fill_peaks(Geom g, Work w, FillCfg c, 
             // ---- vote -------------------------------------------------------
             const uint32_t i = iA + r;
             const FlushList L{s_hot, lists, nullptr, &s_nc, kFusedCand};
-            vote_pass<BlockGroup, true, true>(g, w, tile, hs, beta, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
+            vote_pass<BlockGroup, true, true>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
                                               i, hl, hstride, pitch, L);
             __syncthreads();   // the pass's votes and their candidate list are complete
             const uint32_t n_c = s_nc;
@@ -2090,22 +2080,19 @@ __device__ __forceinline__ ItemInfo item_info(const Geom &g, const Work &w, cons
 __global__ void __launch_bounds__(1024, 1) k_fill_ws(Geom g, Work w, FillCfg c, ScanArgs a)
 {
     extern __shared__ uint4 sm4[];
-    // layout: ScanSmem (256 B) | K entries | 2 tiles | HC staged hits | B thresholds |
+    // layout: ScanSmem (256 B) | K entries | 2 tiles | HC staged vote lines |
     //         candidate lists | 4 mbarriers (FULL 0, FULL 1, EMPTY 0, EMPTY 1)
     ScanSmem &ss = *reinterpret_cast<ScanSmem *>(sm4);
     uint4 *pbuf = sm4 + 16;
     uint32_t *tiles = reinterpret_cast<uint32_t *>(pbuf + a.K);
-    float4 *hs = reinterpret_cast<float4 *>(tiles + 2 * (size_t)c.tile_words);
-    float *beta = reinterpret_cast<float *>(hs + c.HC);
-    uint32_t *lists = reinterpret_cast<uint32_t *>(beta + c.beta_words);
+    float2 *hs = reinterpret_cast<float2 *>(tiles + 2 * (size_t)c.tile_words);
+    uint32_t *lists = reinterpret_cast<uint32_t *>(hs + c.HC);
     uint64_t *bars = reinterpret_cast<uint64_t *>(lists + 4 * kFusedCand);
     __shared__ uint32_t s_hot[2], s_nc;
 
     const uint32_t tid = threadIdx.x, nb = g.nb;
     for (uint32_t k = tid; k < c.tile_words / 2; k += blockDim.x)
         reinterpret_cast<uint4 *>(tiles)[k] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t k = tid; k <= nb; k += blockDim.x)
-        beta[k] = g.bth[k];
     if (tid == 0) {
         for (uint32_t q = 0; q < 4; ++q)
             mbar_init(&bars[q], VoteGroup::size());
@@ -2142,7 +2129,7 @@ __global__ void __launch_bounds__(1024, 1) k_fill_ws(Geom g, Work w, FillCfg c, 
                     }
                 }
                 const uint32_t i = t.i0 + p0 + r;
-                vote_pass<VoteGroup, false, false>(g, w, tile, hs, beta, c.HC, t.es, t.l0, t.l1, cached_es, cached_n,
+                vote_pass<VoteGroup, false, false>(g, w, tile, hs, c.HC, t.es, t.l0, t.l1, cached_es, cached_n,
                                                    t.u16, r, pr, i, hl, hstride, t.pitch, FlushList{});
                 mbar_arrive(&bars[b]);   // tile b holds pass p
             }
@@ -2650,7 +2637,7 @@ cudaError_t launch_bin_cluster(const Geom &g, const Work &w, uint32_t cs, cudaSt
 size_t fill_scan_smem_bytes(const FillCfg &c, const ScanArgs &a, uint32_t nb)
 {
     return 16 * sizeof(uint4) + (size_t)a.K * sizeof(uint4) + (size_t)c.tile_words * 4 +
-           (size_t)staging_words(c, nb) * 4 + (size_t)c.HC * 16 + (size_t)c.beta_words * 4 +
+           (size_t)staging_words(c, nb) * 4 + (size_t)c.HC * 8 +
            (size_t)4 * kFusedCand * 4;
 }
 
@@ -2668,8 +2655,8 @@ cudaError_t launch_fill_scan(const Geom &g, const Work &w, const FillCfg &c, con
 
 size_t fill_ws_smem_bytes(const FillCfg &c, const ScanArgs &a)
 {
-    return 16 * sizeof(uint4) + (size_t)a.K * sizeof(uint4) + (size_t)2 * c.tile_words * 4 + (size_t)c.HC * 16 +
-           (size_t)c.beta_words * 4 + (size_t)4 * kFusedCand * 4 + 4 * sizeof(uint64_t);
+    return 16 * sizeof(uint4) + (size_t)a.K * sizeof(uint4) + (size_t)2 * c.tile_words * 4 + (size_t)c.HC * 8 +
+           (size_t)4 * kFusedCand * 4 + 4 * sizeof(uint64_t);
 }
 
 cudaError_t launch_fill_ws(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
@@ -2710,7 +2697,7 @@ cudaError_t launch_fill_peaks(const Geom &g, const Work &w, const FillCfg &c, co
 size_t fill_tma_smem_bytes(const FillCfg &c, const ScanArgs &a)
 {
     return 16 * sizeof(uint4) + (size_t)a.K * sizeof(uint4) + (size_t)2 * c.tile_words * 4 +
-           (size_t)c.HC * 16 + (size_t)c.beta_words * 4 + (size_t)4 * kFusedCand * 4;
+           (size_t)c.HC * 8 + (size_t)4 * kFusedCand * 4;
 }
 
 cudaError_t launch_fill_tma(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
@@ -2747,7 +2734,7 @@ cudaError_t fill_scan_occupancy(const FillCfg &c, const ScanArgs &a, uint32_t nb
 
 size_t fill_smem_bytes(const FillCfg &c)
 {
-    return (size_t)c.tile_words * 4 + (size_t)c.HC * 16 + (size_t)c.beta_words * 4;
+    return (size_t)c.tile_words * 4 + (size_t)c.HC * 8;
 }
 
 cudaError_t launch_fill_priv(const Geom &g, const Work &w, const FillCfg &c, uint32_t grid,
