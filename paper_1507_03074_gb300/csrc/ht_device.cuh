@@ -58,6 +58,11 @@ struct Work {
     float4 *list;               // list_cap hit records {x, x^2 + y^2, 2y, event}, unit by unit
     float2 *lines;              // [list_cap + 2] the records' vote lines (vote_line), unit by unit as list
     uint32_t list_cap;
+    // k_fill_tma's peaks: {first entry, count} of every pass, and their number in
+    // every kOrderPasses passes (the binning clears the n_seg counts)
+    uint2 *pass_peaks;
+    uint32_t *seg_peaks;
+    uint32_t n_seg;
     // peaks-only fills: the first and last row of every strip pass,
     // [unit][edge_pass][2][n_b] (pass p of a unit covers rows p * rpass ..)
     uint32_t *edge;
@@ -294,14 +299,15 @@ __device__ __forceinline__ float2 vote_line(const Geom &g, float x, float r2, fl
 }
 
 // The bin of the vote of record *rec, whose line is l, in A bin i; n_b or
-// more when it is out of range.  Adding 1.5 * 2^23 rounds t - 1/2 to the
+// more when it is out of range.  on: the record is there (else l is no_line).  Adding 1.5 * 2^23 rounds t - 1/2 to the
 // nearest whole number, which is floor(t) except next to an edge, in the low
 // bits of the sum; whatever lies far outside ends up above n_b.  About one vote
 // in a thousand of a paper-scale event takes the rule.  Against a division and
 // two table look-ups per vote (events with three contexts in flight): 114.9
 // against 143.0 us with admission windows of one bin (27 M votes), 593.7
 // against 648.2 us for an upgrade event, 49.4 against 50.4 us for a paper event.
-__device__ __forceinline__ uint32_t vote_bin_line(const Geom &g, const float2 l, uint32_t i, const float4 *rec)
+__device__ __forceinline__ uint32_t vote_bin_line(const Geom &g, const float2 l, uint32_t i, const float4 *rec,
+                                                  bool on = true)
 {
     const float big = 12582912.0f;
     const float t = __fmaf_rn(l.y, __int2float_rn((int)i - g.mid), l.x);
@@ -309,7 +315,7 @@ __device__ __forceinline__ uint32_t vote_bin_line(const Geom &g, const float2 l,
     const float r = __fsub_rn(t, __fsub_rn(k, big));
     uint32_t j = __float_as_uint(k) - __float_as_uint(big);
     const float lim = __fmaf_rn(-g.err_v, fabsf(l.y), g.err_half);
-    if (!(fabsf(r) <= lim) && (j + 1u <= g.nb + 1u || !(lim > 0.0f))) {
+    if (!(fabsf(r) <= lim) && (j + 1u <= g.nb + 1u || !(lim > 0.0f)) && on) {
         const float4 h = __ldg(rec);
         j = (uint32_t)vote_bin(g, __fmul_rn(2.0f, a_centre(g, i)), h.x, h.y, h.z);
     }

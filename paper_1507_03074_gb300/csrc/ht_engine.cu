@@ -150,16 +150,23 @@ ht_status engine_configure(Engine &E, std::string *why)
     // it) fill_rows sizes its tiles; the other fills (accumulating, peaks-only)
     // keep their own tile height
     bool tma_mode = (t.fused == 5 || t.fused == 0) && (b.n_b & 3u) == 0 && b.n_b <= 4096;
-    if (tma_mode && t.fill_W) {
-        // a requested tile height the bulk-copy-tile fill cannot hold leaves it to the others
-        htk::FillCfg probe = f;
-        probe.W = t.fill_W;
-        probe.tile_words = t.fill_W * b.n_b;
-        probe.HC = 2 * f.threads;
-        htk::ScanArgs tmp{};
-        tmp.K = std::max<uint32_t>(kFusedPeakBuf, f.threads);
-        tma_mode = t.fill_W <= 64 && htk::fill_tma_smem_bytes(probe, tmp) <= kSmemMax;
-    }
+    // the tile fill's shape at W rows per pass: as many of fill_threads' warps as
+    // their tiles fit, twice per SM unless the threads were asked for
+    auto tile_shape = [&](uint32_t W) {
+        htk::TileCfg c{};
+        c.threads = t.fill_threads ? t.fill_threads : 256;
+        c.W = W;
+        c.strips = (b.n_a + W - 1) / W;
+        c.tile_words = round_up(std::max<uint32_t>(W, 2) * b.n_b + 3, 4);
+        c.vote_agg = t.vote_agg;
+        c.warps = std::min<uint32_t>(c.threads / 32, htk::kTileWarps);
+        while (c.warps > 1 && htk::tile_smem_bytes(c) > (t.fill_threads ? kSmemMax : kSmemMax / 2 - 1024))
+            --c.warps;
+        c.run = c.warps;
+        return c;
+    };
+    if (tma_mode && t.fill_W)   // a requested height that the tile fill cannot hold leaves it to the others
+        tma_mode = t.fill_W <= 64 && htk::tile_smem_bytes(tile_shape(t.fill_W)) <= kSmemMax;
     uint32_t W = tma_mode ? 0u : t.fill_W;
     if (!W) {
         // aim at ~64 KB tiles so that two CTAs share an SM
@@ -271,52 +278,31 @@ ht_status engine_configure(Engine &E, std::string *why)
         return HT_E_INVAL;
     }
     E.use_ws = E.ws_ok;
-    // --- fused fill with bulk-copy tiles: two u32 tiles in M_H's layout ----------
+    // --- the tile fill ------------------------------------------------------------
     E.tma_ok = false;
     E.tma_capped = false;
     // the default fused fill wherever it fits (fused 0 = auto)
     if (E.fill_priv_ok && (t.fused == 5 || t.fused == 0) && (b.n_b & 3u) == 0 && b.n_b <= 4096) {
-        htk::FillCfg tf = f;
-        tf.threads = t.fill_threads ? t.fill_threads : 512;
         uint32_t Wt = t.fill_W;
         if (!Wt) {
-            // two tiles of about 64 KB together
-            Wt = 32;
-            while (Wt > 1 && (size_t)2 * Wt * b.n_b * 4 > 64 * 1024)
+            Wt = 64;   // tiles of at most 16 KB, and lower ones while there are fewer passes than warps
+            while (Wt > 2 && ((size_t)Wt * b.n_b * 4 > 16 * 1024 ||
+                              (Wt > 4 && (uint64_t)E.max_events * g.n_slices * ((b.n_a + Wt - 1) / Wt) < 12ull * E.num_sms)))
                 Wt >>= 1;
         }
-        Wt = std::min<uint32_t>(Wt, 64);   // the hot-row mask holds 64 rows
-        tf.W = Wt;
-        tf.strips = (b.n_a + Wt - 1) / Wt;
-        tf.tile_words = Wt * b.n_b;
-        tf.vote_agg = t.vote_agg;
-        tf.bulk = 0;
-        tf.dyn = 1;
-        tf.HC = std::max(t.fill_HC ? t.fill_HC : 2048u, 2 * tf.threads);
-        htk::ScanArgs tmp{};
-        tmp.K = std::max<uint32_t>(kFusedPeakBuf, tf.threads);
-        auto occupancy = [&](const htk::FillCfg &c) {
-            int o = 0;
-            if (htk::fill_tma_smem_bytes(c, tmp) > kSmemMax || htk::fill_tma_occupancy(c, tmp, &o) != cudaSuccess) {
-                cudaGetLastError();
-                return 0;
-            }
-            return o;
-        };
-        int occ = occupancy(tf);
-        while (!t.fill_HC && occ < 2 && tf.HC > 2 * tf.threads) {
-            tf.HC -= tf.threads;
-            occ = occupancy(tf);
-        }
-        E.tma_capped = false;
-        if (occ >= 1) {
+        const htk::TileCfg c = tile_shape(std::min<uint32_t>(Wt, 64));
+        int occ = 0;
+        if (htk::tile_smem_bytes(c) <= kSmemMax &&
+            (uint64_t)E.max_events * g.n_slices * c.strips <= 0x7fffffffull &&
+            htk::fill_tma_occupancy(c, &occ) == cudaSuccess && occ >= 1) {
             E.tma_capped = t.fill_blocks_per_sm && (int)t.fill_blocks_per_sm < occ;
             if (t.fill_blocks_per_sm)
                 occ = std::min<int>(occ, (int)t.fill_blocks_per_sm);
             E.tma_ok = true;
-            E.tma_fill = tf;
-            E.tma_K = tmp.K;
+            E.tile = c;
             E.tma_grid = (uint32_t)E.num_sms * (uint32_t)occ;
+        } else {
+            cudaGetLastError();
         }
     }
     if (t.fused == 5 && !E.tma_ok) {
@@ -382,13 +368,10 @@ ht_status engine_configure(Engine &E, std::string *why)
     const uint64_t items_max = (uint64_t)E.max_events * g.n_slices * f.strips;
     const uint32_t fused_grid = E.fused_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.fused_grid, items_max)) : 0;
     const uint32_t ws_grid = E.ws_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.ws_grid, items_max)) : 0;
-    const uint64_t items_tma = E.tma_ok ? (uint64_t)E.max_events * g.n_slices * E.tma_fill.strips : 0;
-    const uint32_t tma_grid =
-        E.tma_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.tma_grid, items_tma)) : 0;
+    const uint64_t passes = E.tma_ok ? htk::tile_passes(g, E.tile, E.max_events) : 0;
     // the fused fill's candidate lists: one per CTA plus one per handed-out item
     const uint32_t fused_lists = fused_grid + (uint32_t)htk::dyn_items(items_max, fused_grid);
-    const uint32_t tma_lists = E.tma_ok ? tma_grid + (uint32_t)htk::dyn_items(items_tma, tma_grid) : 0;
-    const uint32_t grid_cap = std::max(std::max(std::max(scan_grid, fused_lists), ws_grid), tma_lists);
+    const uint32_t grid_cap = std::max(std::max(scan_grid, fused_lists), ws_grid);
     uint32_t seq = chunks_for((G_max + scan_grid - 1) / scan_grid + 1, (g.nb + 1) / 2, s.K, 2 * kScanThreads);
     // the cost-balanced split gives a CTA at most `spread` times the items of
     // an even split (every strip costs at least its n_b-per-row writing share)
@@ -403,10 +386,6 @@ ht_status engine_configure(Engine &E, std::string *why)
         seq = std::max(seq, chunks_for(fused_rows, g.nb, E.fused_K,
                                        htk::fused_round(E.fused_fill.threads, E.fused_K)));
     }
-    if (E.tma_ok) {
-        const uint64_t tma_rows = (uint64_t)(std::ceil((double)items_tma / tma_grid * spread) + 2) * E.tma_fill.W + 1;
-        seq = std::max(seq, chunks_for(tma_rows, g.nb, E.tma_K, htk::fused_round(E.tma_fill.threads, E.tma_K)));
-    }
     if (E.ws_ok) {
         const uint64_t ws_rows = rows_per_cta(ws_grid);
         seq = std::max(seq, chunks_for(ws_rows, g.nb, E.fused_K, htk::fused_round(E.ws_fill.threads, E.fused_K)));
@@ -414,7 +393,8 @@ ht_status engine_configure(Engine &E, std::string *why)
     s.seq_max = seq;
     const size_t desc_b = (size_t)grid_cap * seq * 8;
     const size_t cta_b = (size_t)grid_cap * 2 * 4;
-    const size_t need = desc_b + cta_b;
+    const size_t pass_b = (size_t)passes * 8, seg_b = (size_t)(passes / htk::kOrderPasses + 1) * 4;
+    const size_t need = pass_b + desc_b + cta_b + seg_b;
     if (need > E.book_bytes || grid_cap != E.grid_cap) {
         if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
             *why = std::string("synchronise before re-allocation: ") + cudaGetErrorString(e);
@@ -441,8 +421,10 @@ ht_status engine_configure(Engine &E, std::string *why)
         E.grid_cap = grid_cap;
     }
     char *p = static_cast<char *>(E.d_book);
-    s.desc = reinterpret_cast<uint2 *>(p);
-    uint32_t *cta = reinterpret_cast<uint32_t *>(p + desc_b);
+    E.pass_peaks = reinterpret_cast<uint2 *>(p);
+    s.desc = reinterpret_cast<uint2 *>(p + pass_b);
+    uint32_t *cta = reinterpret_cast<uint32_t *>(p + pass_b + desc_b);
+    E.seg_peaks = reinterpret_cast<uint32_t *>(p + pass_b + desc_b + cta_b);
     s.cta_nseq = cta;
     s.cta_total = cta + grid_cap;
     s.grid = scan_grid;
@@ -675,6 +657,9 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
     w.list = E.d_list;
     w.lines = E.d_lines;
     w.list_cap = E.list_cap;
+    w.pass_peaks = E.pass_peaks;
+    w.seg_peaks = E.seg_peaks;
+    w.n_seg = E.tma_ok ? (uint32_t)((htk::tile_passes(E.geom, E.tile, n_events) + htk::kOrderPasses - 1) / htk::kOrderPasses) : 0u;
     w.edge = E.d_edge;
     w.edge_pass = E.edge_pass;
     w.split_mode = E.split_mode;
@@ -686,36 +671,30 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
     return w;
 }
 
-// When engine_vote's next fill for these flags is one whose work split
-// k_bin_cluster can hand over -- the bulk-copy-tile fill (k_fill_tma) or the
-// peaks-only fill (k_fill_peaks) -- its configuration and grid, and whether
-// fill_blocks_per_sm holds it below its occupancy (the fill checks the shape
-// and splits by itself on a mismatch).
-static bool split_fill_next(const Engine &E, uint32_t n_events, uint32_t flags, htk::FillCfg &ff, uint32_t &grid,
-                            bool &capped)
+// Whether engine_vote's fill for these flags is the tile fill or the
+// peaks-only fill, and then whether fill_blocks_per_sm holds it below its
+// occupancy; for the peaks-only fill also its configuration and grid, whose
+// work split k_bin_cluster hands over (the fill checks the shape and splits by
+// itself on a mismatch).
+enum NextFill { NEXT_OTHER, NEXT_TILES, NEXT_PEAKS };
+static NextFill next_fill(const Engine &E, uint32_t n_events, uint32_t flags, htk::FillCfg &ff, uint32_t &grid,
+                          bool &capped)
 {
     if ((flags & (HT_FILL_NAIVE | HT_ACCUMULATE)) || !E.fill_priv_ok)
-        return false;
+        return NEXT_OTHER;
     const bool peaks_only = (flags & HT_PEAKS_ONLY) && E.fused_ok && E.d_edge &&
                             E.edge_pass * std::max<uint32_t>(1, E.fused_fill.W / 2) >= E.geom.na;
-    uint32_t g0;
-    if (peaks_only) {
-        ff = E.fused_fill;
-        ff.vote_weight = htk::kPeaksVoteWeight;
-        g0 = E.fused_grid;
-        capped = E.fused_capped;
-    } else {
-        if (!E.use_tma || E.use_ws)
-            return false;
-        ff = E.tma_fill;
-        ff.vote_weight = htk::kVoteWeight;
-        g0 = E.tma_grid;
+    if (!peaks_only) {
         capped = E.tma_capped;
+        return E.use_tma && !E.use_ws ? NEXT_TILES : NEXT_OTHER;
     }
+    ff = E.fused_fill;
+    ff.vote_weight = htk::kPeaksVoteWeight;
     ff.accumulate = 0u;
+    capped = E.fused_capped;
     const uint64_t items = (uint64_t)n_events * E.geom.n_slices * ff.strips;
-    grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(g0, items));
-    return grid + 1 <= E.split_cap;
+    grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.fused_grid, items));
+    return grid + 1 <= E.split_cap ? NEXT_PEAKS : NEXT_OTHER;
 }
 
 cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *z,
@@ -726,8 +705,8 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
     htk::FillCfg ff{};
     uint32_t grid = 0;
     bool capped = false;
-    const bool split_next = split_fill_next(E, n_events, flags, ff, grid, capped);
-    const bool want_cluster = E.tune.bin_cluster == 1 || (E.tune.bin_cluster == 0 && split_next && !capped);
+    const NextFill next = next_fill(E, n_events, flags, ff, grid, capped);
+    const bool want_cluster = E.tune.bin_cluster == 1 || (E.tune.bin_cluster == 0 && next != NEXT_OTHER && !capped);
     const bool cluster = want_cluster && E.bin_cluster > 0 &&
                          n_total <= htk::kBinClusterMax * htk::kBinClusterThreads * htk::kBinClusterHPT &&
                          htk::bin_cluster_smem_bytes(E.geom, n_events) <= htk::kBinClusterSmem;
@@ -735,7 +714,7 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
     if (cluster) {
         // few hits: binning and unit lists in one cluster launch, one CTA per
         // kBinClusterThreads hits (two hits a thread past kBinClusterMax CTAs)
-        if (split_next) {
+        if (next == NEXT_PEAKS) {
             const uint64_t items = (uint64_t)n_events * E.geom.n_slices * ff.strips;
             E.split_mode = htk::kSplitGiven;
             E.split_grid = grid;
@@ -775,11 +754,23 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
         ++E.launches;
     }
     E.ctr_dirty = false;   // the binning zeroed the counters
+    E.counts_fresh = true;
     E.last_hit_off = d_hit_off;
     E.last_n_hits0 = n_hits0;
     E.last_n_events = n_events;
     E.last_accumulate = (flags & HT_ACCUMULATE) != 0;
     return engine_vote(E, d_hit_off, n_hits0, n_events, flags, st);
+}
+
+// Zero what a fill counts up (the binning does the same).
+static cudaError_t engine_clear_counts(Engine &E, cudaStream_t st)
+{
+    cudaError_t e = cudaMemsetAsync(E.d_ctr + htk::CTR_ENTRIES, 0,
+                                    (engine_ctr_words(E) - htk::CTR_ENTRIES) * sizeof(uint32_t), st);
+    if (e == cudaSuccess && E.tma_ok)
+        e = cudaMemsetAsync(E.seg_peaks, 0,
+                            (htk::tile_passes(E.geom, E.tile, E.max_events) / htk::kOrderPasses + 1) * 4, st);
+    return e;
 }
 
 cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, uint32_t n_events, uint32_t flags,
@@ -788,6 +779,8 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     htk::Work w = make_work(E, nullptr, nullptr, nullptr, d_hit_off, n_hits0, n_events);
     cudaError_t e;
     E.fused_valid = false;
+    const bool fresh = E.counts_fresh;
+    E.counts_fresh = false;
     const bool accumulate = (flags & HT_ACCUMULATE) != 0;
     if ((flags & HT_FILL_NAIVE) || !E.fill_priv_ok) {
         if (!accumulate) {
@@ -806,22 +799,41 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     const uint64_t items = (uint64_t)n_events * E.geom.n_slices * f.strips;
     const bool peaks_only = (flags & HT_PEAKS_ONLY) && E.fused_ok && E.d_edge &&
                             E.edge_pass * std::max<uint32_t>(1, E.fused_fill.W / 2) >= E.geom.na;
-    if ((E.use_ws || E.use_tma || E.fused_ok) && !accumulate) {
+    if (E.use_tma && !E.use_ws && !peaks_only && !accumulate) {
+        if (!fresh) {   // voted again without a binning (the autotuner)
+            if ((e = engine_clear_counts(E, st)) != cudaSuccess)
+                return e;
+        }
+        const uint64_t passes = htk::tile_passes(E.geom, E.tile, n_events);
+        const uint32_t grid =
+            (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.tma_grid, (passes + E.tile.warps - 1) / E.tile.warps));
+        {
+            ProfScope ps(E, K_FILL_TMA, st);
+            e = htk::launch_fill_tma(E.geom, w, E.tile, E.scan, grid, st);
+        }
+        ++E.launches;
+        if (e == cudaSuccess) {
+            E.fused_valid = true;
+            E.ctr_dirty = true;
+            E.fused_passes = passes;
+            E.fused_events = n_events;
+        }
+        return e;
+    }
+    if ((E.use_ws || E.fused_ok) && !accumulate) {
         htk::ScanArgs a = E.scan;
         const bool ws = E.use_ws && !peaks_only;
-        const bool tma = !ws && E.use_tma && !peaks_only;
-        a.K = tma ? E.tma_K : E.fused_K;
-        htk::FillCfg ff = ws ? E.ws_fill : tma ? E.tma_fill : E.fused_fill;
+        a.K = E.fused_K;
+        htk::FillCfg ff = ws ? E.ws_fill : E.fused_fill;
         ff.accumulate = 0u;
         ff.vote_weight = peaks_only ? htk::kPeaksVoteWeight : htk::kVoteWeight;
         const uint64_t items_ff = (uint64_t)n_events * E.geom.n_slices * ff.strips;
         const uint32_t grid = (uint32_t)std::max<uint64_t>(
-            1, std::min<uint64_t>(ws ? E.ws_grid : tma ? E.tma_grid : E.fused_grid, items_ff));
+            1, std::min<uint64_t>(ws ? E.ws_grid : E.fused_grid, items_ff));
         const uint32_t lists = grid + (ff.dyn ? (uint32_t)htk::dyn_items(items_ff, grid) : 0u);
         {
-            ProfScope ps(E, ws ? K_FILL_WS : tma ? K_FILL_TMA : peaks_only ? K_FILL_PEAKS : K_FILL_SCAN, st);
+            ProfScope ps(E, ws ? K_FILL_WS : peaks_only ? K_FILL_PEAKS : K_FILL_SCAN, st);
             e = ws ? htk::launch_fill_ws(E.geom, w, ff, a, grid, st)
-               : tma ? htk::launch_fill_tma(E.geom, w, ff, a, grid, st)
                : peaks_only ? htk::launch_fill_peaks(E.geom, w, ff, a, grid, st)
                             : htk::launch_fill_scan(E.geom, w, ff, a, grid, st);
         }
@@ -835,6 +847,7 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
             E.fused_valid = true;
             E.ctr_dirty = true;
             E.fused_grid_used = lists;
+            E.fused_passes = 0;
             E.fused_events = n_events;
         }
         return e;
@@ -860,6 +873,14 @@ cudaError_t engine_scan(Engine &E, uint32_t n_events, htk::Peak *out, uint32_t c
     o.g_count = E.d_ctr + htk::CTR_ENTRIES;
     o.compact = compact ? 1u : 0u;
     cudaError_t e;
+    if (E.fused_valid && E.fused_events == n_events && E.fused_passes) {
+        // the tile fill left its peaks pass by pass
+        E.fused_valid = false;
+        ProfScope ps(E, K_ORDER, st);
+        e = htk::launch_order_passes(E.geom, w, a, o, E.fused_passes, st);
+        ++E.launches;
+        return e;   // the counters keep the peaks until the next binning (ctr_dirty)
+    }
     if (E.fused_valid && E.fused_events == n_events) {
         // the fused fill already found the peaks: only order them
         a.grid = E.fused_grid_used;
@@ -946,11 +967,11 @@ ht_status engine_autotune(Engine &E, uint32_t reps, cudaStream_t st, double *bes
             for (uint32_t th : thr_opts)
                 for (uint32_t kind = 1; kind <= (fused == 2 ? 2u : 1u); ++kind) {
                     if (fused == 5) {
-                        // the bulk-copy-tile kernel: its own row counts (0 = two 64 KB tiles)
+                        // the tile fill: its own row counts (0 = 16 KB tiles)
                         if (th == thr_opts[0])
                             continue;
-                        for (uint32_t Wt : {0u, W / 2})
-                            for (uint32_t tt : {512u, 1024u}) {
+                        for (uint32_t Wt : {0u, W / 4, W / 2})
+                            for (uint32_t tt : {256u, 512u}) {
                                 Tuning t = user;
                                 t.fused = 5;
                                 t.fill_W = Wt;
@@ -985,7 +1006,7 @@ ht_status engine_autotune(Engine &E, uint32_t reps, cudaStream_t st, double *bes
             if (r == 2 && cudaEventRecord(t0, st) != cudaSuccess)
                 ok = false;
             ok = ok && engine_vote(E, E.last_hit_off, E.last_n_hits0, n_events, 0u, st) == cudaSuccess &&
-                 engine_scan(E, n_events, nullptr, 0u, d_counts, st) == cudaSuccess;
+                 engine_scan(E, n_events, nullptr, 0u, d_counts, st, true) == cudaSuccess;
         }
         ok = ok && cudaEventRecord(t1, st) == cudaSuccess && cudaEventSynchronize(t1) == cudaSuccess &&
              cudaEventElapsedTime(&ms, t0, t1) == cudaSuccess;
@@ -1062,12 +1083,12 @@ void engine_get_tuning(const Engine &E, ht_tuning *t)
     t->scan_slots = E.scan.S;
     t->scan_blocks_per_sm = E.num_sms ? E.scan_grid_max / (uint32_t)E.num_sms : 0;
     t->fill_fused_scan = E.use_ws ? 3u : E.use_tma ? 5u : E.fused_ok ? (E.fused_fill.bulk ? 4u : 1u) : 2u;
-    t->fill_vote_agg = E.use_tma ? E.tma_fill.vote_agg : 0u;
+    t->fill_vote_agg = E.use_tma ? E.tile.vote_agg : 0u;
     t->bin_cluster = E.tune.bin_cluster ? E.tune.bin_cluster : (E.use_tma && !E.tma_capped) ? 1u : 2u;
     if (E.use_tma) {
-        t->fill_rows = E.tma_fill.W;
-        t->fill_threads = E.tma_fill.threads;
-        t->fill_hits_staged = E.tma_fill.HC;
+        t->fill_rows = E.tile.W;
+        t->fill_threads = E.tile.threads;
+        t->fill_hits_staged = E.fill.HC;
         t->fill_blocks_per_sm = E.num_sms ? E.tma_grid / (uint32_t)E.num_sms : 0;
     }
 }

@@ -71,9 +71,10 @@ struct Engine {
     uint32_t ws_grid = 0;
     bool use_ws = false;         // fills run the warp-specialised kernel
     bool tma_ok = false;         // the bulk-copy-tile fused kernel fits
-    htk::FillCfg tma_fill{};     // its shape (two u32 tiles of W x n_b)
+    htk::TileCfg tile{};         // its shape
     uint32_t tma_grid = 0;
-    uint32_t tma_K = 0;          // its peak buffer
+    uint2 *pass_peaks = nullptr; // (in d_book) its peaks per pass and per htk::kOrderPasses passes
+    uint32_t *seg_peaks = nullptr;
     bool use_tma = false;        // fills run the bulk-copy-tile kernel
     htk::ScanArgs scan{};
     int scan_kind = 0;            // htk::ScanKind in use
@@ -87,7 +88,9 @@ struct Engine {
     bool fused_valid = false;
     uint32_t fused_grid_used = 0;
     uint32_t fused_events = 0;
-    bool ctr_dirty = false;      // counters hold an unconsumed fused fill's peaks
+    uint64_t fused_passes = 0;   // the tile fill's passes (0: another fused fill's lists)
+    bool ctr_dirty = false;      // counters hold a fused fill's peaks
+    bool counts_fresh = false;   // the binning has just cleared every count the fill adds to
     int bin_cluster = -1;        // k_bin_cluster usable here (-1: not checked yet)
     bool tma_capped = false;     // fill_blocks_per_sm holds the bulk-copy-tile fill below its occupancy
     bool fused_capped = false;   // ... and the fused fills (the peaks-only fill among them)

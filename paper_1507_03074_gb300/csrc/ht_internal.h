@@ -24,8 +24,36 @@ struct FillCfg {
     uint32_t dyn;         // 1: the last dyn_items() items are handed out at run time (see below)
     uint32_t bulk;        // fused fill: 1 = passes leave through u32 staging and bulk copies (k_fill_bulk)
     uint32_t vote_weight; // cost of one vote against one cell written, in the static split (cta_items)
-    uint32_t vote_agg;    // bulk-copy-tile fill: warp-aggregated vote increments (match.any + one add)
 };
+
+// The tile fill (k_fill_tma): passes of W A-rows, each voted by one warp into
+// a u32 tile of its own that leaves as a bulk copy.
+struct TileCfg {
+    uint32_t W;           // A rows per pass (a power of two)
+    uint32_t strips;      // ceil(n_a / W) passes per (event, slice)
+    uint32_t tile_words;  // max(W, 2) rows of n_b words and 3 (a pass starts anywhere inside 16 bytes), a multiple of 4
+    uint32_t warps;       // per CTA
+    uint32_t run;         // neighbouring passes of a CTA's run (= warps)
+    uint32_t threads;     // the tuning's fill_threads (at least 32 * warps)
+    uint32_t vote_agg;    // warp-aggregated vote increments (match.any + one add)
+};
+constexpr uint32_t kTileWarps = 12;    // most warps of a tile-fill CTA (two such CTAs per SM: 80 registers a thread)
+constexpr uint32_t kTileCand = 127;    // cells >= T that a pass lists (more: every cell is looked at)
+constexpr uint32_t kAhead = 4;         // lines per lane loaded ahead
+constexpr uint32_t kHandedOut = 3;     // passes per warp handed out at run time (at least)
+// words of a warp's bits (one per tile cell), of its list (the length and the cells), and of all its shared memory
+__host__ __device__ constexpr uint32_t tile_bit_words(uint32_t tile_words) { return (tile_words / 32u + 4u) & ~3u; }
+__host__ __device__ constexpr uint32_t tile_list_words() { return (1u + kTileCand + 3u) & ~3u; }
+__host__ __device__ constexpr uint32_t tile_warp_words(uint32_t tile_words)
+{
+    return tile_words + tile_bit_words(tile_words) + tile_list_words() + 32u;
+}
+inline size_t tile_smem_bytes(const TileCfg &c) { return (size_t)c.warps * tile_warp_words(c.tile_words) * 4; }
+constexpr uint32_t kOrderPasses = 256; // passes per k_order_passes CTA
+__host__ __device__ inline uint64_t tile_passes(const Geom &g, const TileCfg &c, uint32_t n_events)
+{
+    return (uint64_t)n_events * g.n_slices * c.strips;
+}
 
 // Shared-memory words of the fused fill's two u32 staging buffers (half a
 // u16 pass, W / 2 rows of n_b cells, each), or 0 without bulk copies.
@@ -96,12 +124,13 @@ size_t fill_ws_smem_bytes(const FillCfg &c, const ScanArgs &a);
 cudaError_t launch_fill_ws(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
                            cudaStream_t st);
 cudaError_t fill_ws_occupancy(const FillCfg &c, const ScanArgs &a, int *blocks_per_sm);
-// Fused fill whose passes leave as bulk copies of two alternating u32 tiles
-// of W x n_b cells each (c.tile_words = W * n_b; n_b a multiple of 4).
-size_t fill_tma_smem_bytes(const FillCfg &c, const ScanArgs &a);
-cudaError_t launch_fill_tma(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
+// The tile fill, and the ordering of the peaks it leaves pass by pass (one
+// event, or o.compact).
+cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a, uint32_t grid,
                             cudaStream_t st);
-cudaError_t fill_tma_occupancy(const FillCfg &c, const ScanArgs &a, int *blocks_per_sm);
+cudaError_t fill_tma_occupancy(const TileCfg &c, int *blocks_per_sm);
+cudaError_t launch_order_passes(const Geom &g, const Work &w, const ScanArgs &a, const OrderArgs &o, uint64_t passes,
+                                cudaStream_t st);
 // After a fused fill (same grid): test its candidate entries, keep the peaks
 // (peaks_only: after k_fill_peaks, finishing the edge-flagged tests).
 cudaError_t launch_peaks(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,

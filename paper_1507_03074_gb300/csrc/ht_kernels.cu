@@ -9,11 +9,11 @@
 //   k_bin_cluster k_bin + k_scatter in one thread-block cluster for launches
 //                 of few hits (distributed shared memory for the counts),
 //                 which also writes the work split of the fill after it.
-//   k_fill_tma    Step 1 fused with the candidates of step 2 (default): the
-//                 votes of a pass of W A-rows go into a u32 shared-memory
-//                 tile laid out as M_H's rows, the tile leaves as one bulk
-//                 copy, and a vote taking a cell to T lists it.  k_peaks then
-//                 tests the listed cells against their neighbours.
+//   k_fill_tma    Step 1 fused with step 2 (default): a warp votes a pass of W
+//                 A-rows into a u32 shared-memory tile of its own, laid out as
+//                 M_H's rows, which leaves as one bulk copy; a vote taking a
+//                 cell to T lists it, and the warp tests the listed cells in
+//                 its tile.  k_order_passes puts the peaks in order.
 //   k_fill_priv   Step 1 (Sec. 2), privatised.  Work item = (event, slice,
 //                 strip of W A-rows); each CTA takes a contiguous range of
 //                 items.  It selects the event's hits admitted to the slice
@@ -41,6 +41,7 @@
 
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <atomic>
 #include <utility>
 
@@ -158,6 +159,8 @@ __global__ void __launch_bounds__(256) k_bin(Geom g, Work w)
         for (uint32_t i = tid; i < w.n_events; i += bd)
             w.ctr[CTR_EVENTS + i] = 0u;
     }
+    for (uint32_t i = blockIdx.x * bd + tid; i < w.n_seg; i += gridDim.x * bd)
+        w.seg_peaks[i] = 0u;
     if (w.hit_off)
         for (uint32_t i = tid; i <= w.n_events; i += bd)
             s_off[i] = w.hit_off[i];
@@ -374,6 +377,8 @@ __global__ void __launch_bounds__(1024, 1) k_bin_cluster(Geom g, Work w)
         for (uint32_t i = tid; i < w.n_events; i += bd)
             w.ctr[CTR_EVENTS + i] = 0u;
     }
+    for (uint32_t i = rank * bd + tid; i < w.n_seg; i += cs * bd)
+        w.seg_peaks[i] = 0u;
     if (w.hit_off)
         for (uint32_t i = tid; i <= w.n_events; i += bd)
             s_off[i] = w.hit_off[i];
@@ -766,35 +771,6 @@ __device__ __forceinline__ uint32_t next_dyn_item(const Work &w, uint32_t n_dyn,
         uint32_t d = n_dyn;
         if (n_dyn)
             d = atomicAdd(&w.ctr[CTR_DYN], 1u);
-        if (d >= n_dyn) {
-            d = n_dyn;
-            __threadfence();
-            if (atomicAdd(&w.ctr[CTR_DYN_DONE], 1u) == gridDim.x - 1) {
-                w.ctr[CTR_DYN] = 0u;
-                w.ctr[CTR_DYN_DONE] = 0u;
-            }
-        }
-        *s_word = d;
-    }
-    __syncthreads();
-    return *s_word;
-}
-
-// The run-time items with the claim of the next one in flight: thread 0
-// claims an item (dyn_claim) while the block still works on the one before,
-// and dyn_take publishes the claim to the block, ending the hand-out as
-// next_dyn_item does (rank n_dyn: none left).  Each CTA claims until it
-// gets none, once per rank, so the counters reset as with next_dyn_item.
-__device__ __forceinline__ uint32_t dyn_claim(const Work &w, uint32_t n_dyn)
-{
-    return atomicAdd(&w.ctr[CTR_DYN], 1u);   // thread 0 only; n_dyn > 0
-}
-
-__device__ __forceinline__ uint32_t dyn_take(const Work &w, uint32_t n_dyn, uint32_t claim, uint32_t *s_word)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t d = claim;
         if (d >= n_dyn) {
             d = n_dyn;
             __threadfence();
@@ -1301,10 +1277,8 @@ __device__ __forceinline__ bool is_peak_l2(const uint32_t *row, const uint32_t *
 // when r < split, else from rowsB + (r - split) rs (rs = row_stride, or n_b
 // when it is 0) -- M_H in global memory,
 // or (SMEM) the shared staging buffers.  Entries are {lin within event,
-// event, votes, 0}.  TV (the tile-store fill): the votes of a listed key are
-// read from rowsA[key] (the pass's u32 tile, rows n_b apart) instead of
-// candv.  All threads of the group call it.
-template <class G, bool SMEM = false, bool TV = false>
+// event, votes, 0}.  All threads of the group call it.
+template <class G, bool SMEM = false>
 __device__ __forceinline__ void emit_pass(const Geom &g, const Work &w, const ScanArgs &a, ScanSmem &ss, uint4 *pbuf,
                                           uint32_t &buf_n, uint32_t &nseq, uint32_t &total, const ChunkList &inner,
                                           const uint32_t *cand, const uint32_t *candv, uint32_t *srt, uint32_t *srtv,
@@ -1324,7 +1298,7 @@ __device__ __forceinline__ void emit_pass(const Geom &g, const Work &w, const Sc
             uint32_t rank = 0;
             for (uint32_t m = 0; m < n_c; ++m)
                 rank += cand[m] < key;
-            pbuf[buf_n + rank] = make_uint4(lin0 + key, e, TV ? rowsA[key] : candv[tid], 0u);
+            pbuf[buf_n + rank] = make_uint4(lin0 + key, e, candv[tid], 0u);
         }
         buf_n += n_c;
         total += n_c;
@@ -1338,7 +1312,7 @@ __device__ __forceinline__ void emit_pass(const Geom &g, const Work &w, const Sc
             for (uint32_t m = 0; m < n_c; ++m)
                 rank += cand[m] < key;
             srt[rank] = key;
-            srtv[rank] = TV ? rowsA[key] : candv[k];
+            srtv[rank] = candv[k];
         }
         // the sorted list is dense: append it to the chunk buffer as it is
         // (n_c <= kFusedCand <= K; a chunk is flushed with more than
@@ -1594,234 +1568,6 @@ __global__ void __launch_bounds__(1024) k_fill_scan(Geom g, Work w, FillCfg c, S
 __global__ void __launch_bounds__(1024) k_fill_bulk(Geom g, Work w, FillCfg c, ScanArgs a)
 {
     fill_scan_body<true>(g, w, c, a);
-}
-
-// ---------------------------------------------------------------------------
-// k_fill_tma: the fused fill with the tiles leaving by bulk copies.
-//
-// The tiles hold u32 counters in M_H's own layout (rows n_b cells apart, no
-// swizzle), so a finished pass of W rows is one contiguous run of M_H and
-// leaves the SM as a single bulk copy (cp.async.bulk, shared -> global) that
-// one thread issues: no thread converts, stores or even reads the cells.
-// Two tiles alternate: while the copy engine drains pass p's tile, the
-// threads vote pass p + 1 into the other one; a tile is cleared once the
-// copy that read it is done.  The votes themselves list the cells that
-// reach the threshold (a returned count of T - 1), so no pass scans its
-// tile for candidates.  The candidates go the way of k_fill_scan's (ranked,
-// emitted as ordered entries, tested by k_peaks against the finished M_H).
-// Needs n_b a multiple of 4 (16-byte rows); at most 64 rows per pass.
-// ---------------------------------------------------------------------------
-
-// A thread's share of the candidates q = r * nc + h of a pass over nc staged
-// hits: q = tid, tid + blockDim, ..; (r0, h0) is its first, and each step
-// adds dr rows and dh hits (carrying into r).  Fixed for a unit's staged
-// hits, so the divisions are made once per staging, not once per pass.
-struct FlatMap {
-    uint32_t nc, r0, h0, dr, dh;
-    __device__ __forceinline__ void set(uint32_t n)
-    {
-        nc = n;
-        if (n) {
-            r0 = threadIdx.x / n;
-            h0 = threadIdx.x - r0 * n;
-            dr = blockDim.x / n;
-            dh = blockDim.x - dr * n;
-        }
-    }
-};
-
-// The votes of the staged hits hs[0 .. m.nc) (the lines of rec[0 .. m.nc)) into tile rows 0 .. pr - 1 (A
-// bins iA ..): candidate q = r * nc + h goes to thread q % blockDim, so a
-// warp's lanes take consecutive hits of one row (their B columns, and so
-// their banks, are spread by the hits).  A vote that lifts its cell from
-// T - 1 to T lists the cell as r * n_b + j.  AGG: warp-aggregated increments
-// -- the lanes voting for the same cell find each other (match.any on the
-// cell index) and their lowest lane adds their number with one atomic; the
-// cell is listed by the add that takes it from below T to T or more.
-template <bool AGG>
-__device__ __forceinline__ void vote_flat(const Geom &g, uint32_t *tile, const float2 *hs, const float4 *rec,
-                                          const FlatMap &m, uint32_t pr, uint32_t iA, const FlushList &L)
-{
-    const uint32_t nb = g.nb, nc = m.nc;
-    if (nc == 0 || m.r0 >= pr)
-        return;
-    const uint32_t T = g.threshold, tm1 = T - 1u, lane = threadIdx.x & 31u;
-    uint32_t r = m.r0, h = m.h0;
-#pragma unroll 2
-    while (r < pr) {
-        const uint32_t j = vote_bin_line(g, hs[h], iA + r, rec + h);
-        if (j < nb) {
-            const uint32_t key = r * nb + j;
-            if (AGG) {
-                const uint32_t peers = __match_any_sync(__activemask(), key);
-                if (lane == (uint32_t)(__ffs(peers) - 1)) {
-                    const uint32_t n = (uint32_t)__popc(peers);
-                    const uint32_t old = atomicAdd(&tile[key], n);
-                    if (old < T && old + n >= T)
-                        note_candidate(L, r, key);
-                }
-            } else if (atomicAdd(&tile[key], 1u) == tm1) {
-                note_candidate(L, r, key);
-            }
-        }
-        h += m.dh;
-        r += m.dr;
-        if (h >= nc) {
-            h -= nc;
-            ++r;
-        }
-    }
-}
-
-// One pass's votes from the hits of list entries l0 .. l1 of unit es,
-// staged HC at a time (kept staged, with their FlatMap, for the unit's next
-// passes when they fit, as vote_pass).  Starts with a block barrier in every
-// case: the previous pass's clearing of this tile is complete.  All threads
-// call it.
-template <bool AGG>
-__device__ __forceinline__ void vote_pass_flat(const Geom &g, const Work &w, uint32_t *tile, float2 *hs, uint32_t HC,
-                                               uint64_t es, uint32_t l0, uint32_t l1, uint64_t &cached_es,
-                                               FlatMap &cached, uint32_t pr, uint32_t iA, const FlushList &L)
-{
-    if (cached_es == es) {
-        __syncthreads();
-        vote_flat<AGG>(g, tile, hs, w.list + l0, cached, pr, iA, L);
-        return;
-    }
-    cached_es = ~0ull;   // hs is about to be overwritten
-    uint32_t pos = l0;
-    bool first = true;
-    while (first || pos < l1) {
-        const float4 *rec = w.list + pos;
-        const uint32_t nsel = stage_hits<BlockGroup>(w, hs, HC, pos, l1);   // starts with a barrier
-        FlatMap m;
-        m.set(nsel);
-        if (first && pos >= l1) {
-            cached_es = es;
-            cached = m;
-        }
-        first = false;
-        vote_flat<AGG>(g, tile, hs, rec, m, pr, iA, L);
-    }
-}
-
-// NT = 2 tiles rotate: after pass p's copy is issued, the copy of pass p - 1
-// must have read its tile, which pass p + 1 then takes.  AGG: warp-aggregated
-// vote increments (vote_flat).
-template <bool AGG>
-__global__ void __launch_bounds__(1024) k_fill_tma(Geom g, Work w, FillCfg c, ScanArgs a)
-{
-    constexpr int NT = 2;
-    extern __shared__ uint4 sm4[];
-    // layout: ScanSmem (256 B) | K entries | NT tiles | HC staged vote lines |
-    //         candidate lists (keys, votes, sorted keys, sorted votes)
-    ScanSmem &ss = *reinterpret_cast<ScanSmem *>(sm4);
-    uint4 *pbuf = sm4 + 16;
-    uint32_t *tiles = reinterpret_cast<uint32_t *>(pbuf + a.K);
-    float2 *hs = reinterpret_cast<float2 *>(tiles + NT * c.tile_words);
-    uint32_t *lists = reinterpret_cast<uint32_t *>(hs + c.HC);
-    uint32_t *cand = lists, *candv = lists + kFusedCand, *srt = lists + 2 * kFusedCand,
-             *srtv = lists + 3 * kFusedCand;
-    __shared__ uint32_t s_hot[2], s_nc;
-
-    const uint32_t tid = threadIdx.x, bd = blockDim.x, nb = g.nb;
-    for (uint32_t k = tid; k < NT * c.tile_words / 4; k += bd)
-        reinterpret_cast<uint4 *>(tiles)[k] = make_uint4(0u, 0u, 0u, 0u);
-    if (tid == 0)
-        s_hot[0] = s_hot[1] = s_nc = 0u;
-    const uint32_t cta = blockIdx.x;
-    ChunkList inner = interior_list(a, cta);
-
-    // The static split reads only the unit offsets.  When k_bin wrote them
-    // and k_scatter precedes this kernel (kSplitEarly), k_scatter lets it
-    // launch only after k_bin has finished, so the split runs ahead of the
-    // wait for k_scatter's lists; after k_bin_cluster the split is read
-    // from what that kernel wrote (kSplitGiven), or computed after the wait.
-    __shared__ unsigned long long s_rng[2];
-    __shared__ uint32_t s_dyn;
-    const uint64_t items = (uint64_t)w.n_events * g.n_slices * c.strips;
-    const uint64_t n_dyn = c.dyn ? dyn_items(items, gridDim.x) : 0, n_static = items - n_dyn;
-    uint64_t it0, it1;
-    if (w.split_mode == kSplitEarly)
-        cta_items(g, w, c, cta, gridDim.x, n_static, it0, it1, s_rng);
-    grid_dep_wait();   // the unit lists (and, after k_bin_cluster, the offsets and split)
-    if (w.split_mode == kSplitGiven && w.split_grid == gridDim.x && w.split_strips == c.strips &&
-        w.split_vw == c.vote_weight && w.split_n_static == n_static) {
-        it0 = __ldcg(&w.split[cta]);
-        it1 = __ldcg(&w.split[cta + 1]);
-    } else if (w.split_mode != kSplitEarly) {
-        cta_items(g, w, c, cta, gridDim.x, n_static, it0, it1, s_rng);
-    }
-    uint64_t cached_es = ~0ull;
-    FlatMap cached{};
-    uint32_t buf_n = 0, nseq = 0, total = 0;
-    uint32_t tsel = 0;   // the tile of the next pass
-
-    auto do_item = [&](const ItemCursor &cur) {
-        const uint64_t es = cur.es;
-        const uint32_t e = cur.e;
-        const uint32_t l0 = __ldg(&w.slice_off[es]), l1 = __ldg(&w.slice_off[es + 1]);   // the unit's hits
-        const uint32_t iA = cur.k * c.W;
-        const uint32_t pr = min(c.W, g.na - iA);
-        const uint32_t slice_lin0 = cur.s * g.na * nb;
-        uint32_t *tile = tiles + (size_t)tsel * c.tile_words;
-
-        // ---- vote (tile tsel is clear, the lists empty) ------------------------
-        vote_pass_flat<AGG>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached, pr, iA,
-                       FlushList{s_hot, cand, candv, &s_nc, kFusedCand});
-        fence_proxy_async_smem();   // the tile's counts, visible to the copy engine
-        __syncthreads();            // votes and lists complete
-        // ---- the pass leaves as one bulk copy ------------------------------------
-        if (tid == 0) {
-            bulk_store_evict_first(w.M + (size_t)e * w.n_cells + slice_lin0 + (size_t)iA * nb, tile, pr * nb * 4u);
-            bulk_commit();
-        }
-        // ---- its candidates, votes read from the tile (the copy only reads it) --
-        const uint32_t n_c = s_nc;
-        const uint64_t hotm = (uint64_t)s_hot[0] | ((uint64_t)s_hot[1] << 32);
-        if (n_c)
-            emit_pass<BlockGroup, true, true>(g, w, a, ss, pbuf, buf_n, nseq, total, inner, cand, candv, srt, srtv,
-                                              n_c, hotm, pr, iA, slice_lin0, e, tile, nullptr, pr);
-        // ---- the next pass's tile: the copy that last read it is done -------------
-        const uint32_t next = tsel + 1u == (uint32_t)NT ? 0u : tsel + 1u;
-        if (tid == 0)
-            bulk_wait_read<NT - 1>();
-        __syncthreads();            // the lists are consumed; the next tile is free
-        uint4 *nt = reinterpret_cast<uint4 *>(tiles + (size_t)next * c.tile_words);
-#pragma unroll 4
-        for (uint32_t k = tid; k < c.tile_words / 4; k += bd)
-            nt[k] = make_uint4(0u, 0u, 0u, 0u);
-        if (tid == 0)
-            s_hot[0] = s_hot[1] = s_nc = 0u;
-        tsel = next;                // the next pass's votes start with a barrier
-    };
-    // the first run-time item is claimed during the last static one, each
-    // next one during the item before it (thread 0's claim stays in flight)
-    const bool dyn = c.dyn && n_dyn > 0;
-    uint32_t claim = 0;
-    if (dyn && tid == 0 && it1 <= it0)
-        claim = dyn_claim(w, (uint32_t)n_dyn);
-    ItemCursor cur(g, c, it0);
-    for (uint64_t item = it0; item < it1; ++item, cur.next(g, c)) {
-        if (dyn && tid == 0 && item + 1 == it1)
-            claim = dyn_claim(w, (uint32_t)n_dyn);
-        do_item(cur);
-    }
-    finish_candidates<BlockGroup>(w, a, ss, pbuf, buf_n, nseq, total, inner, cta);
-    if (dyn) {
-        // handed-out items, each with its own list of chunks
-        for (uint32_t d; (d = dyn_take(w, (uint32_t)n_dyn, claim, &s_dyn)) < n_dyn;) {
-            if (tid == 0)
-                claim = dyn_claim(w, (uint32_t)n_dyn);
-            const uint32_t list = gridDim.x + d;
-            inner = interior_list(a, list);
-            buf_n = nseq = total = 0;
-            do_item(ItemCursor(g, c, n_static + d));
-            finish_candidates<BlockGroup>(w, a, ss, pbuf, buf_n, nseq, total, inner, list);
-        }
-    }
-    if (tid == 0)
-        bulk_wait<0>();   // the last copies have written M_H (and read the tiles) before the CTA ends
 }
 
 // ---------------------------------------------------------------------------
@@ -2510,6 +2256,520 @@ __global__ void __launch_bounds__(256) k_order(Geom g, Work w, ScanArgs a, Order
     }
 }
 
+// ---------------------------------------------------------------------------
+// k_fill_tma: the fill fused with the peaks, one warp per tile.
+//
+// A pass is W A-rows of one (event, slice) unit.  A warp votes it into a u32
+// shared-memory tile of its own, laid out as M_H's rows, sends the tile to
+// M_H as one bulk copy (cp.async.bulk, shared -> global), finds the pass's
+// peaks in it while the copy reads, and clears it for its next pass.  Nothing
+// a warp does waits for another warp: the latencies of one pass (offsets,
+// lines, votes, copy) overlap with the other warps' passes.
+//
+// Order of the passes: a CTA's warps take a pass each of its runs (run i of
+// CTA c is run i * grid + c: c.run = warps neighbouring passes), and the last
+// passes
+// go to whichever warp of the grid comes first, so that the whole grid writes
+// one neighbourhood of M_H at any time and the hits' uneven spread over the
+// slices averages out.
+//
+// The peaks are found where the votes are: a vote that lifts its cell from
+// T - 1 to T lists the cell, and the listed cells are compared with their
+// neighbours in the tile.  For a cell on the first or last row of the pass
+// the votes of the row beyond are counted from the unit's lines (nothing waits
+// for the warp that owns it).  Each pass leaves {first entry, count} in
+// pass_peaks, in pass order, for k_order_passes.
+//
+// Bound: the M_H write where votes are few (paper event, one launch: 46.7 us
+// for 268 MB, a third of a warp's time spent waiting for its copy; upgrade
+// event: 592 us for 4.3 GB, 7.25 TB/s), the votes' instructions where they are
+// many (admission windows, 38 M candidate votes: 129 us).  Against CTAs of 512
+// threads that shared a tile, with three block barriers per pass and the peak
+// tests in a kernel of their own (events with three contexts in flight): paper
+// event 50.0 -> 41.0 us, windows 114.9 -> 94.2 us, batch of 100 events 4424 ->
+// 3772 us, four sectors 73.3 -> 56.2 us.  Tried on the way: the old tile
+// rotation behind a feeding warp, 48 us in flight (one barrier per pass, every
+// pass's latency exposed), and voting, draining and feeding warps around four
+// tiles, 44-47 us (the hand-overs cost more than the votes).
+// ---------------------------------------------------------------------------
+
+// Cells of a pass that reached T: keys r * n_b + j, the first kTileCand.
+struct PassList {
+    uint32_t n;
+    uint32_t cand[kTileCand];
+};
+
+// A pass: the unit's nc hits (lines and records), and its rows.
+struct TilePass {
+    const float2 *lines;
+    const float4 *recs;
+    uint32_t nc, iA, pr;
+};
+
+// A line that is no vote in any row (for lanes without a hit).
+__device__ __forceinline__ float2 no_line() { return make_float2(1.0e9f, 0.0f); }
+
+// The first 32 * kAhead of n lines, lane by lane.
+__device__ __forceinline__ void first_lines(float2 (&l)[kAhead], const float2 *lines, uint32_t n)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+    for (uint32_t k = 0; k < kAhead; ++k)
+        l[k] = 32u * k + lane < n ? __ldg(lines + 32u * k + lane) : no_line();
+}
+
+// 1 + the bins of the votes of line l (record *rec) in the R A bins from i on
+// (x: those bins less g.mid); 0 or above n_b for none.  on: this lane has a
+// hit.  As vote_bin_line, the R of them side by side and the rule behind one
+// branch.
+template <int R>
+__device__ __forceinline__ void line_bins(const Geom &g, const float2 l, const float (&x)[R], uint32_t i,
+                                          const float4 *rec, bool on, uint32_t (&j1)[R])
+{
+    const float big = 12582912.0f;
+    const float lim = __fmaf_rn(-g.err_v, fabsf(l.y), g.err_half);
+    const uint32_t near = lim > 0.0f ? g.nb + 1u : ~0u;   // bins whose edges matter
+    bool ask = false;
+    float d[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const float t = __fmaf_rn(l.y, x[q], l.x);
+        const float k = __fadd_rn(t, big);
+        d[q] = __fsub_rn(t, __fsub_rn(k, big));
+        j1[q] = __float_as_uint(k) - (__float_as_uint(big) - 1u);
+        ask |= !(fabsf(d[q]) <= lim) && j1[q] <= near;
+    }
+    if (ask && on) {
+        const float4 h = __ldg(rec);
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+            if (!(fabsf(d[q]) <= lim) && j1[q] <= near)
+                j1[q] = 1u + (uint32_t)vote_bin(g, __fmul_rn(2.0f, a_centre(g, i + q)), h.x, h.y, h.z);
+    }
+}
+
+// The votes of a pass into its tile (l: the first 32 * kAhead lines; the next
+// ones are loaded that far ahead): R rows at a time, a lane holds one hit's
+// line; consecutive lanes hold consecutive hits, whose B columns, and so whose
+// banks, differ.  A vote that lifts its cell from T - 1 to T lists the cell.
+// The R atomics are issued unconditionally, a lane without a vote adding 0 to
+// a word of its own (spare): behind a branch each would wait for the one
+// before it (102 cycles per atomic and warp, against 21 so).  AGG:
+// warp-aggregated increments -- the lanes voting for the same cell find each
+// other (match.any) and their lowest lane adds their number with one atomic;
+// the cell is listed by the add that takes it from below T to T or more.
+template <bool AGG, int R>
+__device__ __forceinline__ void vote_tile(const Geom &g, uint32_t *tile, const TilePass &P, float2 (&l)[kAhead],
+                                          PassList &L, uint32_t spare)
+{
+    const uint32_t nb = g.nb, T = g.threshold, lane = threadIdx.x & 31u;
+    for (uint32_t r0 = 0; r0 < P.pr; r0 += R) {
+        if (r0)
+            first_lines(l, P.lines, P.nc);
+        float x[R];
+        uint32_t row[R], most[R];   // per row: its first cell, less 1; the largest bin, plus 1 (0 beyond the pass)
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            x[q] = __int2float_rn((int)(P.iA + r0 + q) - g.mid);
+            row[q] = (r0 + q) * nb - 1u;
+            most[q] = r0 + q < P.pr ? nb : 0u;
+        }
+        // 32 hits, one per lane
+        auto vote = [&](const float2 line, uint32_t h) {
+            uint32_t j1[R], at[R], n[R], old[R], top = 0;
+            line_bins<R>(g, line, x, P.iA + r0, P.recs + h, h < P.nc, j1);
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const bool ok = j1[q] - 1u < most[q];
+                at[q] = ok ? row[q] + j1[q] : spare;
+                n[q] = ok ? 1u : 0u;
+            }
+            if (AGG) {
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    const uint32_t peers = __match_any_sync(0xffffffffu, at[q]);
+                    n[q] = lane == (uint32_t)(__ffs(peers) - 1) ? n[q] * (uint32_t)__popc(peers) : 0u;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                old[q] = atomicAdd(&tile[at[q]], n[q]);
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                top = max(top, old[q] + n[q]);
+            if (top >= T) {
+#pragma unroll
+                for (int q = 0; q < R; ++q)
+                    if (old[q] < T && old[q] + n[q] >= T) {
+                        const uint32_t p = atomicAdd(&L.n, 1u);
+                        if (p < kTileCand)
+                            L.cand[p] = at[q];
+                    }
+            }
+        };
+        for (uint32_t h0 = 0; h0 < P.nc; h0 += 32u * kAhead) {
+            float2 ahead[kAhead];
+            const uint32_t h1 = h0 + 32u * kAhead;
+            first_lines(ahead, P.lines + h1, P.nc > h1 ? P.nc - h1 : 0u);
+#pragma unroll
+            for (uint32_t k = 0; k < kAhead; ++k) {
+                if (h0 + 32u * k < P.nc)
+                    vote(l[k], h0 + 32u * k + lane);
+                l[k] = ahead[k];
+            }
+        }
+    }
+}
+
+// The votes of A row i into row[0 .. n_b), by one warp.
+__device__ __forceinline__ void vote_row(const Geom &g, uint32_t *row, const TilePass &P, uint32_t i)
+{
+    __syncwarp();
+    for (uint32_t h = threadIdx.x & 31u; h < P.nc; h += 32u) {
+        const uint32_t j = vote_bin_line(g, __ldg(P.lines + h), i, P.recs + h);
+        if (j < g.nb)
+            atomicAdd(&row[j], 1u);
+    }
+    __syncwarp();
+}
+
+// The peaks of pass number `pass` (the warp's own tile and list; bits: one bit
+// per cell of the tile, zero between calls).  reading: a bulk copy may still
+// read the tile.  Every lane calls it.
+__device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const ScanArgs &a, const TilePass &P,
+                                         uint32_t pass, uint32_t unit, uint32_t *tile, const PassList &L,
+                                         uint32_t *bits, bool reading)
+{
+    const uint32_t lane = threadIdx.x & 31u, nb = g.nb, n_c = L.n, full = 0xffffffffu, pr = P.pr;
+    const uint32_t e = unit / g.n_slices, s = unit - e * g.n_slices;
+    const uint32_t lin0 = (s * g.na + P.iA) * nb, last = (pr - 1u) * nb;
+    const bool above = P.iA > 0, below = P.iA + pr < g.na;   // rows of the slice beyond the pass
+    // the test against the neighbours inside the tile
+    auto inner = [&](uint32_t key, uint32_t v) {
+        const uint32_t r = key / nb, j = key - r * nb;
+        const uint32_t *row = tile + r * nb;
+        return is_peak(row, r > 0 ? row - nb : nullptr, r + 1 < pr ? row + nb : nullptr, j, nb, v);
+    };
+    // room for n entries, and the pass's counts
+    auto claim = [&](uint32_t n) {
+        uint32_t base = 0;
+        if (lane == 0) {
+            if (n) {
+                base = atomicAdd(a.g_count, n);
+                atomicAdd(&w.seg_peaks[pass / kOrderPasses], n);
+                atomicAdd(&a.ev_count[e], n);
+                if (base + n > a.entries_cap || base + n < base)
+                    atomicOr(w.status, (uint32_t)ST_SCRATCH_OVERFLOW);
+            }
+            w.pass_peaks[pass] = make_uint2(base, n);
+        }
+        return __shfl_sync(full, base, 0);
+    };
+    auto put = [&](uint32_t at, uint32_t key, uint32_t v) {
+        if (at < a.entries_cap)
+            a.entries[at] = make_uint4(lin0 + key, e, v, 0u);
+    };
+    // many peaks: a bit per cell that is one, then the bits in order
+    const uint32_t cells = pr * nb, words = (cells + 31u) / 32u;
+    auto put_bits = [&]() {
+        __syncwarp();
+        uint32_t n = 0;
+        for (uint32_t q = lane; q < words; q += 32u)
+            n += (uint32_t)__popc(bits[q]);
+        uint32_t base = claim(__reduce_add_sync(full, n));
+        for (uint32_t q0 = 0; q0 < words; q0 += 32u) {
+            const uint32_t q = q0 + lane;
+            uint32_t m = q < words ? bits[q] : 0u;
+            if (q < words)
+                bits[q] = 0u;
+            const uint32_t c = (uint32_t)__popc(m), incl = warp_incl_scan(c);
+            for (uint32_t at = base + incl - c; m; m &= m - 1u, ++at) {
+                const uint32_t key = 32u * q + (uint32_t)(__ffs(m) - 1);
+                put(at, key, tile[key]);
+            }
+            base += __shfl_sync(full, incl, 31);
+        }
+        __syncwarp();
+    };
+    if (n_c <= kTileCand) {   // one listed cell per lane
+        // the three cells of row i next to the cells j of the lanes in m, counted
+        // hit by hit: the most votes one of them holds, for each lane in m
+        auto beyond = [&](uint32_t m, uint32_t i, uint32_t j) {
+            uint32_t c0 = 0, c1 = 0, c2 = 0;
+            const float x[1] = {__int2float_rn((int)i - g.mid)};
+            float2 l = lane < P.nc ? __ldg(P.lines + lane) : no_line();
+            for (uint32_t h0 = 0; h0 < P.nc; h0 += 32u) {
+                const uint32_t h = h0 + lane;
+                uint32_t b[1];
+                line_bins<1>(g, l, x, i, P.recs + h, h < P.nc, b);
+                const uint32_t j1 = b[0] - 1u < nb ? b[0] : 0x80000000u;   // no cell is next to that
+                l = h + 32u < P.nc ? __ldg(P.lines + h + 32u) : no_line();
+                for (uint32_t k = m; k; k &= k - 1u) {
+                    const uint32_t src = (uint32_t)(__ffs(k) - 1);
+                    const uint32_t d = j1 - __shfl_sync(full, j, src);
+                    const uint32_t b0 = __ballot_sync(full, d == 0u), b1 = __ballot_sync(full, d == 1u),
+                                   b2 = __ballot_sync(full, d == 2u);
+                    if (lane == src) {
+                        c0 += (uint32_t)__popc(b0);
+                        c1 += (uint32_t)__popc(b1);
+                        c2 += (uint32_t)__popc(b2);
+                    }
+                }
+            }
+            return max(c1, max(c0, c2));
+        };
+        for (uint32_t k0 = 0; k0 < n_c; k0 += 32u) {
+            const bool has = k0 + lane < n_c;
+            const uint32_t key = has ? L.cand[k0 + lane] : ~0u;
+            const uint32_t v = has ? tile[key] : 0u;
+            bool keep = has && inner(key, v);
+            uint32_t m = __ballot_sync(full, keep && above && key < nb);
+            if (m) {
+                const uint32_t most = beyond(m, P.iA - 1u, key);
+                if ((m >> lane) & 1u)
+                    keep = v > most;
+            }
+            m = __ballot_sync(full, keep && below && key >= last);
+            if (m) {
+                const uint32_t most = beyond(m, P.iA + pr, key - last);
+                if ((m >> lane) & 1u)
+                    keep = v >= most;
+            }
+            if (n_c > 32u) {
+                if (keep)
+                    atomicOr(&bits[key >> 5], 1u << (key & 31u));
+                continue;
+            }
+            m = __ballot_sync(full, keep);
+            uint32_t rank = 0;
+            const uint32_t n = (uint32_t)__popc(m);
+            for (; m; m &= m - 1u)
+                rank += __shfl_sync(full, key, __ffs(m) - 1) < key;
+            const uint32_t base = claim(n);
+            if (keep)
+                put(base + rank, key, v);
+        }
+        if (n_c > 32u)
+            put_bits();
+        return;
+    }
+    // more than the list holds: every cell is looked at
+    for (uint32_t q = 0; q < words; ++q) {
+        const uint32_t key = 32u * q + lane;
+        const uint32_t v = key < cells ? tile[key] : 0u;
+        const uint32_t m = __ballot_sync(full, v >= g.threshold && inner(key, v));
+        if (lane == 0)
+            bits[q] = m;
+    }
+    // the rows beyond, each voted into a row of the tile that the test does
+    // not need (the tile holds at least two rows), which is voted anew after it
+    if ((above || below) && reading) {
+        if (lane == 0)
+            bulk_wait_read<0>();
+        __syncwarp();
+    }
+    auto beyond = [&](uint32_t i, uint32_t key0, uint32_t spare, bool before) {
+        uint32_t *row = tile + spare * nb;
+        auto clear = [&]() {
+            __syncwarp();
+            for (uint32_t j = lane; j < nb; j += 32u)
+                row[j] = 0u;
+        };
+        clear();
+        vote_row(g, row, P, i);
+        for (uint32_t j = lane; j < nb; j += 32u) {
+            const uint32_t key = key0 + j, b = 1u << (key & 31u);
+            const uint32_t most = max(row[j], max(j ? row[j - 1] : 0u, j + 1 < nb ? row[j + 1] : 0u));
+            if ((bits[key >> 5] & b) && !(before ? tile[key] > most : tile[key] >= most))
+                atomicAnd(&bits[key >> 5], ~b);
+        }
+        clear();
+        if (spare < pr)
+            vote_row(g, row, P, P.iA + spare);
+        __syncwarp();
+    };
+    __syncwarp();
+    if (above)
+        beyond(P.iA - 1u, 0u, 1u, true);
+    if (below)
+        beyond(P.iA + pr, last, pr > 1u ? 0u : 1u, false);
+    put_bits();
+}
+
+// STORE: the tiles go to M_H (else the peaks are all that is wanted).  AGG:
+// warp-aggregated vote increments (vote_tile).  passes: over all events; runs:
+// runs of c.run passes per CTA, the passes behind them being handed out.
+template <bool STORE, bool AGG>
+__global__ void __launch_bounds__(kTileWarps * 32, 2) k_fill_tma(const __grid_constant__ Geom g,
+                                                              const __grid_constant__ Work w, const TileCfg c,
+                                                              const __grid_constant__ ScanArgs a, uint32_t passes,
+                                                              uint32_t runs)
+{
+    extern __shared__ uint4 sm4[];
+    // layout: per warp a tile, its bits, its list and 32 idle words
+    __shared__ uint32_t s_left;
+    const uint32_t nb = g.nb, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, warps = blockDim.x >> 5;
+    const uint32_t mine = tile_warp_words(c.tile_words);
+    uint32_t *tile0 = reinterpret_cast<uint32_t *>(sm4) + warp * mine;
+    uint32_t *bits = tile0 + c.tile_words;
+    PassList &L = *reinterpret_cast<PassList *>(bits + tile_bit_words(c.tile_words));
+    const uint32_t *idle = reinterpret_cast<uint32_t *>(&L) + tile_list_words() + lane;   // the lane's own word
+    for (uint32_t k = lane; k < mine / 4u; k += 32u)
+        reinterpret_cast<uint4 *>(tile0)[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0)
+        s_left = warps;
+    __syncthreads();
+    grid_dep_wait();   // the unit lists
+
+    // The warp's passes: one of each of the CTA's runs, then the ones handed out
+    // (the first is the warp's own number in the grid).  Lane 0 claims a
+    // handed-out pass one pass before its number is needed.
+    const uint32_t fixed = runs * c.run * gridDim.x;
+    uint32_t turn = 0, claimed = blockIdx.x * warps + warp;
+    auto next_pass = [&]() {
+        if (turn < runs)
+            return (turn++ * gridDim.x + blockIdx.x) * c.run + warp;
+        const uint32_t q = __shfl_sync(0xffffffffu, claimed, 0);
+        if (q >= passes - fixed)
+            return passes;
+        if (lane == 0)
+            claimed = warps * gridDim.x + atomicAdd(&w.ctr[CTR_DYN], 1u);
+        return fixed + q;
+    };
+    auto offsets = [&](uint32_t pass) {
+        if (pass >= passes)
+            return make_uint2(0u, 0u);
+        const uint32_t u = pass / c.strips;
+        return make_uint2(__ldcg(&w.slice_off[u]), __ldcg(&w.slice_off[u + 1]));
+    };
+    // The next pass's lines are loaded while this one's tile leaves, and the
+    // offsets of the one behind it: nothing that a pass begins with is waited for.
+    uint32_t pass = next_pass(), next = next_pass();
+    uint2 off = offsets(pass), next_off = offsets(next);
+    float2 l[kAhead];
+    first_lines(l, w.lines + off.x, off.y - off.x);
+    while (pass < passes) {
+        const uint32_t unit = pass / c.strips;
+        TilePass P;
+        P.iA = (pass - unit * c.strips) * c.W;
+        P.pr = min(c.W, g.na - P.iA);
+        P.lines = w.lines + off.x;
+        P.recs = w.list + off.x;
+        P.nc = off.y - off.x;
+        // the pass's first cell lies in the tile as in M_H: at the same address modulo 16 bytes
+        const uint64_t cell0 = (uint64_t)unit * ((uint64_t)g.na * nb) + (uint64_t)P.iA * nb;
+        uint32_t *tile = tile0 + (uint32_t)(cell0 & 3u);
+        const uint32_t spare = (uint32_t)(idle - tile);
+        if (P.pr > 2u)
+            vote_tile<AGG, 4>(g, tile, P, l, L, spare);
+        else
+            vote_tile<AGG, 2>(g, tile, P, l, L, spare);
+        if (STORE)
+            fence_proxy_async_smem();   // this lane's counts, visible to the copy engine
+        __syncwarp();
+        // ---- the pass leaves: whole 16 bytes as one bulk copy, up to three words on either side by hand
+        if (STORE) {
+            const uint32_t cells = P.pr * nb, head = min((uint32_t)(-cell0 & 3u), cells), mid = (cells - head) & ~3u;
+            uint32_t *dst = w.M + cell0;
+            if (lane == 0) {
+                if (mid)
+                    bulk_store_evict_first(dst + head, tile + head, mid * 4u);
+                bulk_commit();
+            }
+            if (lane < cells - mid) {
+                const uint32_t k = lane < head ? lane : mid + lane;
+                dst[k] = tile[k];
+            }
+        }
+        first_lines(l, w.lines + next_off.x, next_off.y - next_off.x);
+        const uint32_t next2 = next_pass();
+        const uint2 next2_off = offsets(next2);
+        // ---- its peaks
+        if (L.n)
+            pass_search(g, w, a, P, pass, unit, tile, L, bits, STORE);
+        else if (lane == 0)
+            w.pass_peaks[pass] = make_uint2(0u, 0u);
+        // ---- the tile is cleared once the copy has read it
+        if (STORE && lane == 0)
+            bulk_wait_read<0>();
+        __syncwarp();
+        if (lane == 0)
+            L.n = 0u;
+#pragma unroll 8
+        for (uint32_t k = lane; k < c.tile_words / 4u; k += 32u)
+            reinterpret_cast<uint4 *>(tile0)[k] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+        pass = next;
+        off = next_off;
+        next = next2;
+        next_off = next2_off;
+    }
+    if (lane == 0) {
+        if (STORE)
+            bulk_wait<0>();   // the warp's copies have written M_H (and read its tile) before the CTA ends
+        if (atomicSub(&s_left, 1u) == 1u) {
+            __threadfence();
+            if (atomicAdd(&w.ctr[CTR_DYN_DONE], 1u) == gridDim.x - 1) {   // nobody claims any more
+                w.ctr[CTR_DYN] = 0u;
+                w.ctr[CTR_DYN_DONE] = 0u;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_order_passes: the peaks of k_fill_tma's passes into one list, ascending.
+// A CTA takes a segment of kOrderPasses passes: its first rank is the sum of
+// the segments before it, and one thread per peak finds its pass by a search
+// over the segment's prefix sums.  (One event, or one list over all events.)
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kOrderPasses) k_order_passes(Geom g, Work w, ScanArgs a, OrderArgs o,
+                                                               uint64_t passes)
+{
+    grid_dep_wait();
+    __shared__ uint32_t s_off[kOrderPasses], s_base[kOrderPasses], s_wsum[40];
+    const uint32_t tid = threadIdx.x, seg = blockIdx.x, warp = tid >> 5, lane = tid & 31u;
+    const uint32_t mine = w.seg_peaks[seg];
+    if (seg == 0)
+        for (uint32_t e = tid; e < w.n_events; e += kOrderPasses)
+            o.counts[e] = o.ev_count[e];
+    if (mine == 0)
+        return;
+    const uint64_t pass = (uint64_t)seg * kOrderPasses + tid;
+    const uint2 d = pass < passes ? w.pass_peaks[pass] : make_uint2(0u, 0u);
+    uint32_t before = 0;
+    for (uint32_t q = tid; q < seg; q += kOrderPasses)
+        before += w.seg_peaks[q];
+    before = __reduce_add_sync(0xffffffffu, before);
+    const uint32_t incl = warp_incl_scan(d.y);
+    if (lane == 31u)
+        s_wsum[warp] = incl;
+    if (lane == 0)
+        s_wsum[16 + warp] = before;
+    __syncthreads();
+    uint32_t off = incl - d.y, rank0 = 0;
+    for (uint32_t q = 0; q < kOrderPasses / 32; ++q) {
+        off += q < warp ? s_wsum[q] : 0u;
+        rank0 += s_wsum[16 + q];
+    }
+    s_off[tid] = off;
+    s_base[tid] = d.x;
+    __syncthreads();
+    for (uint32_t k = tid; k < mine; k += kOrderPasses) {
+        uint32_t lo = 0, hi = kOrderPasses - 1;   // the last pass that starts at or before k
+        while (lo < hi) {
+            const uint32_t m = (lo + hi + 1) >> 1;
+            if (s_off[m] <= k)
+                lo = m;
+            else
+                hi = m - 1;
+        }
+        const uint32_t at = s_base[lo] + (k - s_off[lo]);
+        if (at < a.entries_cap && rank0 + k < o.capacity)
+            o.out[rank0 + k] = peak_record(g, a.entries[at]);
+    }
+}
+
 } // namespace htk
 
 // ---------------------------------------------------------------------------
@@ -2694,32 +2954,45 @@ cudaError_t launch_fill_peaks(const Geom &g, const Work &w, const FillCfg &c, co
     return launch_pdl(k_fill_peaks, grid, c.threads, smem, st, g, w, c, a);
 }
 
-size_t fill_tma_smem_bytes(const FillCfg &c, const ScanArgs &a)
+using TileKernel = void (*)(Geom, Work, TileCfg, ScanArgs, uint32_t, uint32_t);
+static TileKernel tile_kernel(const TileCfg &c)
 {
-    return 16 * sizeof(uint4) + (size_t)a.K * sizeof(uint4) + (size_t)2 * c.tile_words * 4 +
-           (size_t)c.HC * 8 + (size_t)4 * kFusedCand * 4;
+    return c.vote_agg ? k_fill_tma<true, true> : k_fill_tma<true, false>;
 }
 
-cudaError_t launch_fill_tma(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
+cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a, uint32_t grid,
                             cudaStream_t st)
 {
-    const size_t smem = fill_tma_smem_bytes(c, a);
-    const void *k = c.vote_agg ? (const void *)k_fill_tma<true> : (const void *)k_fill_tma<false>;
-    cudaError_t e = allow_smem(k, smem);
+    const size_t smem = tile_smem_bytes(c);
+    const TileKernel k = tile_kernel(c);
+    cudaError_t e = allow_smem((const void *)k, smem);
     if (e != cudaSuccess)
         return e;
-    return c.vote_agg ? launch_pdl(k_fill_tma<true>, grid, c.threads, smem, st, g, w, c, a)
-                      : launch_pdl(k_fill_tma<false>, grid, c.threads, smem, st, g, w, c, a);
+    // The SMs do not write at one rate: an eighth of the passes is handed out at
+    // run time (upgrade event, alone: 689 us with 3 passes per warp handed out,
+    // 636 us with an eighth, 639 us with a quarter, 786 us with half of them:
+    // handed-out neighbours go to different SMs, which share no lines in L1).
+    const uint32_t passes = (uint32_t)tile_passes(g, c, w.n_events);
+    const uint32_t handed = std::max(kHandedOut * c.warps * grid, passes / 8u);
+    const uint32_t runs = passes > handed ? (passes - handed) / (grid * c.run) : 0u;
+    return launch_pdl(k, grid, c.warps * 32u, smem, st, g, w, c, a, passes, runs);
 }
 
-cudaError_t fill_tma_occupancy(const FillCfg &c, const ScanArgs &a, int *blocks_per_sm)
+cudaError_t fill_tma_occupancy(const TileCfg &c, int *blocks_per_sm)
 {
-    const size_t smem = fill_tma_smem_bytes(c, a);
-    const void *k = c.vote_agg ? (const void *)k_fill_tma<true> : (const void *)k_fill_tma<false>;
-    cudaError_t e = allow_smem(k, smem);
+    const size_t smem = tile_smem_bytes(c);
+    const TileKernel k = tile_kernel(c);
+    cudaError_t e = allow_smem((const void *)k, smem);
     if (e != cudaSuccess)
         return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, c.threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, (int)c.warps * 32, smem);
+}
+
+cudaError_t launch_order_passes(const Geom &g, const Work &w, const ScanArgs &a, const OrderArgs &o, uint64_t passes,
+                                cudaStream_t st)
+{
+    return launch_pdl(k_order_passes, (uint32_t)((passes + kOrderPasses - 1) / kOrderPasses), kOrderPasses, 0, st, g, w,
+                      a, o, passes);
 }
 
 cudaError_t fill_scan_occupancy(const FillCfg &c, const ScanArgs &a, uint32_t nb, int *blocks_per_sm)

@@ -1,0 +1,59 @@
+"""The tile fill (one warp per tile, peaks found in the tile) against the
+oracle at the edges of its shapes: passes of one row and of a remainder, a
+single A bin, unit lists around the 128 lines a warp loads ahead, passes that
+list up to 32, up to 127 and more cells, peaks on the rows where two passes
+meet, the narrowest and the widest rows."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.test_gpu_parity import ht, _ob, _orr, assert_peaks_equal, random_hits  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+# (n_theta, n_phi, n_a, n_b), hits, thresholds
+SHAPES = [
+    ((1, 1, 1, 64), 127, (1, 6)), ((1, 1, 2, 4), 128, (3, 30)), ((1, 2, 3, 32), 129, (2, 7)),
+    ((1, 2, 5, 1024), 260, (1, 2)), ((2, 3, 13, 100), 900, (2, 4, 6)), ((1, 1, 9, 4096), 1500, (1, 2)),
+    ((3, 2, 67, 256), 3000, (2, 3, 9)), ((1, 1, 33, 128), 2049, (10, 24)), ((4, 8, 130, 512), 33, (1, 2)),
+]
+
+
+@pytest.mark.parametrize("rows", [0, 1, 2, 8, 64], ids=lambda r: f"rows{r}")
+@pytest.mark.parametrize("shape", SHAPES, ids=[str(s[0]) for s in SHAPES])
+def test_tile_fill_shapes(ht, shape, rows):
+    bins, n, thresholds = shape
+    b, r = ht.Binning(*bins), ht.Ranges()
+    x, y, z = random_hits(n, n, rmax=700.0)
+    M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+    for T in thresholds:
+        pk_ref, n_ref = oracle.find_maxima(_ob(b), _orr(r), M_ref, T)
+        with ht.Context(b, r, threshold=T, max_hits=n) as ctx:
+            ctx.set_tuning(fill_rows=rows)
+            for _ in range(2):
+                ctx.fill(x, y, z)
+                pk, total = ctx.find_maxima(capacity=1 << 18)
+                assert total == n_ref, T
+                assert_peaks_equal(pk, pk_ref)
+            assert np.array_equal(ctx.matrix(), M_ref)
+
+
+def test_tile_fill_batch(ht):
+    """Events of very different sizes (one empty) in one launch: the ranks run
+    over all events' passes, and the counts are each event's own."""
+    b, r, T = ht.Binning(2, 4, 37, 64), ht.Ranges(), 3
+    events = [random_hits(n, 50 + n) for n in (1, 0, 700, 31, 128, 2500, 5)]
+    with ht.Batch(b, r, threshold=T, max_events=len(events), max_hits=4000, capacity=1 << 16) as B:
+        for _ in range(3):   # captured after the first run
+            pk, counts = B.run(*ht.Batch.concat(events))
+            at = 0
+            for e, (x, y, z) in enumerate(events):
+                M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+                pk_ref, n_ref = oracle.find_maxima(_ob(b), _orr(r), M_ref, T)
+                assert counts[e] == n_ref, e
+                got = pk[at:at + n_ref]
+                assert np.all(got["event"] == e)
+                assert_peaks_equal(got, pk_ref)
+                assert np.array_equal(B.matrix(e), M_ref)
+                at += n_ref
+            assert len(pk) == at
