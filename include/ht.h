@@ -243,8 +243,11 @@ ht_status ht_profile_read(ht_ctx *ctx, ht_kernel_time *out, uint32_t cap, uint32
 /* Launch shapes.  Every field 0 means automatic; results (M_H and peaks)
  * are identical for every accepted tuning, only the speed changes.
  *   fill_rows          A rows per shared-memory vote tile (power of two)
- *   fill_threads       256, 512 or 1024 threads per fill CTA
- *   fill_hits_staged   hits staged in shared memory per selection chunk
+ *   fill_threads       256, 512 or 1024 threads per fill CTA (the tile fill
+ *                      runs as many of their warps, up to 12, as their tiles
+ *                      fit)
+ *   fill_hits_staged   hits staged in shared memory per selection chunk (not
+ *                      in the tile fill, which stages none)
  *   fill_blocks_per_sm cap on resident fill CTAs per SM
  *   scan_kind          HT_SCAN_BULK (1-D bulk-copy ring), HT_SCAN_STREAM
  *                      (register streaming), HT_SCAN_DIRECT (scalar)
@@ -259,13 +262,14 @@ ht_status ht_profile_read(ht_ctx *ctx, ht_kernel_time *out, uint32_t cap, uint32
  *                      tile leaves through two u32 staging buffers in shared
  *                      memory and bulk async copies (cp.async.bulk), so the
  *                      stores drain while the next votes run (1024 threads
- *                      by default; n_b a multiple of 4); 5: as 1 with u32
- *                      tiles in M_H's own layout (fill_rows rows, two in
- *                      rotation), each pass leaving as one bulk async copy
- *                      that no thread converts or stores, the votes listing
- *                      the cells that reach the threshold (n_b a multiple of
- *                      4); 2: never (a full scan in ht_find_maxima); 0: 5
- *                      when n_b is a multiple of 4, else 1, when it fits
+ *                      by default; n_b a multiple of 4); 5: the tile fill:
+ *                      every warp votes fill_rows rows into a u32 tile of its
+ *                      own in M_H's layout, which leaves as one bulk async
+ *                      copy, and finds the peaks in it (asked for by value,
+ *                      n_b a multiple of 4); 2: never (a full scan in
+ *                      ht_find_maxima); 0: the tile fill for n_b up to 4096
+ *                      when it fits (ht_get_tuning then reports 5, or 0 when
+ *                      n_b is not a multiple of 4), else 1, when it fits
  *                      (the fused modes only for non-accumulating, non-naive
  *                      fills)
  *   fill_vote_agg      1: the bulk-copy-tile fill (fill_fused_scan 5)

@@ -149,7 +149,7 @@ ht_status engine_configure(Engine &E, std::string *why)
     // with the bulk-copy-tile fill (asked for, or automatic where n_b allows
     // it) fill_rows sizes its tiles; the other fills (accumulating, peaks-only)
     // keep their own tile height
-    bool tma_mode = (t.fused == 5 || t.fused == 0) && (b.n_b & 3u) == 0 && b.n_b <= 4096;
+    bool tma_mode = (t.fused == 0 || (t.fused == 5 && (b.n_b & 3u) == 0)) && b.n_b <= 4096;
     // the tile fill's shape at W rows per pass: as many of fill_threads' warps as
     // their tiles fit, twice per SM unless the threads were asked for
     auto tile_shape = [&](uint32_t W) {
@@ -281,8 +281,10 @@ ht_status engine_configure(Engine &E, std::string *why)
     // --- the tile fill ------------------------------------------------------------
     E.tma_ok = false;
     E.tma_capped = false;
-    // the default fused fill wherever it fits (fused 0 = auto)
-    if (E.fill_priv_ok && (t.fused == 5 || t.fused == 0) && (b.n_b & 3u) == 0 && b.n_b <= 4096) {
+    // The default fused fill wherever it fits (fused 0 = auto).  Rows that are not
+    // whole 16 bytes cost a tile up to six words written by hand: 999 x 1001 bins
+    // against the thread-store fill that took them before, 121 -> 44 us per event with three in flight.
+    if (E.fill_priv_ok && (t.fused == 0 || (t.fused == 5 && (b.n_b & 3u) == 0)) && b.n_b <= 4096) {
         uint32_t Wt = t.fill_W;
         if (!Wt) {
             Wt = 64;   // tiles of at most 16 KB, and lower ones while there are fewer passes than warps
@@ -973,7 +975,7 @@ ht_status engine_autotune(Engine &E, uint32_t reps, cudaStream_t st, double *bes
                         for (uint32_t Wt : {0u, W / 4, W / 2})
                             for (uint32_t tt : {256u, 512u}) {
                                 Tuning t = user;
-                                t.fused = 5;
+                                t.fused = E.geom.nb & 3u ? 0u : 5u;
                                 t.fill_W = Wt;
                                 t.fill_threads = tt;
                                 cands.push_back(t);
@@ -1082,7 +1084,8 @@ void engine_get_tuning(const Engine &E, ht_tuning *t)
     t->scan_stage_bytes = E.scan.slot_words * 4;
     t->scan_slots = E.scan.S;
     t->scan_blocks_per_sm = E.num_sms ? E.scan_grid_max / (uint32_t)E.num_sms : 0;
-    t->fill_fused_scan = E.use_ws ? 3u : E.use_tma ? 5u : E.fused_ok ? (E.fused_fill.bulk ? 4u : 1u) : 2u;
+    // (the tile fill of rows that are not whole 16 bytes is automatic only: 0)
+    t->fill_fused_scan = E.use_ws ? 3u : E.use_tma ? (E.geom.nb & 3u ? 0u : 5u) : E.fused_ok ? (E.fused_fill.bulk ? 4u : 1u) : 2u;
     t->fill_vote_agg = E.use_tma ? E.tile.vote_agg : 0u;
     t->bin_cluster = E.tune.bin_cluster ? E.tune.bin_cluster : (E.use_tma && !E.tma_capped) ? 1u : 2u;
     if (E.use_tma) {

@@ -16,6 +16,9 @@ SHAPES = [
     ((1, 1, 1, 64), 127, (1, 6)), ((1, 1, 2, 4), 128, (3, 30)), ((1, 2, 3, 32), 129, (2, 7)),
     ((1, 2, 5, 1024), 260, (1, 2)), ((2, 3, 13, 100), 900, (2, 4, 6)), ((1, 1, 9, 4096), 1500, (1, 2)),
     ((3, 2, 67, 256), 3000, (2, 3, 9)), ((1, 1, 33, 128), 2049, (10, 24)), ((4, 8, 130, 512), 33, (1, 2)),
+    # rows that are not whole 16 bytes: passes start and end anywhere inside them
+    ((1, 1, 1, 1), 50, (1, 20)), ((2, 1, 3, 2), 90, (2, 9)), ((1, 3, 7, 3), 200, (2, 12)), ((1, 2, 5, 1023), 260, (1, 2)),
+    ((2, 3, 13, 101), 900, (2, 4, 6)), ((1, 1, 9, 4095), 1500, (1, 2)), ((3, 2, 67, 258), 3000, (2, 3, 9)),
 ]
 
 
@@ -38,10 +41,11 @@ def test_tile_fill_shapes(ht, shape, rows):
             assert np.array_equal(ctx.matrix(), M_ref)
 
 
-def test_tile_fill_batch(ht):
+@pytest.mark.parametrize("n_b", [64, 61, 30])
+def test_tile_fill_batch(ht, n_b):
     """Events of very different sizes (one empty) in one launch: the ranks run
     over all events' passes, and the counts are each event's own."""
-    b, r, T = ht.Binning(2, 4, 37, 64), ht.Ranges(), 3
+    b, r, T = ht.Binning(2, 4, 37, n_b), ht.Ranges(), 3
     events = [random_hits(n, 50 + n) for n in (1, 0, 700, 31, 128, 2500, 5)]
     with ht.Batch(b, r, threshold=T, max_events=len(events), max_hits=4000, capacity=1 << 16) as B:
         for _ in range(3):   # captured after the first run
