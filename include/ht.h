@@ -124,8 +124,7 @@ ht_status ht_destroy(ht_ctx *ctx);
  * global atomicAdd per vote).  HT_PEAKS_ONLY keeps every vote tile in shared
  * memory: the next ht_find_maxima returns the same peaks, but M_H is left as
  * it was (ht_copy_matrix does not show this fill); not with HT_ACCUMULATE or
- * HT_FILL_NAIVE; the first such fill allocates a small edge-row buffer and
- * waits for the device.  n_hits may be 0 (M_H becomes all zero).
+ * HT_FILL_NAIVE.  n_hits may be 0 (M_H becomes all zero).
  * Errors: HT_E_INVAL (NULL pointer with n_hits > 0, n_hits > max_hits, or
  * accumulated hits beyond max_hits), HT_E_CUDA, HT_E_STATE. */
 ht_status ht_fill(ht_ctx *ctx, const float *x, const float *y, const float *z, uint32_t n_hits,
@@ -346,7 +345,6 @@ ht_status ht_batch_destroy(ht_batch *batch);
  * only enqueues on `stream` (NULL = the batch's own stream); the caller
  * checks counts for truncation; ht_batch_sync reports device-side failures.
  * HT_PEAKS_ONLY: the same peaks without writing the matrices (as ht_fill;
- * the first such run allocates the edge rows and waits for the device;
  * ht_batch_copy_matrix does not show such a run).
  * HT_FILL_NAIVE: the paper's fill for every event (as ht_fill: clear, then
  * one global atomic per vote; the same matrices and peaks); not with

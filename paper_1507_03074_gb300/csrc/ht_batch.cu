@@ -302,17 +302,7 @@ ht_status ht_batch_run(ht_batch *b, const float *x, const float *y, const float 
         return hte::report(HT_E_INVAL, "unknown flag (batches take HT_MEM_DEVICE, HT_PEAKS_ONLY and HT_FILL_NAIVE)");
     if ((flags & HT_PEAKS_ONLY) && (flags & HT_FILL_NAIVE))
         return hte::report(HT_E_INVAL, "HT_PEAKS_ONLY does not combine with HT_FILL_NAIVE");
-    const bool po = (flags & HT_PEAKS_ONLY) != 0;
     const uint32_t fill_flags = flags & (uint32_t)(HT_PEAKS_ONLY | HT_FILL_NAIVE);
-    if (po) {
-        std::string why;
-        s = hte::engine_ensure_edges(E, &why);
-        if (s != HT_OK) {
-            if (s == HT_E_CUDA)
-                b->poisoned = true;
-            return hte::report(s, why);
-        }
-    }
     if (n_events < 1 || n_events > E.max_events)
         return hte::report(HT_E_INVAL, "need 1 <= n_events <= max_events");
     if (n_hits > E.max_hits)

@@ -200,7 +200,6 @@ ht_status engine_configure(Engine &E, std::string *why)
     // A smaller peak buffer than the scan's (the tile needs the room); k_seam
     // keeps kPeakBuf in its own launch.
     E.fused_ok = false;
-    E.fused_capped = false;
     E.fused_K = std::max<uint32_t>(kFusedPeakBuf, f.threads);
     if (E.fill_priv_ok && t.fused != 2 && W <= 64 && b.n_b <= 4096) {
         htk::ScanArgs tmp{};
@@ -244,7 +243,6 @@ ht_status engine_configure(Engine &E, std::string *why)
             occ = 0;   // rows must start on 16 bytes; the block must cover whole rows
         E.fused_fill = ff;
         if (occ >= 1) {
-            E.fused_capped = t.fill_blocks_per_sm && (int)t.fill_blocks_per_sm < occ;
             if (t.fill_blocks_per_sm)
                 occ = std::min<int>(occ, (int)t.fill_blocks_per_sm);
             E.fused_ok = true;
@@ -278,35 +276,36 @@ ht_status engine_configure(Engine &E, std::string *why)
         return HT_E_INVAL;
     }
     E.use_ws = E.ws_ok;
-    // --- the tile fill ------------------------------------------------------------
-    E.tma_ok = false;
-    E.tma_capped = false;
+    // --- the tile fill, and the same without the writing (peaks-only fills) --------
+    E.tma_ok = E.tma_capped = E.po_ok = E.po_capped = false;
+    auto tile_fit = [&](bool store, uint32_t W, htk::TileCfg &out, uint32_t &grid, bool &capped) {
+        if (!W) {
+            W = 64;   // tiles of at most 16 KB, and lower ones while there are fewer passes than warps
+            while (W > 2 && ((size_t)W * b.n_b * 4 > 16 * 1024 ||
+                             (W > 4 && (uint64_t)E.max_events * g.n_slices * ((b.n_a + W - 1) / W) < 12ull * E.num_sms)))
+                W >>= 1;
+        }
+        const htk::TileCfg c = tile_shape(std::min<uint32_t>(W, 64));
+        int occ = 0;
+        if (htk::tile_smem_bytes(c) > kSmemMax || htk::tile_passes(g, c, E.max_events) > 0x7fffffffull ||
+            htk::fill_tma_occupancy(c, store, &occ) != cudaSuccess || occ < 1) {
+            cudaGetLastError();
+            return false;
+        }
+        capped = t.fill_blocks_per_sm && (int)t.fill_blocks_per_sm < occ;
+        if (t.fill_blocks_per_sm)
+            occ = std::min<int>(occ, (int)t.fill_blocks_per_sm);
+        out = c;
+        grid = (uint32_t)E.num_sms * (uint32_t)occ;
+        return true;
+    };
     // The default fused fill wherever it fits (fused 0 = auto).  Rows that are not
     // whole 16 bytes cost a tile up to six words written by hand: 999 x 1001 bins
     // against the thread-store fill that took them before, 121 -> 44 us per event with three in flight.
-    if (E.fill_priv_ok && (t.fused == 0 || (t.fused == 5 && (b.n_b & 3u) == 0)) && b.n_b <= 4096) {
-        uint32_t Wt = t.fill_W;
-        if (!Wt) {
-            Wt = 64;   // tiles of at most 16 KB, and lower ones while there are fewer passes than warps
-            while (Wt > 2 && ((size_t)Wt * b.n_b * 4 > 16 * 1024 ||
-                              (Wt > 4 && (uint64_t)E.max_events * g.n_slices * ((b.n_a + Wt - 1) / Wt) < 12ull * E.num_sms)))
-                Wt >>= 1;
-        }
-        const htk::TileCfg c = tile_shape(std::min<uint32_t>(Wt, 64));
-        int occ = 0;
-        if (htk::tile_smem_bytes(c) <= kSmemMax &&
-            (uint64_t)E.max_events * g.n_slices * c.strips <= 0x7fffffffull &&
-            htk::fill_tma_occupancy(c, &occ) == cudaSuccess && occ >= 1) {
-            E.tma_capped = t.fill_blocks_per_sm && (int)t.fill_blocks_per_sm < occ;
-            if (t.fill_blocks_per_sm)
-                occ = std::min<int>(occ, (int)t.fill_blocks_per_sm);
-            E.tma_ok = true;
-            E.tile = c;
-            E.tma_grid = (uint32_t)E.num_sms * (uint32_t)occ;
-        } else {
-            cudaGetLastError();
-        }
-    }
+    if (E.fill_priv_ok && (t.fused == 0 || (t.fused == 5 && (b.n_b & 3u) == 0)) && b.n_b <= 4096)
+        E.tma_ok = tile_fit(true, t.fill_W, E.tile, E.tma_grid, E.tma_capped);
+    if (E.fill_priv_ok && t.fused != 2 && b.n_b <= 4096)
+        E.po_ok = tile_fit(false, tma_mode ? t.fill_W : 0u, E.po_tile, E.po_grid, E.po_capped);
     if (t.fused == 5 && !E.tma_ok) {
         *why = "the bulk-copy-tile fused fill needs n_b a multiple of 4 (at most 4096) and tiles that fit";
         return HT_E_INVAL;
@@ -370,7 +369,8 @@ ht_status engine_configure(Engine &E, std::string *why)
     const uint64_t items_max = (uint64_t)E.max_events * g.n_slices * f.strips;
     const uint32_t fused_grid = E.fused_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.fused_grid, items_max)) : 0;
     const uint32_t ws_grid = E.ws_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.ws_grid, items_max)) : 0;
-    const uint64_t passes = E.tma_ok ? htk::tile_passes(g, E.tile, E.max_events) : 0;
+    E.max_passes = std::max(E.tma_ok ? htk::tile_passes(g, E.tile, E.max_events) : 0,
+                            E.po_ok ? htk::tile_passes(g, E.po_tile, E.max_events) : 0);
     // the fused fill's candidate lists: one per CTA plus one per handed-out item
     const uint32_t fused_lists = fused_grid + (uint32_t)htk::dyn_items(items_max, fused_grid);
     const uint32_t grid_cap = std::max(std::max(scan_grid, fused_lists), ws_grid);
@@ -379,7 +379,7 @@ ht_status engine_configure(Engine &E, std::string *why)
     // an even split (every strip costs at least its n_b-per-row writing share)
     const double hits_per_unit = (double)std::max<uint32_t>(E.max_hits, 1) * E.max_admit /
                                  ((double)E.max_events * g.n_slices);
-    const double spread = 1.0 + std::max(htk::kVoteWeight, htk::kPeaksVoteWeight) * hits_per_unit / g.nb;
+    const double spread = 1.0 + htk::kVoteWeight * hits_per_unit / g.nb;
     auto rows_per_cta = [&](uint32_t grid) {
         return (uint64_t)(std::ceil((double)items_max / grid * spread) + 2) * f.W + 1;
     };
@@ -395,7 +395,7 @@ ht_status engine_configure(Engine &E, std::string *why)
     s.seq_max = seq;
     const size_t desc_b = (size_t)grid_cap * seq * 8;
     const size_t cta_b = (size_t)grid_cap * 2 * 4;
-    const size_t pass_b = (size_t)passes * 8, seg_b = (size_t)(passes / htk::kOrderPasses + 1) * 4;
+    const size_t pass_b = (size_t)E.max_passes * 8, seg_b = (size_t)(E.max_passes / htk::kOrderPasses + 1) * 4;
     const size_t need = pass_b + desc_b + cta_b + seg_b;
     if (need > E.book_bytes || grid_cap != E.grid_cap) {
         if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
@@ -528,7 +528,6 @@ ht_status engine_create(Engine &E, const ht_binning *b, const ht_ranges *r, uint
     const uint32_t ctr_words = engine_ctr_words(E);
     const size_t units = (size_t)max_events * g.n_slices;
     const uint64_t list_cap = std::min<uint64_t>((uint64_t)hits_cap * E.max_admit, 0xffffffffull);
-    E.split_cap = (uint32_t)E.num_sms * 32 + 1;   // a fill grid of up to 32 CTAs per SM
     E.list_cap = (uint32_t)list_cap;
     if ((e = dalloc(&E.d_edges, (E.et.size() + E.ep.size() + E.bth.size()) * 4, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_M, (size_t)E.n_cells * 4 * max_events + 256, &acc)) != cudaSuccess ||
@@ -538,8 +537,7 @@ ht_status engine_create(Engine &E, const ht_binning *b, const ht_ranges *r, uint
         (e = dalloc(&E.d_list, (size_t)list_cap * 16, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_lines, ((size_t)list_cap + 2) * 8, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_entries, (size_t)s.entries_cap * 16, &acc)) != cudaSuccess ||
-        (e = dalloc(&E.d_ctr, (size_t)ctr_words * 4, &acc)) != cudaSuccess ||
-        (e = dalloc(&E.d_split, (size_t)E.split_cap * 8, &acc)) != cudaSuccess) {
+        (e = dalloc(&E.d_ctr, (size_t)ctr_words * 4, &acc)) != cudaSuccess) {
         std::snprintf(buf, sizeof buf, "device allocation of %zu bytes failed: %s", acc,
                       cudaGetErrorString(e));
         *why = buf;
@@ -613,10 +611,8 @@ void engine_destroy(Engine &E)
     cudaFree(E.d_hits4);
     cudaFree(E.d_codes);
     cudaFree(E.d_slice);
-    cudaFree(E.d_split);
     cudaFree(E.d_list);
     cudaFree(E.d_lines);
-    cudaFree(E.d_edge);
     cudaFree(E.d_entries);
     cudaFree(E.d_book);
     cudaFree(E.d_ctr);
@@ -625,11 +621,8 @@ void engine_destroy(Engine &E)
     E.d_hits4 = nullptr;
     E.d_codes = nullptr;
     E.d_slice = nullptr;
-    E.d_split = nullptr;
     E.d_list = nullptr;
     E.d_lines = nullptr;
-    E.d_edge = nullptr;
-    E.edge_pass = 0;
     E.d_entries = nullptr;
     E.d_book = nullptr;
     E.d_ctr = nullptr;
@@ -661,42 +654,20 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
     w.list_cap = E.list_cap;
     w.pass_peaks = E.pass_peaks;
     w.seg_peaks = E.seg_peaks;
-    w.n_seg = E.tma_ok ? (uint32_t)((htk::tile_passes(E.geom, E.tile, n_events) + htk::kOrderPasses - 1) / htk::kOrderPasses) : 0u;
-    w.edge = E.d_edge;
-    w.edge_pass = E.edge_pass;
-    w.split_mode = E.split_mode;
-    w.split_grid = E.split_grid;
-    w.split_strips = E.split_strips;
-    w.split_vw = E.split_vw;
-    w.split_n_static = E.split_n_static;
-    w.split = E.d_split;
+    w.n_seg = (uint32_t)((E.max_passes / E.max_events * n_events + htk::kOrderPasses - 1) / htk::kOrderPasses);
     return w;
 }
 
-// Whether engine_vote's fill for these flags is the tile fill or the
-// peaks-only fill, and then whether fill_blocks_per_sm holds it below its
-// occupancy; for the peaks-only fill also its configuration and grid, whose
-// work split k_bin_cluster hands over (the fill checks the shape and splits by
-// itself on a mismatch).
-enum NextFill { NEXT_OTHER, NEXT_TILES, NEXT_PEAKS };
-static NextFill next_fill(const Engine &E, uint32_t n_events, uint32_t flags, htk::FillCfg &ff, uint32_t &grid,
-                          bool &capped)
+// engine_vote's fill for these flags: the tile fill (TILES_MH: writing M_H,
+// TILES_PEAKS: for the peaks alone) or another one.
+enum VoteKind { OTHER_FILL, TILES_MH, TILES_PEAKS };
+static VoteKind vote_kind(const Engine &E, uint32_t flags)
 {
     if ((flags & (HT_FILL_NAIVE | HT_ACCUMULATE)) || !E.fill_priv_ok)
-        return NEXT_OTHER;
-    const bool peaks_only = (flags & HT_PEAKS_ONLY) && E.fused_ok && E.d_edge &&
-                            E.edge_pass * std::max<uint32_t>(1, E.fused_fill.W / 2) >= E.geom.na;
-    if (!peaks_only) {
-        capped = E.tma_capped;
-        return E.use_tma && !E.use_ws ? NEXT_TILES : NEXT_OTHER;
-    }
-    ff = E.fused_fill;
-    ff.vote_weight = htk::kPeaksVoteWeight;
-    ff.accumulate = 0u;
-    capped = E.fused_capped;
-    const uint64_t items = (uint64_t)n_events * E.geom.n_slices * ff.strips;
-    grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.fused_grid, items));
-    return grid + 1 <= E.split_cap ? NEXT_PEAKS : NEXT_OTHER;
+        return OTHER_FILL;
+    if ((flags & HT_PEAKS_ONLY) && E.po_ok)
+        return TILES_PEAKS;
+    return E.use_tma && !E.use_ws ? TILES_MH : OTHER_FILL;
 }
 
 cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *z,
@@ -704,11 +675,10 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
                         uint32_t n_total, uint32_t flags, cudaStream_t st)
 {
     E.fused_valid = false;
-    htk::FillCfg ff{};
-    uint32_t grid = 0;
-    bool capped = false;
-    const NextFill next = next_fill(E, n_events, flags, ff, grid, capped);
-    const bool want_cluster = E.tune.bin_cluster == 1 || (E.tune.bin_cluster == 0 && next != NEXT_OTHER && !capped);
+    // one binning launch ahead of a tile fill that has the SMs to itself
+    const VoteKind kind = vote_kind(E, flags);
+    const bool capped = kind == TILES_PEAKS ? E.po_capped : E.tma_capped;
+    const bool want_cluster = E.tune.bin_cluster == 1 || (E.tune.bin_cluster == 0 && kind != OTHER_FILL && !capped);
     const bool cluster = want_cluster && E.bin_cluster > 0 &&
                          n_total <= htk::kBinClusterMax * htk::kBinClusterThreads * htk::kBinClusterHPT &&
                          htk::bin_cluster_smem_bytes(E.geom, n_events) <= htk::kBinClusterSmem;
@@ -716,16 +686,6 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
     if (cluster) {
         // few hits: binning and unit lists in one cluster launch, one CTA per
         // kBinClusterThreads hits (two hits a thread past kBinClusterMax CTAs)
-        if (next == NEXT_PEAKS) {
-            const uint64_t items = (uint64_t)n_events * E.geom.n_slices * ff.strips;
-            E.split_mode = htk::kSplitGiven;
-            E.split_grid = grid;
-            E.split_strips = ff.strips;
-            E.split_vw = ff.vote_weight;
-            E.split_n_static = items - (ff.dyn ? htk::dyn_items(items, grid) : 0);
-        } else {
-            E.split_mode = htk::kSplitAfterWait;   // the offsets come from the launch right before the fill
-        }
         const htk::Work w = make_work(E, x, y, z, d_hit_off, n_hits0, n_events);
         const uint32_t cs = std::min<uint32_t>(
             htk::kBinClusterMax, std::max<uint32_t>(1u, (n_total + htk::kBinClusterThreads - 1) / htk::kBinClusterThreads));
@@ -737,7 +697,6 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
             return e;
         ++E.launches;
     } else {
-        E.split_mode = htk::kSplitEarly;
         const htk::Work w = make_work(E, x, y, z, d_hit_off, n_hits0, n_events);
         const uint32_t bgrid = std::max<uint32_t>(1, std::min<uint32_t>((n_total + 255) / 256, E.num_sms * 8));
         {
@@ -769,9 +728,8 @@ static cudaError_t engine_clear_counts(Engine &E, cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(E.d_ctr + htk::CTR_ENTRIES, 0,
                                     (engine_ctr_words(E) - htk::CTR_ENTRIES) * sizeof(uint32_t), st);
-    if (e == cudaSuccess && E.tma_ok)
-        e = cudaMemsetAsync(E.seg_peaks, 0,
-                            (htk::tile_passes(E.geom, E.tile, E.max_events) / htk::kOrderPasses + 1) * 4, st);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(E.seg_peaks, 0, (E.max_passes / htk::kOrderPasses + 1) * 4, st);
     return e;
 }
 
@@ -799,19 +757,20 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     htk::FillCfg f = E.fill;
     f.accumulate = accumulate ? 1u : 0u;
     const uint64_t items = (uint64_t)n_events * E.geom.n_slices * f.strips;
-    const bool peaks_only = (flags & HT_PEAKS_ONLY) && E.fused_ok && E.d_edge &&
-                            E.edge_pass * std::max<uint32_t>(1, E.fused_fill.W / 2) >= E.geom.na;
-    if (E.use_tma && !E.use_ws && !peaks_only && !accumulate) {
+    const VoteKind kind = vote_kind(E, flags);
+    if (kind != OTHER_FILL) {
+        const bool store = kind == TILES_MH;
+        const htk::TileCfg &c = store ? E.tile : E.po_tile;
         if (!fresh) {   // voted again without a binning (the autotuner)
             if ((e = engine_clear_counts(E, st)) != cudaSuccess)
                 return e;
         }
-        const uint64_t passes = htk::tile_passes(E.geom, E.tile, n_events);
-        const uint32_t grid =
-            (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.tma_grid, (passes + E.tile.warps - 1) / E.tile.warps));
+        const uint64_t passes = htk::tile_passes(E.geom, c, n_events);
+        const uint32_t grid = (uint32_t)std::max<uint64_t>(
+            1, std::min<uint64_t>(store ? E.tma_grid : E.po_grid, (passes + c.warps - 1) / c.warps));
         {
-            ProfScope ps(E, K_FILL_TMA, st);
-            e = htk::launch_fill_tma(E.geom, w, E.tile, E.scan, grid, st);
+            ProfScope ps(E, store ? K_FILL_TMA : K_FILL_PEAKS, st);
+            e = htk::launch_fill_tma(E.geom, w, c, E.scan, grid, store, st);
         }
         ++E.launches;
         if (e == cudaSuccess) {
@@ -824,25 +783,24 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     }
     if ((E.use_ws || E.fused_ok) && !accumulate) {
         htk::ScanArgs a = E.scan;
-        const bool ws = E.use_ws && !peaks_only;
+        const bool ws = E.use_ws;
         a.K = E.fused_K;
         htk::FillCfg ff = ws ? E.ws_fill : E.fused_fill;
         ff.accumulate = 0u;
-        ff.vote_weight = peaks_only ? htk::kPeaksVoteWeight : htk::kVoteWeight;
+        ff.vote_weight = htk::kVoteWeight;
         const uint64_t items_ff = (uint64_t)n_events * E.geom.n_slices * ff.strips;
         const uint32_t grid = (uint32_t)std::max<uint64_t>(
             1, std::min<uint64_t>(ws ? E.ws_grid : E.fused_grid, items_ff));
         const uint32_t lists = grid + (ff.dyn ? (uint32_t)htk::dyn_items(items_ff, grid) : 0u);
         {
-            ProfScope ps(E, ws ? K_FILL_WS : peaks_only ? K_FILL_PEAKS : K_FILL_SCAN, st);
+            ProfScope ps(E, ws ? K_FILL_WS : K_FILL_SCAN, st);
             e = ws ? htk::launch_fill_ws(E.geom, w, ff, a, grid, st)
-               : peaks_only ? htk::launch_fill_peaks(E.geom, w, ff, a, grid, st)
-                            : htk::launch_fill_scan(E.geom, w, ff, a, grid, st);
+               : htk::launch_fill_scan(E.geom, w, ff, a, grid, st);
         }
         ++E.launches;
         if (e == cudaSuccess) {
             ProfScope ps(E, K_PEAKS, st);
-            e = htk::launch_peaks(E.geom, w, ff, a, lists, peaks_only, st);
+            e = htk::launch_peaks(E.geom, w, a, lists, st);
             ++E.launches;
         }
         if (e == cudaSuccess) {
@@ -1122,32 +1080,6 @@ cudaError_t engine_set_phi_edges(Engine &E, const float *ep)
     // on the legacy stream the object's streams do not wait for
     cudaError_t e = cudaMemcpy(E.d_edges + E.et.size(), E.ep.data(), E.ep.size() * 4, cudaMemcpyHostToDevice);
     return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
-}
-
-ht_status engine_ensure_edges(Engine &E, std::string *why)
-{
-    // passes per unit at the smallest pass height (u32 tiles: W / 2 rows)
-    const uint32_t rpass_min = std::max<uint32_t>(1, E.fused_fill.W / 2);
-    const uint32_t passes = (E.geom.na + rpass_min - 1) / rpass_min;
-    if (E.d_edge && E.edge_pass >= passes)
-        return HT_OK;
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) {
-        *why = std::string("synchronise before allocation: ") + cudaGetErrorString(e);
-        return HT_E_CUDA;
-    }
-    cudaFree(E.d_edge);
-    E.d_edge = nullptr;
-    E.edge_pass = 0;
-    const size_t bytes = (size_t)E.max_events * E.geom.n_slices * passes * 2 * E.geom.nb * 4;
-    if ((e = cudaMalloc(&E.d_edge, bytes)) != cudaSuccess) {
-        cudaGetLastError();
-        *why = std::string("edge-row buffer allocation failed: ") + cudaGetErrorString(e);
-        return HT_E_NOMEM;
-    }
-    E.edge_pass = passes;
-    E.device_bytes += bytes;
-    return HT_OK;
 }
 
 } // namespace hte

@@ -73,6 +73,10 @@ struct Engine {
     bool tma_ok = false;         // the bulk-copy-tile fused kernel fits
     htk::TileCfg tile{};         // its shape
     uint32_t tma_grid = 0;
+    bool po_ok = false;          // the tile fill without the writing fits: peaks-only fills
+    htk::TileCfg po_tile{};
+    uint32_t po_grid = 0;
+    uint64_t max_passes = 0;     // of either, over max_events events
     uint2 *pass_peaks = nullptr; // (in d_book) its peaks per pass and per htk::kOrderPasses passes
     uint32_t *seg_peaks = nullptr;
     bool use_tma = false;        // fills run the bulk-copy-tile kernel
@@ -93,12 +97,7 @@ struct Engine {
     bool counts_fresh = false;   // the binning has just cleared every count the fill adds to
     int bin_cluster = -1;        // k_bin_cluster usable here (-1: not checked yet)
     bool tma_capped = false;     // fill_blocks_per_sm holds the bulk-copy-tile fill below its occupancy
-    bool fused_capped = false;   // ... and the fused fills (the peaks-only fill among them)
-    uint32_t split_mode = htk::kSplitEarly;   // Work::split_mode of the fill after the last binning
-    uint32_t split_grid = 0, split_strips = 0, split_vw = 0;
-    uint64_t split_n_static = 0;
-    uint64_t *d_split = nullptr;              // [split_cap] k_bin_cluster's split for the fill
-    uint32_t split_cap = 0;
+    bool po_capped = false;      // ... and the peaks-only fill
     const uint32_t *last_hit_off = nullptr;   // what the last fill binned
     uint32_t last_n_hits0 = 0, last_n_events = 0;
     bool last_accumulate = false;
@@ -107,8 +106,6 @@ struct Engine {
     uint32_t *d_M = nullptr;
     float4 *d_hits4 = nullptr;
     uint32_t *d_codes = nullptr;
-    uint32_t *d_edge = nullptr;   // peaks-only fills: edge rows of every pass (allocated on first use)
-    uint32_t edge_pass = 0;       // passes per unit the edge buffer holds
     uint32_t *d_slice = nullptr;  // unit counts | scatter cursors | offsets (3 * units + 1)
     float4 *d_list = nullptr;     // hit records unit by unit
     float2 *d_lines = nullptr;    // their vote lines
@@ -172,10 +169,6 @@ void engine_get_tuning(const Engine &E, ht_tuning *t);
 
 // Per-kernel totals into the ABI's records (waits for recorded events).
 cudaError_t prof_read(Engine &E, ht_kernel_time *out, uint32_t cap, uint32_t *n);
-
-// Allocate the edge-row buffer of peaks-only fills (once; synchronises the
-// device the first time).
-ht_status engine_ensure_edges(Engine &E, std::string *why);
 
 // Replace the phi edge table (n_phi + 1 pseudo-angles, host memory) on the
 // host and on the device (synchronous copy).  A sector context takes its

@@ -124,20 +124,16 @@ size_t fill_ws_smem_bytes(const FillCfg &c, const ScanArgs &a);
 cudaError_t launch_fill_ws(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
                            cudaStream_t st);
 cudaError_t fill_ws_occupancy(const FillCfg &c, const ScanArgs &a, int *blocks_per_sm);
-// The tile fill, and the ordering of the peaks it leaves pass by pass (one
-// event, or o.compact).
+// The tile fill (store: M_H is written, else only the peaks are found), and the
+// ordering of the peaks it leaves pass by pass (one event, or o.compact).
 cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a, uint32_t grid,
-                            cudaStream_t st);
-cudaError_t fill_tma_occupancy(const TileCfg &c, int *blocks_per_sm);
+                            bool store, cudaStream_t st);
+cudaError_t fill_tma_occupancy(const TileCfg &c, bool store, int *blocks_per_sm);
 cudaError_t launch_order_passes(const Geom &g, const Work &w, const ScanArgs &a, const OrderArgs &o, uint64_t passes,
                                 cudaStream_t st);
-// After a fused fill (same grid): test its candidate entries, keep the peaks
-// (peaks_only: after k_fill_peaks, finishing the edge-flagged tests).
-cudaError_t launch_peaks(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
-                         bool peaks_only, cudaStream_t st);
-// The fused fill without writing M_H (same shapes and grid as k_fill_scan).
-cudaError_t launch_fill_peaks(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
-                              cudaStream_t st);
+// After k_fill_scan, k_fill_bulk or k_fill_ws (same grid): test its candidate
+// entries, keep the peaks.
+cudaError_t launch_peaks(const Geom &g, const Work &w, const ScanArgs &a, uint32_t grid, cudaStream_t st);
 cudaError_t launch_clear(uint32_t *M, uint64_t words, uint32_t grid, cudaStream_t st);
 cudaError_t launch_fill_naive(const Geom &g, const Work &w, uint32_t num_sms, cudaStream_t st);
 size_t scan_smem_bytes(const ScanArgs &a);
@@ -153,13 +149,9 @@ enum : uint32_t {
 };
 
 // Cost model of the balanced split of (event, slice, strip) work items over
-// the fill CTAs: a strip of r rows in a slice of h hits costs
-// r * (n_b + v * h) (writing a cell ~ 1, one vote ~ v = FillCfg::vote_weight).
-// The fills that write M_H take kVoteWeight; the peaks-only fill, whose
-// cells cost only their clearing, weighs votes more (kPeaksVoteWeight; 6,
-// 12 and 24 were measured on paper-scale events, 24 balancing its CTAs best).
+// the CTAs of the fills other than the tile fill: a strip of r rows in a slice
+// of h hits costs r * (n_b + v * h) (writing a cell ~ 1, one vote ~ v).
 constexpr uint32_t kVoteWeight = 6;
-constexpr uint32_t kPeaksVoteWeight = 24;
 
 // Scan variants: bulk-copy (TMA) ring, register streaming, direct (any n_b).
 // The streaming variant keeps kLdgUPT 16-byte loads per thread in flight.

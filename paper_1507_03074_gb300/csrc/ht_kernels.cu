@@ -7,8 +7,7 @@
 //                 x, x^2 + y^2, 2y of the vote.
 //   k_scatter     the admitted hits into per-(event, slice) unit lists.
 //   k_bin_cluster k_bin + k_scatter in one thread-block cluster for launches
-//                 of few hits (distributed shared memory for the counts),
-//                 which also writes the work split of the fill after it.
+//                 of few hits (distributed shared memory for the counts).
 //   k_fill_tma    Step 1 fused with step 2 (default): a warp votes a pass of W
 //                 A-rows into a u32 shared-memory tile of its own, laid out as
 //                 M_H's rows, which leaves as one bulk copy; a vote taking a
@@ -100,9 +99,8 @@ struct WarpGroup {
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream launch once every CTA of this one has
 // passed this point (its grid_dep_wait still waits for this kernel to end).
-// Only k_scatter uses it, after its own wait: what k_bin wrote is then
-// complete when the fill after k_scatter starts, so the fill may read the
-// unit offsets before its own wait.
+// k_scatter and k_bin_cluster use it: the fill's set-up (clearing its tiles)
+// then overlaps the binning's end.
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Exclusive scan of n values in shared memory (in place); returns the total.
@@ -268,78 +266,6 @@ __global__ void __launch_bounds__(256) k_scatter(Geom g, Work w)
         w.slice_cnt[u] = 0u;
 }
 
-// The static split of the fill that follows (the split cta_items computes,
-// for the shape Work::split_* names), from unit offsets off[0..U) in shared
-// memory and their total: split[c] = the first static item of fill CTA c.
-// Work item cost as in cta_items: g.na * (g.nb * u + vote weight * off[u])
-// up to unit u, strictly increasing in u; a CTA boundary at cost T falls in
-// the unit u with cost(u) <= T < cost(u + 1), at the strip it reaches.
-// Int: the arithmetic type, uint32_t when every cost (and G * G) is below
-// 2^31, which spares the 64-bit divisions.
-template <typename Int>
-__device__ __forceinline__ void split_for_fill_t(const Geom &g, const Work &w, const uint32_t *off, uint32_t total,
-                                                 uint64_t tot64)
-{
-    const uint32_t U = w.n_events * g.n_slices, G = w.split_grid, S = w.split_strips;
-    const uint64_t ns = w.split_n_static;
-    auto cost = [&](uint32_t u) {
-        return (Int)((uint64_t)g.na * ((uint64_t)g.nb * u + (uint64_t)w.split_vw * (u < U ? off[u] : total)));
-    };
-    const Int tot = (Int)tot64, c_end = cost(U), q = tot / G, r = tot % G;
-    for (uint32_t c = threadIdx.x; c <= G; c += blockDim.x) {
-        uint64_t item = ns;
-        if (c == 0) {
-            item = 0;
-        } else if (c < G) {
-            const Int T = q * c + (r * c) / G;
-            if (T < c_end) {
-                uint32_t lo = 0, hi = U - 1;
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi + 1) >> 1;
-                    if (cost(mid) <= T)
-                        lo = mid;
-                    else
-                        hi = mid - 1;
-                }
-                const Int a = cost(lo), b = cost(lo + 1);
-                const Int per = (b - a + S - 1) / S;
-                const Int k = (T - a) / per;
-                item = min((uint64_t)lo * S + min((uint64_t)k, (uint64_t)S - 1), ns);
-            }
-        }
-        w.split[c] = item;
-    }
-}
-
-__device__ void split_for_fill(const Geom &g, const Work &w, const uint32_t *off, uint32_t total)
-{
-    const uint32_t U = w.n_events * g.n_slices, G = w.split_grid, S = w.split_strips;
-    const uint64_t ns = w.split_n_static;
-    auto cost = [&](uint32_t u) {
-        return (uint64_t)g.na * ((uint64_t)g.nb * u + (uint64_t)w.split_vw * (u < U ? off[u] : total));
-    };
-    const bool small = cost(U) < (1ull << 31) && ns < (1ull << 31) && (uint64_t)G * (G + 1) < (1ull << 31) &&
-                       S < (1u << 30);
-    // the cost of the first ns items
-    uint64_t tot;
-    if (small) {
-        const uint32_t n32 = (uint32_t)ns, us = n32 / S, ks = n32 % S;
-        uint32_t t = (uint32_t)cost(us);
-        if (ks)
-            t += ks * (((uint32_t)cost(us + 1) - t + S - 1) / S);
-        tot = t;
-    } else {
-        const uint32_t us = (uint32_t)(ns / S), ks = (uint32_t)(ns % S);
-        tot = cost(us);
-        if (ks)
-            tot += ks * ((cost(us + 1) - tot + S - 1) / S);
-    }
-    if (small)
-        split_for_fill_t<uint32_t>(g, w, off, total, tot);
-    else
-        split_for_fill_t<uint64_t>(g, w, off, total, tot);
-}
-
 // k_bin and k_scatter in one launch for launches of few hits: one cluster of
 // up to kBinClusterMax CTAs.  Each CTA counts its hits per unit in its own
 // shared memory; after one cluster barrier every CTA reads all the CTAs'
@@ -458,8 +384,6 @@ __global__ void __launch_bounds__(1024, 1) k_bin_cluster(Geom g, Work w)
             }
         });
     }
-    if (rank == 0 && w.split_mode == kSplitGiven)
-        split_for_fill(g, w, s_tot, total);
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -484,57 +408,23 @@ struct FlushList {
     uint32_t cap;
 };
 
-// Votes of tile cell (r, j) (u16 or u32 counters, row swizzle as vote_rows).
-__device__ __forceinline__ uint32_t tile_cell(const uint32_t *tile, uint32_t pitch, bool u16, uint32_t r, uint32_t j)
-{
-    if (u16)
-        return (tile[r * pitch + ((j >> 1) ^ (row_hash(r) & 0x1Eu))] >> ((j & 1u) << 4)) & 0xffffu;
-    return tile[r * pitch + (j ^ (row_hash(r) & 0x1Cu))];
-}
-
-// A cell of row r that just reached T: mark the row, list the cell.
-__device__ __forceinline__ void note_candidate(const FlushList &L, uint32_t r, uint32_t key)
-{
-    atomicOr(&L.hot[r >> 5], 1u << (r & 31u));
-    const uint32_t p = atomicAdd(L.n, 1u);
-    if (p < L.cap)
-        L.cand[p] = key;
-}
-
 // Votes of hits hs[hl], hs[hl + hstride], .. < nc (the vote lines of the
 // records rec[0 .. nc)) into tile row r (A bin i).
-// With LIST, a vote that lifts its cell from T - 1 to T lists the cell
-// (note_candidate): votes are +1 increments and T >= 1 (the context
-// rejects T = 0), so every cell >= T is listed exactly once.
-template <bool U16, bool LIST = false>
+template <bool U16>
 __device__ __forceinline__ void vote_rows(const Geom &g, uint32_t *tile, const float2 *hs, const float4 *rec,
                                           uint32_t nc, uint32_t r, uint32_t i, uint32_t hl, uint32_t hstride,
-                                          uint32_t pitch, const FlushList &L = FlushList{})
+                                          uint32_t pitch)
 {
     const uint32_t rowbase = r * pitch;
     const uint32_t sw = U16 ? (row_hash(r) & 0x1Eu) : (row_hash(r) & 0x1Cu);
-    const uint32_t tm1 = g.threshold - 1u;
 #pragma unroll 4
     for (uint32_t h = hl; h < nc; h += hstride) {
         const uint32_t j = vote_bin_line(g, hs[h], i, rec + h);
         if (j < g.nb) {
-            if (U16) {
-                const uint32_t word = rowbase + ((j >> 1) ^ sw);
-                const uint32_t sh = (j & 1u) << 4;
-                if (LIST) {
-                    if (((atomicAdd(&tile[word], 1u << sh) >> sh) & 0xffffu) == tm1)
-                        note_candidate(L, r, r * g.nb + j);
-                } else {
-                    atomicAdd(&tile[word], 1u << sh);
-                }
-            } else {
-                if (LIST) {
-                    if (atomicAdd(&tile[rowbase + (j ^ sw)], 1u) == tm1)
-                        note_candidate(L, r, r * g.nb + j);
-                } else {
-                    atomicAdd(&tile[rowbase + (j ^ sw)], 1u);
-                }
-            }
+            if (U16)
+                atomicAdd(&tile[rowbase + ((j >> 1) ^ sw)], 1u << ((j & 1u) << 4));
+            else
+                atomicAdd(&tile[rowbase + (j ^ sw)], 1u);
         }
     }
 }
@@ -678,20 +568,20 @@ __device__ __forceinline__ uint32_t stage_hits(const Work &w, float2 *hs, uint32
 // (cached_es / cached_n).  SYNC: a cached pass starts with a group barrier
 // (the previous pass's readers of the tile are done); without it the caller
 // orders the tile by other means.  All threads of the group call it.
-template <class G, bool SYNC, bool LIST>
+template <class G, bool SYNC>
 __device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t *tile, float2 *hs, uint32_t HC,
                                           uint64_t es, uint32_t l0, uint32_t l1, uint64_t &cached_es,
                                           uint32_t &cached_n, bool u16, uint32_t r, uint32_t pr, uint32_t i,
-                                          uint32_t hl, uint32_t hstride, uint32_t pitch, const FlushList &L)
+                                          uint32_t hl, uint32_t hstride, uint32_t pitch)
 {
     if (cached_es == es) {
         if (SYNC)
             G::sync();
         if (r < pr) {
             if (u16)
-                vote_rows<true, LIST>(g, tile, hs, w.list + l0, cached_n, r, i, hl, hstride, pitch, L);
+                vote_rows<true>(g, tile, hs, w.list + l0, cached_n, r, i, hl, hstride, pitch);
             else
-                vote_rows<false, LIST>(g, tile, hs, w.list + l0, cached_n, r, i, hl, hstride, pitch, L);
+                vote_rows<false>(g, tile, hs, w.list + l0, cached_n, r, i, hl, hstride, pitch);
         }
         return;
     }
@@ -708,9 +598,9 @@ __device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t
         first = false;
         if (r < pr) {
             if (u16)
-                vote_rows<true, LIST>(g, tile, hs, rec, nsel, r, i, hl, hstride, pitch, L);
+                vote_rows<true>(g, tile, hs, rec, nsel, r, i, hl, hstride, pitch);
             else
-                vote_rows<false, LIST>(g, tile, hs, rec, nsel, r, i, hl, hstride, pitch, L);
+                vote_rows<false>(g, tile, hs, rec, nsel, r, i, hl, hstride, pitch);
         }
     }
 }
@@ -849,8 +739,8 @@ __global__ void __launch_bounds__(1024) k_fill_priv(Geom g, Work w, FillCfg c)
         for (uint32_t p0 = 0; p0 < rows; p0 += rpass) {
             const uint32_t pr = min(rpass, rows - p0);
             const uint32_t i = i0 + p0 + r;
-            vote_pass<BlockGroup, true, false>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
-                                               i, hl, hstride, pitch, FlushList{});
+            vote_pass<BlockGroup, true>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
+                                               i, hl, hstride, pitch);
             __syncthreads();
             uint32_t *dst = Mrow + (size_t)p0 * g.nb;
             if (c.accumulate) {
@@ -1355,24 +1245,6 @@ __device__ __forceinline__ void emit_pass(const Geom &g, const Work &w, const Sc
     }
 }
 
-// Rank-sort the n_c (<= kFusedCand) distinct keys r * n_b + j of cand into
-// srt, with their votes read from the tile into srtv.  All threads of the
-// group call it; the caller synchronises before srt / srtv are read.
-template <class G, bool U16>
-__device__ __forceinline__ void sort_tile_candidates(const Geom &g, const uint32_t *tile, uint32_t pitch,
-                                                     const uint32_t *cand, uint32_t n_c, uint32_t *srt, uint32_t *srtv)
-{
-    for (uint32_t k = G::rank(); k < n_c; k += G::size()) {
-        const uint32_t key = cand[k];
-        uint32_t rank = 0;
-        for (uint32_t m = 0; m < n_c; ++m)
-            rank += cand[m] < key;
-        const uint32_t rr = key / g.nb;
-        srt[rank] = key;
-        srtv[rank] = tile_cell(tile, pitch, U16, rr, key - rr * g.nb);
-    }
-}
-
 // Write one pass from the tile to M_H, clear the tile, and emit its
 // candidates (emit_pass).  empty_bar: arrived on once the tile is clear
 // (the warp-specialised fill), or null.  All threads of the group call it.
@@ -1519,8 +1391,8 @@ __device__ __forceinline__ void fill_scan_body(const Geom &g, const Work &w, con
             // ---- vote (no barrier first: the previous pass, the previous item's
             // hand-out or the set-up ended with one) ---------------------------
             const uint32_t i = iA + r;
-            vote_pass<BlockGroup, false, false>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
-                                                i, hl, hstride, pitch, FlushList{});
+            vote_pass<BlockGroup, false>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
+                                                i, hl, hstride, pitch);
             // ---- write the pass, clear the tile, emit its candidates --------
             if (BULK) {
                 if (u16)
@@ -1568,218 +1440,6 @@ __global__ void __launch_bounds__(1024) k_fill_scan(Geom g, Work w, FillCfg c, S
 __global__ void __launch_bounds__(1024) k_fill_bulk(Geom g, Work w, FillCfg c, ScanArgs a)
 {
     fill_scan_body<true>(g, w, c, a);
-}
-
-// ---------------------------------------------------------------------------
-// k_fill_peaks: the fused fill without M_H in HBM (peaks-only fills).
-//
-// The passes are voted as in k_fill_scan, but the tile is not written out.
-// The votes themselves list the cells that reach T (vote_rows with LIST),
-// so no pass scans its tile for candidates: the listed cells are tested at
-// once against the neighbours the tile holds, and the pass's first and last
-// rows go to a small edge buffer.  A cell on the first (last) row of its
-// pass whose row above (below) belongs to another pass is emitted with a
-// flag; k_peaks finishes its test from the edge rows.  The output is the
-// same ordered peak list; M_H is left as it was.
-// ---------------------------------------------------------------------------
-
-// Test of cell (r, j) with votes v against the neighbours inside the tile
-// rows 0 .. pr - 1 (rule of Sec. 3 as read: > neighbours before it, >= after).
-__device__ __forceinline__ bool tile_peak(const uint32_t *tile, uint32_t pitch, bool u16, uint32_t pr, uint32_t nb,
-                                          uint32_t r, uint32_t j, uint32_t v)
-{
-    const bool hl = j > 0, hr = j + 1 < nb;
-    if (r > 0) {
-        if (hl && !(v > tile_cell(tile, pitch, u16, r - 1, j - 1))) return false;
-        if (!(v > tile_cell(tile, pitch, u16, r - 1, j))) return false;
-        if (hr && !(v > tile_cell(tile, pitch, u16, r - 1, j + 1))) return false;
-    }
-    if (hl && !(v > tile_cell(tile, pitch, u16, r, j - 1))) return false;
-    if (hr && !(v >= tile_cell(tile, pitch, u16, r, j + 1))) return false;
-    if (r + 1 < pr) {
-        if (hl && !(v >= tile_cell(tile, pitch, u16, r + 1, j - 1))) return false;
-        if (!(v >= tile_cell(tile, pitch, u16, r + 1, j))) return false;
-        if (hr && !(v >= tile_cell(tile, pitch, u16, r + 1, j + 1))) return false;
-    }
-    return true;
-}
-
-// Copy the first and last rows of a voted pass (tile rows 0 and rows - 1)
-// to edge[0, n_b) and edge[n_b, 2 n_b), 4 cells per thread and step when
-// n_b % 4 == 0.  The tile is left as it is.
-template <bool U16>
-__device__ __forceinline__ void edge_rows(const Geom &g, const uint32_t *tile, uint32_t rows, uint32_t pitch,
-                                          uint32_t *edge)
-{
-    const uint32_t tid = threadIdx.x, bd = blockDim.x, nb = g.nb;
-    if ((nb & 3u) == 0) {
-        const uint32_t q = nb >> 2;
-        for (uint32_t u = tid; u < 2 * q; u += bd) {
-            const uint32_t side = u >= q, c4 = u - side * q, r = side ? rows - 1 : 0;
-            uint4 v;
-            if (U16) {
-                const uint2 pr =
-                    *reinterpret_cast<const uint2 *>(&tile[r * pitch + ((2u * c4) ^ (row_hash(r) & 0x1Eu))]);
-                v = make_uint4(pr.x & 0xffffu, pr.x >> 16, pr.y & 0xffffu, pr.y >> 16);
-            } else {
-                v = *reinterpret_cast<const uint4 *>(&tile[r * pitch + ((4u * c4) ^ (row_hash(r) & 0x1Cu))]);
-            }
-            reinterpret_cast<uint4 *>(edge)[u] = v;
-        }
-    } else {
-        for (uint32_t u = tid; u < 2 * nb; u += bd) {
-            const uint32_t side = u >= nb, j = u - side * nb;
-            edge[u] = tile_cell(tile, pitch, U16, side ? rows - 1 : 0, j);
-        }
-    }
-}
-
-// Edge-flag bits of a peaks-only entry (in its .w): its test still needs
-// the row above / below, which lies in another pass.
-enum : uint32_t { EDGE_UP = 1u, EDGE_DN = 2u };
-
-__global__ void __launch_bounds__(1024) k_fill_peaks(Geom g, Work w, FillCfg c, ScanArgs a)
-{
-    extern __shared__ uint4 sm4[];
-    // layout as k_fill_scan
-    ScanSmem &ss = *reinterpret_cast<ScanSmem *>(sm4);
-    uint4 *pbuf = sm4 + 16;
-    uint32_t *tile = reinterpret_cast<uint32_t *>(pbuf + a.K);
-    float2 *hs = reinterpret_cast<float2 *>(tile + c.tile_words);
-    uint32_t *lists = reinterpret_cast<uint32_t *>(hs + c.HC);
-    uint32_t *cand = lists, *srt = lists + 2 * kFusedCand, *srtv = lists + 3 * kFusedCand;
-    __shared__ uint32_t s_hot[2], s_nc;
-
-    const uint32_t tid = threadIdx.x, bd = blockDim.x, nb = g.nb, T = g.threshold;
-    if (tid == 0)
-        s_hot[0] = s_hot[1] = s_nc = 0u;
-    for (uint32_t k = tid; k < c.tile_words / 4; k += bd)
-        sm4[16 + a.K + k] = make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t cta = blockIdx.x;
-    ChunkList inner = interior_list(a, cta);
-
-    // the static split as in k_fill_tma (Work::split_mode)
-    __shared__ unsigned long long s_rng[2];
-    __shared__ uint32_t s_dyn;
-    const uint64_t items = (uint64_t)w.n_events * g.n_slices * c.strips;
-    const uint64_t n_dyn = c.dyn ? dyn_items(items, gridDim.x) : 0, n_static = items - n_dyn;
-    uint64_t it0, it1;
-    if (w.split_mode == kSplitEarly)
-        cta_items(g, w, c, cta, gridDim.x, n_static, it0, it1, s_rng);
-    grid_dep_wait();   // the unit lists (and, after k_bin_cluster, the offsets and split)
-    if (w.split_mode == kSplitGiven && w.split_grid == gridDim.x && w.split_strips == c.strips &&
-        w.split_vw == c.vote_weight && w.split_n_static == n_static) {
-        it0 = __ldcg(&w.split[cta]);
-        it1 = __ldcg(&w.split[cta + 1]);
-    } else if (w.split_mode != kSplitEarly) {
-        cta_items(g, w, c, cta, gridDim.x, n_static, it0, it1, s_rng);
-    }
-    uint64_t cached_es = ~0ull;
-    uint32_t cached_n = 0;
-    uint32_t buf_n = 0, nseq = 0, total = 0;
-    const uint32_t rc = fused_round(bd, a.K);
-
-    auto do_item = [&](const ItemCursor &cur) {
-        const uint32_t k = cur.k;
-        const uint64_t es = cur.es;
-        const uint32_t s = cur.s;
-        const uint32_t e = cur.e;
-        const uint32_t l0 = __ldg(&w.slice_off[es]), l1 = __ldg(&w.slice_off[es + 1]);
-        const uint32_t i0 = k * c.W;
-        const uint32_t rows = min(c.W, g.na - i0);
-        const bool u16 = (l1 - l0) < 65536u;
-        const uint32_t rpass = u16 ? c.W : c.W / 2;
-        const uint32_t pitch = u16 ? c.pitch16 : c.pitch32;
-        const uint32_t slice_lin0 = s * g.na * nb;
-        const uint32_t r = tid % rpass, hl = tid / rpass, hstride = bd / rpass;
-
-        for (uint32_t p0 = 0; p0 < rows; p0 += rpass) {
-            const uint32_t pr = min(rpass, rows - p0);
-            const uint32_t iA = i0 + p0;
-            // ---- vote -------------------------------------------------------
-            const uint32_t i = iA + r;
-            const FlushList L{s_hot, lists, nullptr, &s_nc, kFusedCand};
-            vote_pass<BlockGroup, true, true>(g, w, tile, hs, c.HC, es, l0, l1, cached_es, cached_n, u16, r, pr,
-                                              i, hl, hstride, pitch, L);
-            __syncthreads();   // the pass's votes and their candidate list are complete
-            const uint32_t n_c = s_nc;
-            const uint64_t hotm = (uint64_t)s_hot[0] | ((uint64_t)s_hot[1] << 32);
-            // ---- the pass's first and last rows to the edge buffer ------------
-            const uint32_t pass = iA / rpass;
-            uint32_t *edge = w.edge + ((size_t)es * w.edge_pass + pass) * 2 * nb;
-            if (u16)
-                edge_rows<true>(g, tile, pr, pitch, edge);
-            else
-                edge_rows<false>(g, tile, pr, pitch, edge);
-            const bool up_out = iA > 0, dn_out = iA + pr < g.na;   // neighbours in other passes
-            // ---- test against the tile, emit peaks and flagged edge cells ----
-            if (n_c) {
-                const bool fits = n_c <= kFusedCand;
-                if (fits) {
-                    if (u16)
-                        sort_tile_candidates<BlockGroup, true>(g, tile, pitch, cand, n_c, srt, srtv);
-                    else
-                        sort_tile_candidates<BlockGroup, false>(g, tile, pitch, cand, n_c, srt, srtv);
-                    __syncthreads();
-                }
-                // rounds of rc cells: the sorted list, or every cell of the hot rows
-                const uint32_t m_total = fits ? n_c : pr * nb;
-                for (uint32_t base = 0; base < m_total; base += rc) {
-                    const uint32_t q = base + tid;
-                    uint32_t has = 0;
-                    uint4 ent = make_uint4(0u, 0u, 0u, 0u);
-                    if (tid < rc && q < m_total) {
-                        uint32_t key, v;
-                        bool ok = true;
-                        if (fits) {
-                            key = srt[q];
-                            v = srtv[q];
-                        } else {
-                            key = q;
-                            const uint32_t rr = q / nb;
-                            ok = (hotm >> rr) & 1ull;
-                            v = ok ? tile_cell(tile, pitch, u16, rr, q - rr * nb) : 0u;
-                            ok = ok && v >= T;
-                        }
-                        if (ok) {
-                            const uint32_t rr = key / nb, j = key - rr * nb;
-                            if (tile_peak(tile, pitch, u16, pr, nb, rr, j, v)) {
-                                const uint32_t flags = (rr == 0 && up_out ? EDGE_UP : 0u) |
-                                                       (rr == pr - 1 && dn_out ? EDGE_DN : 0u);
-                                has = 1;
-                                ent = make_uint4(slice_lin0 + iA * nb + key, e, v, flags);
-                            }
-                        }
-                    }
-                    if (__syncthreads_or(has)) {
-                        if (buf_n + rc > a.K)
-                            flush_chunk(a, ss, pbuf, buf_n, nseq, inner, w.status);
-                        compact_entry<BlockGroup, false>(ss, pbuf, buf_n, has, ent, nullptr);
-                        total += ss.round_total;
-                    }
-                }
-            }
-            __syncthreads();
-            // ---- clear the tile and the lists for the next pass ----------------
-            for (uint32_t q = tid; q < pr * pitch / 4; q += bd)
-                reinterpret_cast<uint4 *>(tile)[q] = make_uint4(0u, 0u, 0u, 0u);
-            if (tid == 0)
-                s_hot[0] = s_hot[1] = s_nc = 0u;   // the next votes start with a barrier
-        }
-    };
-    ItemCursor cur(g, c, it0);
-    for (uint64_t item = it0; item < it1; ++item, cur.next(g, c))
-        do_item(cur);
-    finish_candidates<BlockGroup>(w, a, ss, pbuf, buf_n, nseq, total, inner, cta);
-    if (c.dyn) {
-        for (uint32_t d; (d = next_dyn_item(w, (uint32_t)n_dyn, &s_dyn)) < n_dyn;) {
-            const uint32_t list = gridDim.x + d;
-            inner = interior_list(a, list);
-            buf_n = nseq = total = 0;
-            do_item(ItemCursor(g, c, n_static + d));
-            finish_candidates<BlockGroup>(w, a, ss, pbuf, buf_n, nseq, total, inner, list);
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1875,8 +1535,8 @@ __global__ void __launch_bounds__(1024, 1) k_fill_ws(Geom g, Work w, FillCfg c, 
                     }
                 }
                 const uint32_t i = t.i0 + p0 + r;
-                vote_pass<VoteGroup, false, false>(g, w, tile, hs, c.HC, t.es, t.l0, t.l1, cached_es, cached_n,
-                                                   t.u16, r, pr, i, hl, hstride, t.pitch, FlushList{});
+                vote_pass<VoteGroup, false>(g, w, tile, hs, c.HC, t.es, t.l0, t.l1, cached_es, cached_n,
+                                                   t.u16, r, pr, i, hl, hstride, t.pitch);
                 mbar_arrive(&bars[b]);   // tile b holds pass p
             }
         }
@@ -1927,7 +1587,7 @@ __global__ void __launch_bounds__(1024, 1) k_fill_ws(Geom g, Work w, FillCfg c, 
 // entries against their neighbours in the now complete M_H and compacts
 // every chunk in place to its peaks (order kept), counting them per event.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_peaks(Geom g, Work w, FillCfg c, ScanArgs a, uint32_t peaks_only)
+__global__ void __launch_bounds__(256) k_peaks(Geom g, Work w, ScanArgs a)
 {
     grid_dep_wait();
     __shared__ uint32_t s_wsum[40];
@@ -1946,29 +1606,9 @@ __global__ void __launch_bounds__(256) k_peaks(Geom g, Work w, FillCfg c, ScanAr
             if (k < d.y && d.x + k < a.entries_cap) {
                 en = a.entries[d.x + k];
                 const uint32_t s = en.x / sl, rem = en.x - s * sl, i = rem / g.nb, j = rem - i * g.nb;
-                if (!peaks_only) {
-                    const uint32_t *row = w.M + (size_t)en.y * w.n_cells + (size_t)(s * g.na + i) * g.nb;
-                    has = is_peak_l2(row, i > 0 ? row - g.nb : nullptr, i + 1 < g.na ? row + g.nb : nullptr, j,
-                                     g.nb, en.z) ? 1u : 0u;
-                } else {
-                    // the rows above / below from the edge rows of the neighbouring passes
-                    const uint32_t u = en.y * g.n_slices + s;
-                    const bool u16 = (__ldg(&w.slice_off[u + 1]) - __ldg(&w.slice_off[u])) < 65536u;
-                    const uint32_t rpass = u16 ? c.W : c.W / 2, pass = i / rpass;
-                    const uint32_t *eu = w.edge + (size_t)u * w.edge_pass * 2 * g.nb;
-                    const uint32_t *up = (en.w & EDGE_UP) ? eu + ((size_t)(pass - 1) * 2 + 1) * g.nb : nullptr;
-                    const uint32_t *dn = (en.w & EDGE_DN) ? eu + ((size_t)(pass + 1) * 2) * g.nb : nullptr;
-                    const bool hl = j > 0, hr = j + 1 < g.nb;
-                    const uint32_t v = en.z;
-                    bool ok = true;
-                    if (up)
-                        ok = (!hl || v > __ldcg(up + j - 1)) && v > __ldcg(up + j) && (!hr || v > __ldcg(up + j + 1));
-                    if (dn)
-                        ok = ok && (!hl || v >= __ldcg(dn + j - 1)) && v >= __ldcg(dn + j) &&
-                             (!hr || v >= __ldcg(dn + j + 1));
-                    has = ok ? 1u : 0u;
-                    en.w = 0u;
-                }
+                const uint32_t *row = w.M + (size_t)en.y * w.n_cells + (size_t)(s * g.na + i) * g.nb;
+                has = is_peak_l2(row, i > 0 ? row - g.nb : nullptr, i + 1 < g.na ? row + g.nb : nullptr, j, g.nb,
+                                 en.z) ? 1u : 0u;
             }
             // stable compaction: every read of this round happens before the
             // barrier, every write after, and no write passes its own read
@@ -2596,7 +2236,10 @@ __device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const 
     put_bits();
 }
 
-// STORE: the tiles go to M_H (else the peaks are all that is wanted).  AGG:
+// STORE: the tiles go to M_H, else the peaks are all that is wanted (the same
+// passes without the copies: 29.4 us for a paper event, 23.5 us per event in
+// flight; the u16 tiles of 512 threads that it replaces, whose cross-pass tests
+// went through rows in global memory and k_peaks, 31.8 and 31.5 us).  AGG:
 // warp-aggregated vote increments (vote_tile).  passes: over all events; runs:
 // runs of c.run passes per CTA, the passes behind them being handed out.
 template <bool STORE, bool AGG>
@@ -2938,33 +2581,24 @@ cudaError_t fill_ws_occupancy(const FillCfg &c, const ScanArgs &a, int *blocks_p
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_fill_ws, kWsThreads, smem);
 }
 
-cudaError_t launch_peaks(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
-                         bool peaks_only, cudaStream_t st)
+cudaError_t launch_peaks(const Geom &g, const Work &w, const ScanArgs &a, uint32_t grid, cudaStream_t st)
 {
-    return launch_pdl(k_peaks, grid, 256, 0, st, g, w, c, a, peaks_only ? 1u : 0u);
-}
-
-cudaError_t launch_fill_peaks(const Geom &g, const Work &w, const FillCfg &c, const ScanArgs &a, uint32_t grid,
-                              cudaStream_t st)
-{
-    const size_t smem = fill_scan_smem_bytes(c, a, g.nb);
-    cudaError_t e = allow_smem((const void *)k_fill_peaks, smem);
-    if (e != cudaSuccess)
-        return e;
-    return launch_pdl(k_fill_peaks, grid, c.threads, smem, st, g, w, c, a);
+    return launch_pdl(k_peaks, grid, 256, 0, st, g, w, a);
 }
 
 using TileKernel = void (*)(Geom, Work, TileCfg, ScanArgs, uint32_t, uint32_t);
-static TileKernel tile_kernel(const TileCfg &c)
+static TileKernel tile_kernel(const TileCfg &c, bool store)
 {
+    if (!store)
+        return k_fill_tma<false, false>;
     return c.vote_agg ? k_fill_tma<true, true> : k_fill_tma<true, false>;
 }
 
 cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a, uint32_t grid,
-                            cudaStream_t st)
+                            bool store, cudaStream_t st)
 {
     const size_t smem = tile_smem_bytes(c);
-    const TileKernel k = tile_kernel(c);
+    const TileKernel k = tile_kernel(c, store);
     cudaError_t e = allow_smem((const void *)k, smem);
     if (e != cudaSuccess)
         return e;
@@ -2978,10 +2612,10 @@ cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, cons
     return launch_pdl(k, grid, c.warps * 32u, smem, st, g, w, c, a, passes, runs);
 }
 
-cudaError_t fill_tma_occupancy(const TileCfg &c, int *blocks_per_sm)
+cudaError_t fill_tma_occupancy(const TileCfg &c, bool store, int *blocks_per_sm)
 {
     const size_t smem = tile_smem_bytes(c);
-    const TileKernel k = tile_kernel(c);
+    const TileKernel k = tile_kernel(c, store);
     cudaError_t e = allow_smem((const void *)k, smem);
     if (e != cudaSuccess)
         return e;

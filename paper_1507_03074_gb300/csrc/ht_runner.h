@@ -49,7 +49,7 @@ void runner_drop_graphs(Runner &R);
 // to_host: peaks and counts into the mapped pinned outputs, plus the status
 // word into h_counts[max_events]; else into d_out / d_counts.  fill_flags:
 // HT_PEAKS_ONLY (the fill keeps its tiles in shared memory, M_H is not
-// written; the edge rows must have been allocated, engine_ensure_edges),
+// written),
 // HT_FILL_NAIVE (the paper's fill: clear, one global atomic per vote) or 0.
 cudaError_t runner_enqueue(Runner &R, uint32_t n_events, uint32_t n_hits, bool host_in, bool to_host,
                            cudaStream_t st, uint32_t fill_flags = 0);

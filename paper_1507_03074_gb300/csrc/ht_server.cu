@@ -268,13 +268,6 @@ Lane *make_lane(ht_server *s, const Key &k, bool *never)
             return nullptr;
         }
     }
-    if ((c.flags & HT_PEAKS_ONLY) && hte::engine_ensure_edges(l->R.E, &why) != HT_OK) {
-        cudaGetLastError();
-        cudaEventDestroy(l->done_ev);
-        cudaStreamDestroy(l->st);
-        hte::runner_destroy(l->R);
-        return nullptr;
-    }
     l->bytes = std::max<uint64_t>(need, l->R.E.device_bytes);
     l->last_used = Clock::now();
     std::lock_guard<std::mutex> g(s->mu);

@@ -39,6 +39,14 @@ def test_tile_fill_shapes(ht, shape, rows):
                 assert total == n_ref, T
                 assert_peaks_equal(pk, pk_ref)
             assert np.array_equal(ctx.matrix(), M_ref)
+            # the same passes without the writing: M_H stays what it was
+            for _ in range(2):
+                ctx.fill(x[:n // 2], y[:n // 2], z[:n // 2], peaks_only=True)
+                ctx.fill(x, y, z, peaks_only=True)
+                pk, total = ctx.find_maxima(capacity=1 << 18)
+                assert total == n_ref, T
+                assert_peaks_equal(pk, pk_ref)
+            assert np.array_equal(ctx.matrix(), M_ref)
 
 
 @pytest.mark.parametrize("n_b", [64, 61, 30])
