@@ -529,8 +529,15 @@ ht_status engine_create(Engine &E, const ht_binning *b, const ht_ranges *r, uint
     const size_t units = (size_t)max_events * g.n_slices;
     const uint64_t list_cap = std::min<uint64_t>((uint64_t)hits_cap * E.max_admit, 0xffffffffull);
     E.list_cap = (uint32_t)list_cap;
+    auto alloc_matrices = [&] {
+        const size_t bytes = (size_t)E.n_cells * 4 * max_events + 256;
+        acc += bytes;
+        const cudaError_t em = matrix_alloc(E.M, bytes, E.device, E.tma_ok);
+        E.d_M = E.M.p;
+        return em;
+    };
     if ((e = dalloc(&E.d_edges, (E.et.size() + E.ep.size() + E.bth.size()) * 4, &acc)) != cudaSuccess ||
-        (e = dalloc(&E.d_M, (size_t)E.n_cells * 4 * max_events + 256, &acc)) != cudaSuccess ||
+        (e = alloc_matrices()) != cudaSuccess ||
         (e = dalloc(&E.d_hits4, hits_cap * 16, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_codes, hits_cap * 4, &acc)) != cudaSuccess ||
         (e = dalloc(&E.d_slice, (3 * units + 1) * 4, &acc)) != cudaSuccess ||
@@ -607,7 +614,7 @@ void engine_destroy(Engine &E)
         cudaEventDestroy(ev);
     E.prof.pool.clear();
     cudaFree(E.d_edges);
-    cudaFree(E.d_M);
+    matrix_free(E.M);
     cudaFree(E.d_hits4);
     cudaFree(E.d_codes);
     cudaFree(E.d_slice);

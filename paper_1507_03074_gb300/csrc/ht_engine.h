@@ -46,6 +46,17 @@ struct Prof {
     uint64_t n[K_NKINDS] = {};
 };
 
+// Memory of the vote matrices (ht_matrix_mem.cu): from kCompressMin bytes on
+// compressible where asked for and the device has it, else cudaMalloc's.
+// (Below that the matrices stay in L2.)
+struct MatrixMem {
+    uint32_t *p = nullptr;
+    size_t mapped = 0;           // bytes mapped by the driver calls (0: from cudaMalloc)
+};
+constexpr size_t kCompressMin = (size_t)32 << 20;
+cudaError_t matrix_alloc(MatrixMem &m, size_t bytes, int device, bool compressible);
+void matrix_free(MatrixMem &m);   // waits for the device, as cudaFree does
+
 struct Engine {
     ht_binning b{};
     ht_ranges r{};
@@ -103,7 +114,8 @@ struct Engine {
     bool last_accumulate = false;
 
     float *d_edges = nullptr;
-    uint32_t *d_M = nullptr;
+    MatrixMem M;
+    uint32_t *d_M = nullptr;      // M.p
     float4 *d_hits4 = nullptr;
     uint32_t *d_codes = nullptr;
     uint32_t *d_slice = nullptr;  // unit counts | scatter cursors | offsets (3 * units + 1)

@@ -1,0 +1,45 @@
+"""The vote matrices' memory on both sides of the size from which it is
+compressible: the contents are the oracle's through fills, copies out and in,
+the paper's fill and accumulation, and destroying a context gives its memory
+back."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.test_gpu_parity import ht, _ob, _orr, assert_peaks_equal, random_hits  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_a", [2047, 2048, 4096], ids=["below_32MiB", "32MiB", "64MiB"])
+def test_matrix_memory_holds_the_counts(ht, n_a):
+    b, r, T = ht.Binning(1, 2, n_a, 2048), ht.Ranges(), 3
+    x, y, z = random_hits(600, n_a)
+    M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+    pk_ref, n_ref = oracle.find_maxima(_ob(b), _orr(r), M_ref, T)
+    with ht.Context(b, r, threshold=T, max_hits=1200) as ctx:
+        for fills in (((0, 600, {}),), ((0, 600, dict(naive=True)),), ((0, 200, {}), (200, 600, dict(accumulate=True)))):
+            for i, j, kw in fills:
+                ctx.fill(x[i:j], y[i:j], z[i:j], **kw)
+            pk, n = ctx.find_maxima(capacity=1 << 16)
+            assert n == n_ref
+            assert_peaks_equal(pk, pk_ref)
+            assert np.array_equal(ctx.matrix(), M_ref)
+        noise = np.random.default_rng(1).integers(0, 1 << 32, M_ref.shape, dtype=np.uint32)
+        ctx.set_matrix(noise)
+        assert np.array_equal(ctx.matrix(), noise)
+
+
+def test_matrix_memory_is_given_back(ht):
+    import torch
+    b, r = ht.Binning(4, 16, 512, 1024), ht.Ranges()   # 128 MiB
+    ctx = ht.Context(b, r, threshold=3, max_hits=16)
+    ctx.close()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for _ in range(5):
+        ctxs = [ht.Context(b, r, threshold=3, max_hits=16) for _ in range(3)]
+        assert torch.cuda.mem_get_info()[0] <= free - 3 * b.n_cells * 4
+        for c in ctxs:
+            c.close()
+    assert torch.cuda.mem_get_info()[0] >= free - (8 << 20)
