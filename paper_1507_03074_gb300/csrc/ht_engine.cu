@@ -18,7 +18,7 @@ static const uint32_t kFusedPeakBuf = 512;     // K of a fused-fill CTA (at leas
 
 const char *const kKernelNames[K_NKINDS] = {"k_bin", "k_scatter", "k_fill_priv", "k_fill_scan", "k_fill_ws",
                                              "k_fill_peaks", "k_peaks", "k_clear", "k_fill_naive", "k_scan",
-                                             "k_order", "k_peaks4d", "k_fill_tma", "k_bin_cluster"};
+                                             "k_order", "k_peaks4d", "k_fill_tma", "k_bin_cluster", "k_fill_add"};
 
 // ---------------------------------------------------------------------------
 // Profiling
@@ -666,12 +666,20 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
 }
 
 // engine_vote's fill for these flags: the tile fill (TILES_MH: writing M_H,
-// TILES_PEAKS: for the peaks alone) or another one.
-enum VoteKind { OTHER_FILL, TILES_MH, TILES_PEAKS };
+// TILES_PEAKS: for the peaks alone), reductions into M_H (ADD_VOTES), or
+// another one.
+enum VoteKind { OTHER_FILL, TILES_MH, TILES_PEAKS, ADD_VOTES };
 static VoteKind vote_kind(const Engine &E, uint32_t flags)
 {
-    if ((flags & (HT_FILL_NAIVE | HT_ACCUMULATE)) || !E.fill_priv_ok)
+    if ((flags & HT_FILL_NAIVE) || !E.fill_priv_ok)
         return OTHER_FILL;
+    if (flags & HT_ACCUMULATE) {
+        // By the most votes that the hits can cast, per cell (us, reductions /
+        // k_fill_priv): 4x16x1024^2 0.02: 14.5 / 88, 0.15: 47 / 106, 0.31: 86 / 119,
+        // 0.61: 161 / 141; 4x16x256^2 0.08: 12.4 / 16.0, 0.31: 22.0 / 18.5;
+        // 8x32x2048^2 0.02: 239 / 1465, 0.15: 1524 / 1779.  The line is at 1 / 6.
+        return (uint64_t)E.binned * E.max_admit * E.geom.na <= E.n_cells / 6 ? ADD_VOTES : OTHER_FILL;
+    }
     if ((flags & HT_PEAKS_ONLY) && E.po_ok)
         return TILES_PEAKS;
     return E.use_tma && !E.use_ws ? TILES_MH : OTHER_FILL;
@@ -682,6 +690,7 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
                         uint32_t n_total, uint32_t flags, cudaStream_t st)
 {
     E.fused_valid = false;
+    E.binned = n_total;
     // one binning launch ahead of a tile fill that has the SMs to itself
     const VoteKind kind = vote_kind(E, flags);
     const bool capped = kind == TILES_PEAKS ? E.po_capped : E.tma_capped;
@@ -765,6 +774,12 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     f.accumulate = accumulate ? 1u : 0u;
     const uint64_t items = (uint64_t)n_events * E.geom.n_slices * f.strips;
     const VoteKind kind = vote_kind(E, flags);
+    if (kind == ADD_VOTES) {
+        ProfScope ps(E, K_FILL_ADD, st);
+        e = htk::launch_fill_add(E.geom, w, (uint32_t)E.num_sms, st);
+        ++E.launches;
+        return e;
+    }
     if (kind != OTHER_FILL) {
         const bool store = kind == TILES_MH;
         const htk::TileCfg &c = store ? E.tile : E.po_tile;

@@ -33,7 +33,7 @@ struct Tuning {
 // stream around every launch (enabled by ht_profile).
 enum KernelKind {
     K_BIN, K_SCATTER, K_FILL_PRIV, K_FILL_SCAN, K_FILL_WS, K_FILL_PEAKS, K_PEAKS, K_CLEAR, K_FILL_NAIVE, K_SCAN,
-    K_ORDER, K_PEAKS4D, K_FILL_TMA, K_BIN_CLUSTER, K_NKINDS
+    K_ORDER, K_PEAKS4D, K_FILL_TMA, K_BIN_CLUSTER, K_FILL_ADD, K_NKINDS
 };
 extern const char *const kKernelNames[K_NKINDS];
 
@@ -112,6 +112,7 @@ struct Engine {
     const uint32_t *last_hit_off = nullptr;   // what the last fill binned
     uint32_t last_n_hits0 = 0, last_n_events = 0;
     bool last_accumulate = false;
+    uint32_t binned = 0;         // hits the last binning was given
 
     float *d_edges = nullptr;
     MatrixMem M;

@@ -134,6 +134,9 @@ cudaError_t launch_order_passes(const Geom &g, const Work &w, const ScanArgs &a,
 // After k_fill_scan, k_fill_bulk or k_fill_ws (same grid): test its candidate
 // entries, keep the peaks.
 cudaError_t launch_peaks(const Geom &g, const Work &w, const ScanArgs &a, uint32_t grid, cudaStream_t st);
+// Accumulating fills of few hits: M_H += their votes, one reduction each (kAddRows A rows of a slice per warp).
+constexpr uint32_t kAddRows = 32;
+cudaError_t launch_fill_add(const Geom &g, const Work &w, uint32_t num_sms, cudaStream_t st);
 cudaError_t launch_clear(uint32_t *M, uint64_t words, uint32_t grid, cudaStream_t st);
 cudaError_t launch_fill_naive(const Geom &g, const Work &w, uint32_t num_sms, cudaStream_t st);
 size_t scan_smem_bytes(const ScanArgs &a);

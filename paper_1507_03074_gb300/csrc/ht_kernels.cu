@@ -13,6 +13,7 @@
 //                 M_H's rows, which leaves as one bulk copy; a vote taking a
 //                 cell to T lists it, and the warp tests the listed cells in
 //                 its tile.  k_order_passes puts the peaks in order.
+//   k_fill_add    Accumulating fills of few hits: a reduction per vote.
 //   k_fill_priv   Step 1 (Sec. 2), privatised.  Work item = (event, slice,
 //                 strip of W A-rows); each CTA takes a contiguous range of
 //                 items.  It selects the event's hits admitted to the slice
@@ -2361,6 +2362,42 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) k_fill_tma(const __grid_co
 }
 
 // ---------------------------------------------------------------------------
+// k_fill_add: accumulating fills of few hits.  A warp takes kAddRows A rows of
+// one (event, slice) unit and adds its votes to M_H one by one (reductions in
+// L2, results unused): a fill that touches few cells does not read and write
+// the others, as k_fill_priv does.  Bound by the L2's reductions and by the
+// sectors of M_H that they bring in.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_fill_add(Geom g, Work w, uint32_t strips)
+{
+    grid_dep_wait();   // the unit lists
+    const uint32_t lane = threadIdx.x & 31u, nb = g.nb;
+    const uint64_t slice_cells = (uint64_t)g.na * nb, items = (uint64_t)w.n_events * g.n_slices * strips;
+    const uint64_t stride = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    for (uint64_t it = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < items; it += stride) {
+        const uint32_t u = (uint32_t)(it / strips), i0 = (uint32_t)(it - (uint64_t)u * strips) * kAddRows;
+        const uint32_t i1 = min(i0 + kAddRows, g.na), l0 = w.slice_off[u], nc = w.slice_off[u + 1] - l0;
+        uint32_t *Ms = w.M + (uint64_t)u * slice_cells;   // unit u = e * n_slices + s, n_cells = n_slices * slice_cells
+        for (uint32_t h = lane; h < nc; h += 32u) {
+            const float2 l = __ldg(w.lines + l0 + h);
+            const float4 *rec = w.list + l0 + h;
+            for (uint32_t i = i0; i < i1; i += 4u) {
+                float x[4];
+                uint32_t j1[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    x[q] = __int2float_rn((int)(i + q) - g.mid);
+                line_bins<4>(g, l, x, i, rec, true, j1);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (j1[q] - 1u < nb && i + q < i1)
+                        atomicAdd(Ms + (size_t)(i + q) * nb + (j1[q] - 1u), 1u);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // k_order_passes: the peaks of k_fill_tma's passes into one list, ascending.
 // A CTA takes a segment of kOrderPasses passes: its first rank is the sum of
 // the segments before it, and one thread per peak finds its pass by a search
@@ -2652,6 +2689,13 @@ cudaError_t launch_fill_priv(const Geom &g, const Work &w, const FillCfg &c, uin
     if (e != cudaSuccess)
         return e;
     return launch_pdl(k_fill_priv, grid, c.threads, smem, st, g, w, c);
+}
+
+cudaError_t launch_fill_add(const Geom &g, const Work &w, uint32_t num_sms, cudaStream_t st)
+{
+    const uint32_t strips = (g.na + kAddRows - 1) / kAddRows;
+    const uint64_t items = (uint64_t)w.n_events * g.n_slices * strips;
+    return launch_pdl(k_fill_add, (uint32_t)std::min<uint64_t>((items + 7) / 8, num_sms * 8u), 256, 0, st, g, w, strips);
 }
 
 cudaError_t launch_clear(uint32_t *M, uint64_t words, uint32_t grid, cudaStream_t st)
