@@ -701,7 +701,7 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
     cudaError_t e;
     if (cluster) {
         // few hits: binning and unit lists in one cluster launch, one CTA per
-        // kBinClusterThreads hits (two hits a thread past kBinClusterMax CTAs)
+        // kBinClusterThreads hits (up to kBinClusterHPT hits a thread past kBinClusterMax CTAs)
         const htk::Work w = make_work(E, x, y, z, d_hit_off, n_hits0, n_events);
         const uint32_t cs = std::min<uint32_t>(
             htk::kBinClusterMax, std::max<uint32_t>(1u, (n_total + htk::kBinClusterThreads - 1) / htk::kBinClusterThreads));

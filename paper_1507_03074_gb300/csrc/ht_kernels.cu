@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(256) k_scatter(Geom g, Work w)
 // most kBinClusterHPT) hits in registers between counting and listing.
 // Dynamic shared memory: U counts, U + 1 totals / offsets, U places and
 // n_events + 1 hit offsets, where U = n_events * n_slices.
-__global__ void __launch_bounds__(1024, 1) k_bin_cluster(Geom g, Work w)
+__global__ void __launch_bounds__(kBinClusterThreads, 2) k_bin_cluster(Geom g, Work w)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
