@@ -312,17 +312,23 @@ __global__ void __launch_bounds__(kBinClusterThreads, 2) k_bin_cluster(Geom g, W
     __syncthreads();
     const uint32_t n = w.hit_off ? min(s_off[w.n_events], w.n_hits0) : w.n_hits0;
     uint32_t code[kBinClusterHPT], ev[kBinClusterHPT];
-    float4 hv[kBinClusterHPT];
+    float4 hv[kBinClusterHPT];   // x, y, z until the hit is binned
+#pragma unroll
+    for (uint32_t q = 0; q < kBinClusterHPT; ++q) {   // every hit's loads in flight
+        const uint32_t h = (q * cs + rank) * bd + tid;
+        hv[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (h < n)
+            hv[q] = make_float4(__ldg(&w.x[h]), __ldg(&w.y[h]), __ldg(&w.z[h]), 0.0f);
+    }
 #pragma unroll
     for (uint32_t q = 0; q < kBinClusterHPT; ++q) {
         const uint32_t h = (q * cs + rank) * bd + tid;
         code[q] = kDropped;
         ev[q] = 0u;
-        hv[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (h < n) {
-            const float x = __ldg(&w.x[h]), y = __ldg(&w.y[h]);
+            const float x = hv[q].x, y = hv[q].y;
             float r2;
-            code[q] = bin_code(g, et, ep, x, y, __ldg(&w.z[h]), r2);
+            code[q] = bin_code(g, et, ep, x, y, hv[q].z, r2);
             if (w.hit_off) {   // the last event whose first hit is <= h
                 uint32_t lo = 0, hi = w.n_events - 1;
                 while (lo < hi) {
@@ -339,7 +345,17 @@ __global__ void __launch_bounds__(kBinClusterThreads, 2) k_bin_cluster(Geom g, W
             for_each_slice(g, code[q], [&](uint32_t s) { atomicAdd(&s_cnt[e * g.n_slices + s], 1u); });
         }
     }
-    cl.sync();   // every CTA's counts are complete (and every CTA of the cluster runs)
+    // every CTA's counts are complete (and every CTA of the cluster runs); the
+    // hits' lines are made while the others arrive
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    float2 line[kBinClusterHPT];
+#pragma unroll
+    for (uint32_t q = 0; q < kBinClusterHPT; ++q) {
+        line[q] = make_float2(0.0f, 0.0f);
+        if (code[q] != kDropped)
+            line[q] = vote_line(g, hv[q].x, hv[q].y, hv[q].z);
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     const uint32_t *r_cnt[kBinClusterMax];
 #pragma unroll
     for (uint32_t r = 0; r < kBinClusterMax; ++r)
@@ -376,12 +392,11 @@ __global__ void __launch_bounds__(kBinClusterThreads, 2) k_bin_cluster(Geom g, W
 #pragma unroll
     for (uint32_t q = 0; q < kBinClusterHPT; ++q) {
         const uint32_t e = ev[q];
-        const float2 line = vote_line(g, hv[q].x, hv[q].y, hv[q].z);
         for_each_slice(g, code[q], [&](uint32_t s) {
             const uint32_t idx = atomicAdd(&s_pl[e * g.n_slices + s], 1u);
             if (idx < w.list_cap) {
                 w.list[idx] = hv[q];
-                w.lines[idx] = line;
+                w.lines[idx] = line[q];
             }
         });
     }
