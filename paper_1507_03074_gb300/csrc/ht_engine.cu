@@ -1095,13 +1095,4 @@ cudaError_t prof_read(Engine &E, ht_kernel_time *out, uint32_t cap, uint32_t *n)
     return cudaSuccess;
 }
 
-cudaError_t engine_set_phi_edges(Engine &E, const float *ep)
-{
-    std::copy(ep, ep + E.ep.size(), E.ep.begin());
-    // a pageable-source copy may still be in flight when cudaMemcpy returns,
-    // on the legacy stream the object's streams do not wait for
-    cudaError_t e = cudaMemcpy(E.d_edges + E.et.size(), E.ep.data(), E.ep.size() * 4, cudaMemcpyHostToDevice);
-    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
-}
-
 } // namespace hte

@@ -183,12 +183,6 @@ void engine_get_tuning(const Engine &E, ht_tuning *t);
 // Per-kernel totals into the ABI's records (waits for recorded events).
 cudaError_t prof_read(Engine &E, ht_kernel_time *out, uint32_t cap, uint32_t *n);
 
-// Replace the phi edge table (n_phi + 1 pseudo-angles, host memory) on the
-// host and on the device (synchronous copy).  A sector context takes its
-// slice of the full circle's table, so that it bins hits exactly as the
-// unsplit matrix does.
-cudaError_t engine_set_phi_edges(Engine &E, const float *ep);
-
 // Step 2 with the 4-D neighbourhood for one event: the 2-D peaks into
 // p2 (p2_cap entries, total in *p2_count), then those that also beat their
 // neighbours in the adjacent (theta, phi) slices, in order, into out

@@ -521,8 +521,8 @@ class Context:
 
 
 class Sectors:
-    """Phi sectors (ht_sectors_*): one context per sector, forked and joined
-    on the device, peaks merged into the unsplit numbering and order."""
+    """Phi sectors (ht_sectors_*): parts of one matrix, peaks merged into the
+    unsplit numbering and order."""
 
     def __init__(self, binning: Binning, ranges: Ranges = Ranges(), threshold: int = 10, n_sectors: int = 4,
                  max_hits: int = 65536):
