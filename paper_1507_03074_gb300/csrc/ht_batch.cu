@@ -97,7 +97,7 @@ static cudaError_t enqueue_compute(Runner &R, uint32_t n_events, bool to_host, u
     if (e != cudaSuccess)
         return e;
     return engine_scan(E, n_events, to_host ? R.h_out_dev : R.d_out, R.capacity, to_host ? R.h_counts_dev : R.d_counts,
-                       st, true);
+                       st, true, to_host ? R.h_counts_dev + E.max_events : nullptr);
 }
 
 // Replay the graph for (n_events, to_host), or run directly and capture one
@@ -162,8 +162,6 @@ cudaError_t runner_enqueue(Runner &R, uint32_t n_events, uint32_t n_hits, bool h
     E.last_n_hits0 = (uint32_t)mh;
     E.last_n_events = n_events;
     E.last_accumulate = false;
-    if (to_host)
-        return cudaMemcpyAsync(R.h_counts + E.max_events, engine_status(E), 4, cudaMemcpyDeviceToHost, st);
     return cudaSuccess;
 }
 

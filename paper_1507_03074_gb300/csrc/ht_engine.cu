@@ -842,7 +842,7 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
 }
 
 cudaError_t engine_scan(Engine &E, uint32_t n_events, htk::Peak *out, uint32_t capacity,
-                        uint32_t *counts, cudaStream_t st, bool compact)
+                        uint32_t *counts, cudaStream_t st, bool compact, uint32_t *status_out)
 {
     htk::Work w = make_work(E, nullptr, nullptr, nullptr, nullptr, 0, n_events);
     htk::ScanArgs a = E.scan;
@@ -854,6 +854,7 @@ cudaError_t engine_scan(Engine &E, uint32_t n_events, htk::Peak *out, uint32_t c
     o.ticket = E.d_ctr + htk::CTR_OTICKET;
     o.g_count = E.d_ctr + htk::CTR_ENTRIES;
     o.compact = compact ? 1u : 0u;
+    o.status_out = status_out;
     cudaError_t e;
     if (E.fused_valid && E.fused_events == n_events && E.fused_passes) {
         // the tile fill left its peaks pass by pass

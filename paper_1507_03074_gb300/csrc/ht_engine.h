@@ -165,9 +165,10 @@ ht_status engine_autotune(Engine &E, uint32_t reps, cudaStream_t st, double *bes
 
 // Step 2: peaks of every event into out[e * capacity ...], totals into counts[e].
 // compact: one list ordered by (event, linear index) in out[0 .. capacity)
-// instead of capacity entries per event.
+// instead of capacity entries per event.  status_out: mapped host memory that
+// receives the status word with the peaks, or nullptr.
 cudaError_t engine_scan(Engine &E, uint32_t n_events, htk::Peak *out, uint32_t capacity,
-                        uint32_t *counts, cudaStream_t st, bool compact = false);
+                        uint32_t *counts, cudaStream_t st, bool compact = false, uint32_t *status_out = nullptr);
 
 // Grow the peak-entry scratch to the bound that holds for any matrix (no two
 // peaks are neighbours): needed once M_H is written by something else than

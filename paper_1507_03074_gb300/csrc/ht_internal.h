@@ -96,6 +96,7 @@ struct OrderArgs {
     uint32_t *ticket;     // last-CTA detection (reset by k_order)
     uint32_t *g_count;    // entries used (reset by the last CTA)
     uint32_t compact;     // 1: one list out[rank] over all events, else out[e][capacity]
+    uint32_t *status_out; // receives the status word (mapped host memory), or nullptr
 };
 
 cudaError_t launch_bin(const Geom &g, const Work &w, uint32_t grid, cudaStream_t st);

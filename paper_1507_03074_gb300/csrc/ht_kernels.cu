@@ -1823,6 +1823,8 @@ __global__ void __launch_bounds__(256) k_order(Geom g, Work w, ScanArgs a, Order
     uint32_t *red = ev_base + w.n_events + 1; // 40
     __shared__ uint32_t s_tot[32], s_last;
     const uint32_t tid = threadIdx.x, bd = blockDim.x, warp = tid >> 5, lane = tid & 31u, nw = bd >> 5;
+    if (blockIdx.x == 0 && tid == 0 && o.status_out)
+        *o.status_out = *w.status;   // this kernel raises nothing itself
     // one list per warp: lists c0 .. c0 + nw - 1
     const uint32_t c0 = blockIdx.x * nw, c = c0 + warp;
     const bool valid = c < a.grid;
@@ -2425,9 +2427,12 @@ __global__ void __launch_bounds__(kOrderPasses) k_order_passes(Geom g, Work w, S
     __shared__ uint32_t s_off[kOrderPasses], s_base[kOrderPasses], s_wsum[40];
     const uint32_t tid = threadIdx.x, seg = blockIdx.x, warp = tid >> 5, lane = tid & 31u;
     const uint32_t mine = w.seg_peaks[seg];
-    if (seg == 0)
+    if (seg == 0) {
+        if (tid == 0 && o.status_out)
+            *o.status_out = *w.status;
         for (uint32_t e = tid; e < w.n_events; e += kOrderPasses)
             o.counts[e] = o.ev_count[e];
+    }
     if (mine == 0)
         return;
     const uint64_t pass = (uint64_t)seg * kOrderPasses + tid;

@@ -69,3 +69,23 @@ def test_tile_fill_batch(ht, n_b):
                 assert np.array_equal(B.matrix(e), M_ref)
                 at += n_ref
             assert len(pk) == at
+
+
+@pytest.mark.parametrize("S", [4, 16])
+def test_sectors_count_edge_hits_once(ht, S):
+    """Hits on the axes and diagonals, which are sector edges: the sectors'
+    matrices are their phi bins of the unsplit one, the peaks the unsplit
+    peaks."""
+    from tests.test_gpu_parity import degenerate_hits
+    x, y, z = degenerate_hits()
+    b, r, T = ht.Binning(4, 16, 128, 100), ht.Ranges(), 3
+    M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+    pk_ref, n_ref = oracle.find_maxima(_ob(b), _orr(r), M_ref, T)
+    with ht.Sectors(b, r, threshold=T, n_sectors=S, max_hits=len(x)) as sec:
+        sec.fill(x, y, z)
+        pk, n = sec.find_maxima(capacity=1 << 18)
+        assert n == n_ref
+        assert_peaks_equal(pk, pk_ref)
+        m = b.n_phi // S
+        for k in range(S):
+            assert np.array_equal(sec.matrix(k), M_ref[:, k * m:(k + 1) * m])
