@@ -59,10 +59,10 @@ struct Work {
     float2 *lines;              // [list_cap + 2] the records' vote lines (vote_line), unit by unit as list
     uint32_t list_cap;
     // k_fill_tma's peaks: {first entry, count} of every pass, and their number in
-    // every kOrderPasses passes (the binning clears the n_seg counts)
+    // every 1 << seg_shift passes (the binning clears the n_seg counts)
     uint2 *pass_peaks;
     uint32_t *seg_peaks;
-    uint32_t n_seg;
+    uint32_t n_seg, seg_shift;
 };
 
 constexpr uint32_t kDropped = 0xffffffffu;

@@ -18,7 +18,8 @@ static const uint32_t kFusedPeakBuf = 512;     // K of a fused-fill CTA (at leas
 
 const char *const kKernelNames[K_NKINDS] = {"k_bin", "k_scatter", "k_fill_priv", "k_fill_scan", "k_fill_ws",
                                              "k_fill_peaks", "k_peaks", "k_clear", "k_fill_naive", "k_scan",
-                                             "k_order", "k_peaks4d", "k_fill_tma", "k_bin_cluster", "k_fill_add"};
+                                             "k_order", "k_peaks4d", "k_fill_tma", "k_bin_cluster", "k_fill_add",
+                                             "k_edges"};
 
 // ---------------------------------------------------------------------------
 // Profiling
@@ -371,6 +372,11 @@ ht_status engine_configure(Engine &E, std::string *why)
     const uint32_t ws_grid = E.ws_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.ws_grid, items_max)) : 0;
     E.max_passes = std::max(E.tma_ok ? htk::tile_passes(g, E.tile, E.max_events) : 0,
                             E.po_ok ? htk::tile_passes(g, E.po_tile, E.max_events) : 0);
+    // segments of the passes' peaks (a CTA of k_edges and k_order_passes each):
+    // enough to fill the GPU, few enough for each CTA to add up those before it
+    E.seg_shift = 5;
+    while ((2u << E.seg_shift) <= htk::kOrderPasses && (E.max_passes >> E.seg_shift) > (uint64_t)E.num_sms)
+        ++E.seg_shift;
     // the fused fill's candidate lists: one per CTA plus one per handed-out item
     const uint32_t fused_lists = fused_grid + (uint32_t)htk::dyn_items(items_max, fused_grid);
     const uint32_t grid_cap = std::max(std::max(scan_grid, fused_lists), ws_grid);
@@ -395,7 +401,7 @@ ht_status engine_configure(Engine &E, std::string *why)
     s.seq_max = seq;
     const size_t desc_b = (size_t)grid_cap * seq * 8;
     const size_t cta_b = (size_t)grid_cap * 2 * 4;
-    const size_t pass_b = (size_t)E.max_passes * 8, seg_b = (size_t)(E.max_passes / htk::kOrderPasses + 1) * 4;
+    const size_t pass_b = (size_t)E.max_passes * 8, seg_b = (size_t)((E.max_passes >> E.seg_shift) + 1) * 4;
     const size_t need = pass_b + desc_b + cta_b + seg_b;
     if (need > E.book_bytes || grid_cap != E.grid_cap) {
         if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
@@ -661,7 +667,8 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
     w.list_cap = E.list_cap;
     w.pass_peaks = E.pass_peaks;
     w.seg_peaks = E.seg_peaks;
-    w.n_seg = (uint32_t)((E.max_passes / E.max_events * n_events + htk::kOrderPasses - 1) / htk::kOrderPasses);
+    w.n_seg = (uint32_t)((E.max_passes / E.max_events * n_events) >> E.seg_shift) + 1u;
+    w.seg_shift = E.seg_shift;
     return w;
 }
 
@@ -745,7 +752,7 @@ static cudaError_t engine_clear_counts(Engine &E, cudaStream_t st)
     cudaError_t e = cudaMemsetAsync(E.d_ctr + htk::CTR_ENTRIES, 0,
                                     (engine_ctr_words(E) - htk::CTR_ENTRIES) * sizeof(uint32_t), st);
     if (e == cudaSuccess)
-        e = cudaMemsetAsync(E.seg_peaks, 0, (E.max_passes / htk::kOrderPasses + 1) * 4, st);
+        e = cudaMemsetAsync(E.seg_peaks, 0, ((E.max_passes >> E.seg_shift) + 1) * 4, st);
     return e;
 }
 
@@ -782,7 +789,9 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     }
     if (kind != OTHER_FILL) {
         const bool store = kind == TILES_MH;
-        const htk::TileCfg &c = store ? E.tile : E.po_tile;
+        htk::TileCfg c = store ? E.tile : E.po_tile;
+        c.edges_later = store && (double)E.binned * E.max_admit >=
+                                     (double)htk::kEdgeHits * E.geom.n_slices * n_events;
         if (!fresh) {   // voted again without a binning (the autotuner)
             if ((e = engine_clear_counts(E, st)) != cudaSuccess)
                 return e;
@@ -795,6 +804,11 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
             e = htk::launch_fill_tma(E.geom, w, c, E.scan, grid, store, st);
         }
         ++E.launches;
+        if (e == cudaSuccess && c.edges_later) {
+            ProfScope ps(E, K_EDGES, st);
+            e = htk::launch_edges(E.geom, w, c, E.scan, passes, st);
+            ++E.launches;
+        }
         if (e == cudaSuccess) {
             E.fused_valid = true;
             E.ctr_dirty = true;

@@ -33,7 +33,7 @@ struct Tuning {
 // stream around every launch (enabled by ht_profile).
 enum KernelKind {
     K_BIN, K_SCATTER, K_FILL_PRIV, K_FILL_SCAN, K_FILL_WS, K_FILL_PEAKS, K_PEAKS, K_CLEAR, K_FILL_NAIVE, K_SCAN,
-    K_ORDER, K_PEAKS4D, K_FILL_TMA, K_BIN_CLUSTER, K_FILL_ADD, K_NKINDS
+    K_ORDER, K_PEAKS4D, K_FILL_TMA, K_BIN_CLUSTER, K_FILL_ADD, K_EDGES, K_NKINDS
 };
 extern const char *const kKernelNames[K_NKINDS];
 
@@ -88,8 +88,9 @@ struct Engine {
     htk::TileCfg po_tile{};
     uint32_t po_grid = 0;
     uint64_t max_passes = 0;     // of either, over max_events events
-    uint2 *pass_peaks = nullptr; // (in d_book) its peaks per pass and per htk::kOrderPasses passes
+    uint2 *pass_peaks = nullptr; // (in d_book) its peaks per pass and per segment of 1 << seg_shift passes
     uint32_t *seg_peaks = nullptr;
+    uint32_t seg_shift = 5;
     bool use_tma = false;        // fills run the bulk-copy-tile kernel
     htk::ScanArgs scan{};
     int scan_kind = 0;            // htk::ScanKind in use

@@ -36,6 +36,7 @@ struct TileCfg {
     uint32_t run;         // neighbouring passes of a CTA's run (= warps)
     uint32_t threads;     // the tuning's fill_threads (at least 32 * warps)
     uint32_t vote_agg;    // warp-aggregated vote increments (match.any + one add)
+    uint32_t edges_later; // tiles that go to M_H: comparisons across passes are left to k_edges
 };
 constexpr uint32_t kTileWarps = 12;    // most warps of a tile-fill CTA (two such CTAs per SM: 80 registers a thread)
 constexpr uint32_t kTileCand = 127;    // cells >= T that a pass lists (more: every cell is looked at)
@@ -49,7 +50,7 @@ __host__ __device__ constexpr uint32_t tile_warp_words(uint32_t tile_words)
     return tile_words + tile_bit_words(tile_words) + tile_list_words() + 32u;
 }
 inline size_t tile_smem_bytes(const TileCfg &c) { return (size_t)c.warps * tile_warp_words(c.tile_words) * 4; }
-constexpr uint32_t kOrderPasses = 256; // passes per k_order_passes CTA
+constexpr uint32_t kOrderPasses = 256; // threads of a k_order_passes or k_edges CTA, and most passes of its segment
 __host__ __device__ inline uint64_t tile_passes(const Geom &g, const TileCfg &c, uint32_t n_events)
 {
     return (uint64_t)n_events * g.n_slices * c.strips;
@@ -137,6 +138,15 @@ cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, cons
 cudaError_t fill_tma_occupancy(const TileCfg &c, bool store, int *blocks_per_sm);
 cudaError_t launch_order_passes(const Geom &g, const Work &w, const ScanArgs &a, const OrderArgs &o, uint64_t passes,
                                 cudaStream_t st);
+// After a tile fill with edges_later: drop its candidates that a row of another pass outdoes.
+cudaError_t launch_edges(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a, uint64_t passes,
+                         cudaStream_t st);
+// k_edges from this many admissions per (event, slice) on, on average.  Voting
+// the rows beyond costs more the more hits a slice has, k_edges one more launch:
+// paper matrix, 78 hits per slice, without and with: 33.8 and 34.0 us in flight,
+// 48.7 and 51.2 us alone; 156: 36.7 and 35.9, 60.1 and 56.7; 250: 49.3 and 42.6,
+// 85.2 and 69.7; windows with 169 (at most): 33.9 and 34.1, 49.2 and 53.0.
+constexpr uint32_t kEdgeHits = 192;
 // After k_fill_scan, k_fill_bulk or k_fill_ws (same grid): test its candidate
 // entries, keep the peaks.
 cudaError_t launch_peaks(const Geom &g, const Work &w, const ScanArgs &a, uint32_t grid, cudaStream_t st);

@@ -13,6 +13,7 @@
 //                 M_H's rows, which leaves as one bulk copy; a vote taking a
 //                 cell to T lists it, and the warp tests the listed cells in
 //                 its tile.  k_order_passes puts the peaks in order.
+//   k_edges       Crowded tile fills: peaks against the rows of other passes.
 //   k_fill_add    Accumulating fills of few hits: a reduction per vote.
 //   k_fill_priv   Step 1 (Sec. 2), privatised.  Work item = (event, slice,
 //                 strip of W A-rows); each CTA takes a contiguous range of
@@ -1926,8 +1927,7 @@ __global__ void __launch_bounds__(256) k_order(Geom g, Work w, ScanArgs a, Order
 //
 // Order of the passes: a CTA's warps take a pass each of its runs (run i of
 // CTA c is run i * grid + c: c.run = warps neighbouring passes), and the last
-// passes
-// go to whichever warp of the grid comes first, so that the whole grid writes
+// passes go to whichever warp of the grid comes first, so that the whole grid writes
 // one neighbourhood of M_H at any time and the hits' uneven spread over the
 // slices averages out.
 //
@@ -1935,7 +1935,7 @@ __global__ void __launch_bounds__(256) k_order(Geom g, Work w, ScanArgs a, Order
 // T - 1 to T lists the cell, and the listed cells are compared with their
 // neighbours in the tile.  For a cell on the first or last row of the pass
 // the votes of the row beyond are counted from the unit's lines (nothing waits
-// for the warp that owns it).  Each pass leaves {first entry, count} in
+// for the warp that owns it), or k_edges compares them later.  Each pass leaves {first entry, count} in
 // pass_peaks, in pass order, for k_order_passes.
 //
 // Bound: the M_H write where votes are few (paper event, one launch: 46.7 us
@@ -2093,15 +2093,17 @@ __device__ __forceinline__ void vote_row(const Geom &g, uint32_t *row, const Til
 
 // The peaks of pass number `pass` (the warp's own tile and list; bits: one bit
 // per cell of the tile, zero between calls).  reading: a bulk copy may still
-// read the tile.  Every lane calls it.
+// read the tile.  edges_later: the rows beyond the pass are left to k_edges.
+// Every lane calls it.
 __device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const ScanArgs &a, const TilePass &P,
                                          uint32_t pass, uint32_t unit, uint32_t *tile, const PassList &L,
-                                         uint32_t *bits, bool reading)
+                                         uint32_t *bits, bool reading, bool edges_later)
 {
     const uint32_t lane = threadIdx.x & 31u, nb = g.nb, n_c = L.n, full = 0xffffffffu, pr = P.pr;
     const uint32_t e = unit / g.n_slices, s = unit - e * g.n_slices;
     const uint32_t lin0 = (s * g.na + P.iA) * nb, last = (pr - 1u) * nb;
-    const bool above = P.iA > 0, below = P.iA + pr < g.na;   // rows of the slice beyond the pass
+    // the pass has a row of the slice before / behind it, which this kernel compares with
+    const bool above = !edges_later && P.iA > 0, below = !edges_later && P.iA + pr < g.na;
     // the test against the neighbours inside the tile
     auto inner = [&](uint32_t key, uint32_t v) {
         const uint32_t r = key / nb, j = key - r * nb;
@@ -2114,7 +2116,7 @@ __device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const 
         if (lane == 0) {
             if (n) {
                 base = atomicAdd(a.g_count, n);
-                atomicAdd(&w.seg_peaks[pass / kOrderPasses], n);
+                atomicAdd(&w.seg_peaks[pass >> w.seg_shift], n);
                 atomicAdd(&a.ev_count[e], n);
                 if (base + n > a.entries_cap || base + n < base)
                     atomicOr(w.status, (uint32_t)ST_SCRATCH_OVERFLOW);
@@ -2347,7 +2349,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) k_fill_tma(const __grid_co
         const uint2 next2_off = offsets(next2);
         // ---- its peaks
         if (L.n)
-            pass_search(g, w, a, P, pass, unit, tile, L, bits, STORE);
+            pass_search(g, w, a, P, pass, unit, tile, L, bits, STORE, STORE && c.edges_later);
         else if (lane == 0)
             w.pass_peaks[pass] = make_uint2(0u, 0u);
         // ---- the tile is cleared once the copy has read it
@@ -2414,9 +2416,123 @@ __global__ void __launch_bounds__(256) k_fill_add(Geom g, Work w, uint32_t strip
     }
 }
 
+// The peaks (or candidates) of a segment of 1 << seg_shift passes, as k_edges and
+// k_order_passes read them, one thread per pass: each pass's first rank in the
+// segment and first entry.  Returns how many there are.
+constexpr uint32_t kNoPeak = 0xffffffffu;
+struct SegmentPeaks {
+    uint32_t off[kOrderPasses], base[kOrderPasses], wsum[kOrderPasses / 32];
+};
+
+__device__ __forceinline__ uint32_t load_segment(SegmentPeaks &sp, const Work &w, uint32_t seg, uint64_t passes)
+{
+    const uint32_t tid = threadIdx.x, warp = tid >> 5;
+    const uint64_t pass = ((uint64_t)seg << w.seg_shift) + tid;
+    const uint2 d = pass < passes && tid >> w.seg_shift == 0u ? w.pass_peaks[pass] : make_uint2(0u, 0u);
+    const uint32_t incl = warp_incl_scan(d.y);
+    if ((tid & 31u) == 31u)
+        sp.wsum[warp] = incl;
+    __syncthreads();
+    uint32_t off = incl - d.y, n = 0;
+    for (uint32_t q = 0; q < kOrderPasses / 32; ++q) {
+        off += q < warp ? sp.wsum[q] : 0u;
+        n += sp.wsum[q];
+    }
+    sp.off[tid] = off;
+    sp.base[tid] = d.x;
+    __syncthreads();
+    return n;
+}
+
+// The pass (of the segment) that holds the segment's peak k: the last one that
+// starts at or before k.
+__device__ __forceinline__ uint32_t segment_pass(const SegmentPeaks &sp, uint32_t k)
+{
+    uint32_t lo = 0, hi = kOrderPasses - 1;
+    while (lo < hi) {
+        const uint32_t m = (lo + hi + 1) >> 1;
+        if (sp.off[m] <= k)
+            lo = m;
+        else
+            hi = m - 1;
+    }
+    return lo;
+}
+
+// ---------------------------------------------------------------------------
+// k_edges: the comparisons that the tile fill left (TileCfg::edges_later).  An
+// entry on the first or last row of its pass is compared with the row beyond in
+// M_H; .w becomes the rank in the segment plus 1, or kNoPeak (0, as the fill
+// leaves it: the position is the rank), and the segment's and events' counts
+// become those of the peaks.  Voting the row beyond anew, as passes of few hits
+// do, costs a pass its hits over again for both of its edges; here a comparison
+// is three words out of L2.  One event in flight and alone, without and with
+// this: admission windows 87.0 -> 63.9 and 143.7 -> 96.5 us, 24000 hits in the
+// paper's matrix 79.5 -> 58.9 and 138 -> 98.6 us.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kOrderPasses) k_edges(Geom g, Work w, TileCfg c, ScanArgs a, uint64_t passes)
+{
+    grid_dep_wait();
+    __shared__ SegmentPeaks sp;
+    __shared__ uint32_t s_kept[kOrderPasses / 32];
+    const uint32_t tid = threadIdx.x, seg = blockIdx.x, warp = tid >> 5, lane = tid & 31u, nb = g.nb, full = 0xffffffffu;
+    if (w.seg_peaks[seg] == 0u)
+        return;
+    const uint32_t n = load_segment(sp, w, seg, passes);
+    uint32_t kept = 0;
+    for (uint32_t k0 = 0; k0 < n; k0 += kOrderPasses) {
+        const uint32_t k = k0 + tid;
+        bool has = k < n, keep = has;
+        uint32_t at = 0, e = 0;
+        if (has) {
+            const uint32_t q = segment_pass(sp, k);
+            at = sp.base[q] + (k - sp.off[q]);
+            has = keep = at < a.entries_cap;
+            if (has) {
+                const uint4 en = a.entries[at];
+                e = en.y;
+                const uint64_t pass = ((uint64_t)seg << w.seg_shift) + q;
+                const uint32_t unit = (uint32_t)(pass / c.strips), strip = (uint32_t)(pass - (uint64_t)unit * c.strips);
+                const uint32_t first = strip * c.W, last = min(first + c.W, g.na) - 1u;
+                const uint32_t row = en.x / nb, j = en.x - row * nb, i = row % g.na;
+                // the most votes of the three cells of row i next to column j
+                auto beyond = [&](uint32_t i) {
+                    const uint32_t *r = w.M + ((uint64_t)unit * g.na + i) * nb + j;
+                    return max(__ldcg(r), max(j ? __ldcg(r - 1) : 0u, j + 1u < nb ? __ldcg(r + 1) : 0u));
+                };
+                if (i == first && i > 0u)
+                    keep = en.z > beyond(i - 1u);
+                if (keep && i == last && i + 1u < g.na)
+                    keep = en.z >= beyond(i + 1u);
+            }
+        }
+        const uint32_t m = __ballot_sync(full, keep);
+        if (lane == 0)
+            s_kept[warp] = (uint32_t)__popc(m);
+        __syncthreads();
+        uint32_t rank = kept + (uint32_t)__popc(m & ((1u << lane) - 1u));
+        for (uint32_t q = 0; q < kOrderPasses / 32; ++q) {
+            rank += q < warp ? s_kept[q] : 0u;
+            kept += s_kept[q];
+        }
+        if (has)
+            a.entries[at].w = keep ? rank + 1u : kNoPeak;
+        for (uint32_t out = __ballot_sync(full, has && !keep); out;) {   // by event
+            const uint32_t src = (uint32_t)(__ffs(out) - 1), es = __shfl_sync(full, e, src);
+            const uint32_t same = __ballot_sync(full, e == es) & out;
+            if (lane == src)
+                atomicSub(&a.ev_count[es], (uint32_t)__popc(same));
+            out &= ~same;
+        }
+        __syncthreads();
+    }
+    if (tid == 0)
+        w.seg_peaks[seg] = kept;
+}
+
 // ---------------------------------------------------------------------------
 // k_order_passes: the peaks of k_fill_tma's passes into one list, ascending.
-// A CTA takes a segment of kOrderPasses passes: its first rank is the sum of
+// A CTA takes a segment of 1 << seg_shift passes: its first rank is the sum of
 // the segments before it, and one thread per peak finds its pass by a search
 // over the segment's prefix sums.  (One event, or one list over all events.)
 // ---------------------------------------------------------------------------
@@ -2424,8 +2540,9 @@ __global__ void __launch_bounds__(kOrderPasses) k_order_passes(Geom g, Work w, S
                                                                uint64_t passes)
 {
     grid_dep_wait();
-    __shared__ uint32_t s_off[kOrderPasses], s_base[kOrderPasses], s_wsum[40];
-    const uint32_t tid = threadIdx.x, seg = blockIdx.x, warp = tid >> 5, lane = tid & 31u;
+    __shared__ SegmentPeaks sp;
+    __shared__ uint32_t s_before[kOrderPasses / 32];
+    const uint32_t tid = threadIdx.x, seg = blockIdx.x;
     const uint32_t mine = w.seg_peaks[seg];
     if (seg == 0) {
         if (tid == 0 && o.status_out)
@@ -2435,38 +2552,24 @@ __global__ void __launch_bounds__(kOrderPasses) k_order_passes(Geom g, Work w, S
     }
     if (mine == 0)
         return;
-    const uint64_t pass = (uint64_t)seg * kOrderPasses + tid;
-    const uint2 d = pass < passes ? w.pass_peaks[pass] : make_uint2(0u, 0u);
     uint32_t before = 0;
     for (uint32_t q = tid; q < seg; q += kOrderPasses)
         before += w.seg_peaks[q];
     before = __reduce_add_sync(0xffffffffu, before);
-    const uint32_t incl = warp_incl_scan(d.y);
-    if (lane == 31u)
-        s_wsum[warp] = incl;
-    if (lane == 0)
-        s_wsum[16 + warp] = before;
-    __syncthreads();
-    uint32_t off = incl - d.y, rank0 = 0;
-    for (uint32_t q = 0; q < kOrderPasses / 32; ++q) {
-        off += q < warp ? s_wsum[q] : 0u;
-        rank0 += s_wsum[16 + q];
-    }
-    s_off[tid] = off;
-    s_base[tid] = d.x;
-    __syncthreads();
-    for (uint32_t k = tid; k < mine; k += kOrderPasses) {
-        uint32_t lo = 0, hi = kOrderPasses - 1;   // the last pass that starts at or before k
-        while (lo < hi) {
-            const uint32_t m = (lo + hi + 1) >> 1;
-            if (s_off[m] <= k)
-                lo = m;
-            else
-                hi = m - 1;
-        }
-        const uint32_t at = s_base[lo] + (k - s_off[lo]);
-        if (at < a.entries_cap && rank0 + k < o.capacity)
-            o.out[rank0 + k] = peak_record(g, a.entries[at]);
+    if ((tid & 31u) == 0)
+        s_before[tid >> 5] = before;
+    const uint32_t n = load_segment(sp, w, seg, passes);
+    uint32_t rank0 = 0;
+    for (uint32_t q = 0; q < kOrderPasses / 32; ++q)
+        rank0 += s_before[q];
+    for (uint32_t k = tid; k < n; k += kOrderPasses) {
+        const uint32_t q = segment_pass(sp, k), at = sp.base[q] + (k - sp.off[q]);
+        if (at >= a.entries_cap)
+            continue;
+        const uint4 en = a.entries[at];
+        const uint32_t rank = en.w ? en.w - 1u : k;
+        if (en.w != kNoPeak && (uint64_t)rank0 + rank < o.capacity)
+            o.out[rank0 + rank] = peak_record(g, en);
     }
 }
 
@@ -2682,8 +2785,14 @@ cudaError_t fill_tma_occupancy(const TileCfg &c, bool store, int *blocks_per_sm)
 cudaError_t launch_order_passes(const Geom &g, const Work &w, const ScanArgs &a, const OrderArgs &o, uint64_t passes,
                                 cudaStream_t st)
 {
-    return launch_pdl(k_order_passes, (uint32_t)((passes + kOrderPasses - 1) / kOrderPasses), kOrderPasses, 0, st, g, w,
-                      a, o, passes);
+    return launch_pdl(k_order_passes, (uint32_t)(((passes - 1) >> w.seg_shift) + 1), kOrderPasses, 0, st, g, w, a, o,
+                      passes);
+}
+
+cudaError_t launch_edges(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a, uint64_t passes,
+                         cudaStream_t st)
+{
+    return launch_pdl(k_edges, (uint32_t)(((passes - 1) >> w.seg_shift) + 1), kOrderPasses, 0, st, g, w, c, a, passes);
 }
 
 cudaError_t fill_scan_occupancy(const FillCfg &c, const ScanArgs &a, uint32_t nb, int *blocks_per_sm)

@@ -89,3 +89,42 @@ def test_sectors_count_edge_hits_once(ht, S):
         m = b.n_phi // S
         for k in range(S):
             assert np.array_equal(sec.matrix(k), M_ref[:, k * m:(k + 1) * m])
+
+
+@pytest.mark.parametrize("rows", [0, 1, 2, 16], ids=lambda r: f"rows{r}")
+@pytest.mark.parametrize("n_b", [96, 45])
+def test_crowded_passes(ht, n_b, rows):
+    """Many hits per slice (admission windows, crowded batches): the rows where
+    two passes meet are compared after the fill.  Around the number of hits per
+    slice that this begins at, with equal votes on both sides of an edge, and
+    with counts above the capacity."""
+    b, r = ht.Binning(2, 3, 53, n_b, 1, 1), ht.Ranges()
+    # 9 admissions per hit, 6 slices, 192 hits per slice: from 128 hits on (n // 2 of them) for one event, from 384 for three
+    for n in (254, 256, 383, 384, 3000):
+        events = [random_hits(n // 2, n), random_hits(0, 1), random_hits(n - n // 2, n + 1)]
+        for T in (1, 3, 9):
+            ref = []
+            for x, y, z in events:
+                M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+                ref.append((M_ref, *oracle.find_maxima(_ob(b), _orr(r), M_ref, T)))
+            with ht.Context(b, r, threshold=T, max_hits=n) as ctx:
+                ctx.set_tuning(fill_rows=rows)
+                for (x, y, z), (M_ref, pk_ref, n_ref) in zip(events, ref):
+                    ctx.fill(x, y, z)
+                    pk, total = ctx.find_maxima(capacity=1 << 16)
+                    assert total == n_ref
+                    assert_peaks_equal(pk, pk_ref)
+                    assert np.array_equal(ctx.matrix(), M_ref)
+                    ctx.fill(x, y, z)
+                    pk, total = ctx.find_maxima(capacity=7)
+                    assert total == n_ref
+                    assert_peaks_equal(pk, pk_ref[:7])
+            with ht.Batch(b, r, threshold=T, max_events=3, max_hits=n, capacity=1 << 16) as B:
+                for _ in range(3):
+                    pk, counts = B.run(*ht.Batch.concat(events))
+                    assert list(counts[:3]) == [q[2] for q in ref]
+                    at = 0
+                    for e, (M_ref, pk_ref, n_ref) in enumerate(ref):
+                        assert np.all(pk[at:at + n_ref]["event"] == e)
+                        assert_peaks_equal(pk[at:at + n_ref], pk_ref)
+                        at += n_ref
