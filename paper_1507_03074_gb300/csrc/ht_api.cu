@@ -379,10 +379,12 @@ ht_status ht_copy_matrix(ht_ctx *ctx, uint32_t *dst, uint64_t n_cells, uint32_t 
     if (!dst || n_cells != ctx->E.n_cells)
         return set_err(HT_E_INVAL, "dst must hold exactly n_theta*n_phi*n_a*n_b cells");
     cudaStream_t st = stream ? (cudaStream_t)stream : ctx->stream;
-    const cudaMemcpyKind kind = (flags & HT_MEM_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    CK(cudaMemcpyAsync(dst, ctx->E.d_M, n_cells * 4, kind, st));
-    if (!(flags & HT_MEM_DEVICE))
-        CK(cudaStreamSynchronize(st));
+    if (flags & HT_MEM_DEVICE) {
+        CK(hte::engine_copy_matrix(ctx->E, dst, st));
+        return HT_OK;
+    }
+    CK(cudaMemcpyAsync(dst, ctx->E.d_M, n_cells * 4, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
     return HT_OK;
 }
 

@@ -19,7 +19,7 @@ static const uint32_t kFusedPeakBuf = 512;     // K of a fused-fill CTA (at leas
 const char *const kKernelNames[K_NKINDS] = {"k_bin", "k_scatter", "k_fill_priv", "k_fill_scan", "k_fill_ws",
                                              "k_fill_peaks", "k_peaks", "k_clear", "k_fill_naive", "k_scan",
                                              "k_order", "k_peaks4d", "k_fill_tma", "k_bin_cluster", "k_fill_add",
-                                             "k_edges"};
+                                             "k_edges", "k_copy"};
 
 // ---------------------------------------------------------------------------
 // Profiling
@@ -853,6 +853,19 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     e = htk::launch_fill_priv(E.geom, w, f, grid, st);
     ++E.launches;
     return e;
+}
+
+cudaError_t engine_copy_matrix(Engine &E, uint32_t *dst, cudaStream_t st)
+{
+    cudaPointerAttributes at{};
+    if ((reinterpret_cast<uintptr_t>(dst) & 31u) || cudaPointerGetAttributes(&at, dst) != cudaSuccess ||
+        at.type != cudaMemoryTypeDevice || at.device != E.device) {
+        cudaGetLastError();
+        return cudaMemcpyAsync(dst, E.d_M, E.n_cells * 4, cudaMemcpyDeviceToDevice, st);
+    }
+    ProfScope ps(E, K_COPY, st);
+    ++E.launches;
+    return htk::launch_copy(dst, E.d_M, E.n_cells, st);
 }
 
 cudaError_t engine_scan(Engine &E, uint32_t n_events, htk::Peak *out, uint32_t capacity,

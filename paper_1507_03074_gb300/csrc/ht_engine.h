@@ -33,7 +33,7 @@ struct Tuning {
 // stream around every launch (enabled by ht_profile).
 enum KernelKind {
     K_BIN, K_SCATTER, K_FILL_PRIV, K_FILL_SCAN, K_FILL_WS, K_FILL_PEAKS, K_PEAKS, K_CLEAR, K_FILL_NAIVE, K_SCAN,
-    K_ORDER, K_PEAKS4D, K_FILL_TMA, K_BIN_CLUSTER, K_FILL_ADD, K_EDGES, K_NKINDS
+    K_ORDER, K_PEAKS4D, K_FILL_TMA, K_BIN_CLUSTER, K_FILL_ADD, K_EDGES, K_COPY, K_NKINDS
 };
 extern const char *const kKernelNames[K_NKINDS];
 
@@ -153,6 +153,10 @@ ht_status engine_configure(Engine &E, std::string *why);
 cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *z,
                         const uint32_t *d_hit_off, uint32_t n_hits0, uint32_t n_events,
                         uint32_t n_total, uint32_t flags, cudaStream_t st);
+
+// M_H to dst, device memory: the GPU's own, 32-byte aligned, by a kernel, else by
+// cudaMemcpyAsync.
+cudaError_t engine_copy_matrix(Engine &E, uint32_t *dst, cudaStream_t st);
 
 // The voting part of engine_fill alone, on the hits engine_fill last binned
 // (the autotuner re-runs it under each candidate tuning).

@@ -153,6 +153,8 @@ cudaError_t launch_peaks(const Geom &g, const Work &w, const ScanArgs &a, uint32
 // Accumulating fills of few hits: M_H += their votes, one reduction each (kAddRows A rows of a slice per warp).
 constexpr uint32_t kAddRows = 32;
 cudaError_t launch_fill_add(const Geom &g, const Work &w, uint32_t num_sms, cudaStream_t st);
+// n cells of M_H to device memory (both 32-byte aligned).
+cudaError_t launch_copy(uint32_t *dst, const uint32_t *src, uint64_t n, cudaStream_t st);
 cudaError_t launch_clear(uint32_t *M, uint64_t words, uint32_t grid, cudaStream_t st);
 cudaError_t launch_fill_naive(const Geom &g, const Work &w, uint32_t num_sms, cudaStream_t st);
 size_t scan_smem_bytes(const ScanArgs &a);

@@ -43,3 +43,23 @@ def test_matrix_memory_is_given_back(ht):
         for c in ctxs:
             c.close()
     assert torch.cuda.mem_get_info()[0] >= free - (8 << 20)
+
+
+@pytest.mark.parametrize("bins", [(1, 1, 1, 3), (1, 1, 2, 4), (1, 2, 31, 33), (2, 3, 64, 128), (1, 5, 1023, 9)], ids=str)
+@pytest.mark.parametrize("shift", [0, 1, 4, 8])
+def test_matrix_into_device_memory(ht, bins, shift):
+    """The matrix copied to device memory at any word, to its last cell and
+    not beyond."""
+    import torch
+    b, n = ht.Binning(*bins), 300
+    x, y, z = random_hits(n, 9, rmax=700.0)
+    with ht.Context(b, ht.Ranges(), threshold=2, max_hits=n) as ctx:
+        ctx.fill(x, y, z)
+        buf = torch.full((b.n_cells + 64,), -1, dtype=torch.int32, device="cuda")
+        dst = buf[shift:shift + b.n_cells]
+        torch.cuda.synchronize()
+        ctx.matrix_into(dst)
+        ctx.sync()
+        got = buf.cpu().numpy()
+        assert np.array_equal(got[shift:shift + b.n_cells].view(np.uint32), ctx.matrix().ravel())
+        assert np.all(got[:shift] == -1) and np.all(got[shift + b.n_cells:] == -1)
