@@ -228,8 +228,8 @@ uint64_t ht_launch_count(const ht_ctx *ctx);
  * then on, records a pair of CUDA events on the launching stream around
  * every kernel launch of the context; ht_profile(ctx, 0) stops recording.
  * ht_profile_read waits for the recorded events and writes up to cap
- * entries (one per kernel kind: k_prep, k_fill_priv, k_clear, k_fill_naive,
- * k_scan, k_order) with their launch count and summed duration. */
+ * entries (one per kernel kind that has run: k_bin_cluster, k_fill_tma,
+ * k_order and so on) with their launch count and summed duration. */
 typedef struct {
     char name[32];
     uint64_t launches;
@@ -271,7 +271,7 @@ ht_status ht_profile_read(ht_ctx *ctx, ht_kernel_time *out, uint32_t cap, uint32
  *                      n_b is not a multiple of 4), else 1, when it fits
  *                      (the fused modes only for non-accumulating, non-naive
  *                      fills)
- *   fill_vote_agg      1: the bulk-copy-tile fill (fill_fused_scan 5)
+ *   fill_vote_agg      1: the tile fill of M_H (fill_fused_scan 5)
  *                      aggregates the vote increments of a warp -- lanes
  *                      voting for the same cell find each other and one of
  *                      them adds their number; 0: one shared-memory atomic
@@ -280,15 +280,13 @@ ht_status ht_profile_read(ht_ctx *ctx, ht_kernel_time *out, uint32_t cap, uint32
  *                      units fit the cluster's 40 KB of counts (3 words per
  *                      unit and 1 per event: up to 53 events of 64 slices)
  *                      bins them and builds the unit lists in one launch of
- *                      a thread-block cluster (up to 8 CTAs of 1024 threads
- *                      reading each other's counts), which also splits the
- *                      work of the fill after it (bulk-copy-tile or
- *                      peaks-only) ahead of it -- shorter latency of one
- *                      event; larger fills take two launches anyway; 2: two
+ *                      a thread-block cluster (up to 8 CTAs of 512 threads
+ *                      reading each other's counts) -- shorter latency of
+ *                      one event; larger fills take two launches anyway; 2: two
  *                      launches (binning, lists) of small CTAs that fit
  *                      beside other events' kernels -- more events per
  *                      second when several contexts' events overlap; 0: 1
- *                      for the bulk-copy-tile and the peaks-only fill
+ *                      for the tile fill (with or without M_H)
  *                      unless fill_blocks_per_sm holds that fill below the
  *                      CTAs per SM that fit (the SMs are then shared with
  *                      other events), else 2
@@ -452,7 +450,7 @@ ht_status ht_validate(const ht_binning *binning, const ht_ranges *ranges, uint32
 ht_status ht_compute_edges(const ht_binning *binning, const ht_ranges *ranges, float *theta_edges,
                            float *phi_edges);
 
-/* The B-bin thresholds the kernels use (n_b + 1 floats): beta[k] is the
+/* The B-bin thresholds of the vote rule (n_b + 1 floats): beta[k] is the
  * smallest float B whose bin floor(fl(fl(B - b_min) / dB)) is >= k, so a vote
  * is in range iff beta[0] <= B < beta[n_b] and its bin is the number of
  * beta[1..n_b-1] that are <= B -- identical to the division rule for every

@@ -1230,9 +1230,8 @@ __device__ __forceinline__ bool is_peak_l2(const uint32_t *row, const uint32_t *
 // Append the candidate cells of one pass (rows iA .. iA + pr - 1 of slice
 // unit `slice_lin0`) to the CTA's candidate chunks, in linear order.  n_c
 // cells were listed as r * n_b + j in cand / candv (up to kFusedCand); with
-// more, the rows marked in hotm are read back: pass row r from rowsA + r rs
-// when r < split, else from rowsB + (r - split) rs (rs = row_stride, or n_b
-// when it is 0) -- M_H in global memory,
+// more, the rows marked in hotm are read back: pass row r from rowsA + r n_b
+// when r < split, else from rowsB + (r - split) n_b -- M_H in global memory,
 // or (SMEM) the shared staging buffers.  Entries are {lin within event,
 // event, votes, 0}.  All threads of the group call it.
 template <class G, bool SMEM = false>
@@ -1240,11 +1239,9 @@ __device__ __forceinline__ void emit_pass(const Geom &g, const Work &w, const Sc
                                           uint32_t &buf_n, uint32_t &nseq, uint32_t &total, const ChunkList &inner,
                                           const uint32_t *cand, const uint32_t *candv, uint32_t *srt, uint32_t *srtv,
                                           uint32_t n_c, uint64_t hotm, uint32_t pr, uint32_t iA, uint32_t slice_lin0,
-                                          uint32_t e, const uint32_t *rowsA, const uint32_t *rowsB, uint32_t split,
-                                          uint32_t row_stride = 0)
+                                          uint32_t e, const uint32_t *rowsA, const uint32_t *rowsB, uint32_t split)
 {
     const uint32_t tid = G::rank(), bd = G::size(), nb = g.nb;
-    const size_t rs = row_stride ? row_stride : nb;   // words between consecutive rows of rowsA / rowsB
     const uint32_t lin0 = slice_lin0 + iA * nb;
     if (n_c <= 32u) {
         // few candidates: the first warp ranks them and writes them in order
@@ -1290,7 +1287,7 @@ __device__ __forceinline__ void emit_pass(const Geom &g, const Work &w, const Sc
     for (uint32_t r = 0; r < pr; ++r) {
         if (!((hotm >> r) & 1ull))
             continue;
-        const uint32_t *row = r < split ? rowsA + (size_t)r * rs : rowsB + (size_t)(r - split) * rs;
+        const uint32_t *row = r < split ? rowsA + (size_t)r * nb : rowsB + (size_t)(r - split) * nb;
         for (uint32_t j0 = 0; j0 < nb; j0 += per_round) {
             const uint32_t j = j0 + tid;
             uint32_t cnt = 0, pj[1], pv[1];
@@ -1977,25 +1974,26 @@ __global__ void __launch_bounds__(256) k_order(Geom g, Work w, ScanArgs a, Order
 //
 // Order of the passes: a CTA's warps take a pass each of its runs (run i of
 // CTA c is run i * grid + c: c.run = warps neighbouring passes), and the last
-// passes go to whichever warp of the grid comes first, so that the whole grid writes
-// one neighbourhood of M_H at any time and the hits' uneven spread over the
-// slices averages out.
+// passes go to whichever warp of the grid comes first, so that the whole grid
+// writes one neighbourhood of M_H at any time (compressible memory wants that)
+// and the hits' uneven spread over the slices averages out.
 //
 // The peaks are found where the votes are: a vote that lifts its cell from
 // T - 1 to T lists the cell, and the listed cells are compared with their
 // neighbours in the tile.  For a cell on the first or last row of the pass
 // the votes of the row beyond are counted from the unit's lines (nothing waits
-// for the warp that owns it), or k_edges compares them later.  Each pass leaves {first entry, count} in
-// pass_peaks, in pass order, for k_order_passes.
+// for the warp that owns it), or k_edges compares them later.  Each pass leaves
+// {first entry, count} in pass_peaks, in pass order, for k_order_passes.
 //
-// Bound: the M_H write where votes are few (paper event, one launch: 46.7 us
-// for 268 MB, a third of a warp's time spent waiting for its copy; upgrade
-// event: 592 us for 4.3 GB, 7.25 TB/s), the votes' instructions where they are
-// many (admission windows, 38 M candidate votes: 129 us).  Against CTAs of 512
+// Bound: writing M_H where votes are few (paper event, one launch: 42 us for
+// 268 MB, 54 MB of which reach HBM, as M_H is compressed; upgrade event, in
+// flight: 498 us for 4.3 GB), the votes' instructions where they are many
+// (admission windows, 38 M candidate votes: 76 us).  Against CTAs of 512
 // threads that shared a tile, with three block barriers per pass and the peak
-// tests in a kernel of their own (events with three contexts in flight): paper
-// event 50.0 -> 41.0 us, windows 114.9 -> 94.2 us, batch of 100 events 4424 ->
-// 3772 us, four sectors 73.3 -> 56.2 us.  Tried on the way: the old tile
+// tests in a kernel of their own (events with three contexts in flight, with
+// what else changed around it): paper event 50.0 -> 33.7 us, windows 142.5 ->
+// 63.9 us, batch of 100 events 4424 -> 3090 us, four sectors 73.3 -> 33.8 us.
+// Tried on the way: the old tile
 // rotation behind a feeding warp, 48 us in flight (one barrier per pass, every
 // pass's latency exposed), and voting, draining and feeding warps around four
 // tiles, 44-47 us (the hand-overs cost more than the votes).
@@ -2307,7 +2305,7 @@ __device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const 
 }
 
 // STORE: the tiles go to M_H, else the peaks are all that is wanted (the same
-// passes without the copies: 29.4 us for a paper event, 23.5 us per event in
+// passes without the copies: 29.6 us for a paper event, 20.0 us per event in
 // flight; the u16 tiles of 512 threads that it replaces, whose cross-pass tests
 // went through rows in global memory and k_peaks, 31.8 and 31.5 us).  AGG:
 // warp-aggregated vote increments (vote_tile).  passes: over all events; runs:
