@@ -746,7 +746,8 @@ cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *
     return engine_vote(E, d_hit_off, n_hits0, n_events, flags, st);
 }
 
-// Zero what a fill counts up (the binning does the same).
+// Zero what a fill counts up (the binning does the same): before votes without a
+// binning, on top of a fill that no scan has ordered or, in the tile fill, of any.
 static cudaError_t engine_clear_counts(Engine &E, cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(E.d_ctr + htk::CTR_ENTRIES, 0,
@@ -781,6 +782,9 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     f.accumulate = accumulate ? 1u : 0u;
     const uint64_t items = (uint64_t)n_events * E.geom.n_slices * f.strips;
     const VoteKind kind = vote_kind(E, flags);
+    if (!fresh && (e = engine_clear_counts(E, st)) != cudaSuccess)   // voted again (the autotuner)
+        return e;
+    E.ctr_dirty = false;
     if (kind == ADD_VOTES) {
         ProfScope ps(E, K_FILL_ADD, st);
         e = htk::launch_fill_add(E.geom, w, (uint32_t)E.num_sms, st);
@@ -792,10 +796,6 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
         htk::TileCfg c = store ? E.tile : E.po_tile;
         c.edges_later = store && (double)E.binned * E.max_admit >=
                                      (double)htk::kEdgeHits * E.geom.n_slices * n_events;
-        if (!fresh) {   // voted again without a binning (the autotuner)
-            if ((e = engine_clear_counts(E, st)) != cudaSuccess)
-                return e;
-        }
         const uint64_t passes = htk::tile_passes(E.geom, c, n_events);
         const uint32_t grid = (uint32_t)std::max<uint64_t>(
             1, std::min<uint64_t>(store ? E.tma_grid : E.po_grid, (passes + c.warps - 1) / c.warps));
@@ -889,7 +889,8 @@ cudaError_t engine_scan(Engine &E, uint32_t n_events, htk::Peak *out, uint32_t c
         ProfScope ps(E, K_ORDER, st);
         e = htk::launch_order_passes(E.geom, w, a, o, E.fused_passes, st);
         ++E.launches;
-        return e;   // the counters keep the peaks until the next binning (ctr_dirty)
+        E.ctr_dirty = false;   // its first CTA zeroes them
+        return e;
     }
     if (E.fused_valid && E.fused_events == n_events) {
         // the fused fill already found the peaks: only order them

@@ -2595,8 +2595,13 @@ __global__ void __launch_bounds__(kOrderPasses) k_order_passes(Geom g, Work w, S
     if (seg == 0) {
         if (tid == 0 && o.status_out)
             *o.status_out = *w.status;
-        for (uint32_t e = tid; e < w.n_events; e += kOrderPasses)
+        // no other CTA reads the counters: this one leaves them as k_order does
+        for (uint32_t e = tid; e < w.n_events; e += kOrderPasses) {
             o.counts[e] = o.ev_count[e];
+            o.ev_count[e] = 0u;
+        }
+        if (tid == 0)
+            *o.g_count = 0u;
     }
     if (mine == 0)
         return;
