@@ -466,7 +466,10 @@ ht_status ht_compute_b_thresholds(const ht_binning *binning, const ht_ranges *ra
  * sector and merges the results.  Here the n_sectors sectors are parts of one
  * matrix on the current device: sector k owns phi bins [k m, (k + 1) m) of the
  * binning (m = n_phi / n_sectors), so its matrix equals those phi bins of the
- * unsplit M_H and the merged peaks equal the unsplit peaks.
+ * unsplit M_H and the merged peaks equal the unsplit peaks.  Calls on one
+ * object run on the device in the order they are made, also when they name
+ * different streams (eager calls among themselves, and the calls inside one
+ * stream capture).
  * Requirements: n_phi % n_sectors == 0 and win_phi == 0 (a phi window would
  * need the neighbouring sector's hits); otherwise as ht_create.  max_hits
  * bounds one fill.  Errors: HT_E_INVAL, HT_E_NOMEM, HT_E_CUDA. */

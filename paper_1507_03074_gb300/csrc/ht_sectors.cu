@@ -27,6 +27,11 @@ struct ht_sectors {
     uint32_t max_hits = 0;
     ht_ctx *ctx = nullptr;            // the unsplit binning
     cudaStream_t stream = nullptr;    // the object's own stream
+    // the end of the last call, and of the last one that was captured (in the
+    // capture cap_id): calls run in the order they are made, on whichever streams
+    cudaEvent_t done = nullptr, cap_done = nullptr;
+    bool done_pending = false;
+    unsigned long long cap_id = 0;
     bool poisoned = false;
 };
 
@@ -64,6 +69,30 @@ ht_status pass_on(ht_sectors *sec, ht_status s)
     return s;
 }
 
+// Run a step of the object on st, behind the step before it whatever stream
+// that took: `call` enqueues it.  A captured step and an eager one do not wait for each
+// other (a capture cannot wait for work outside it, nor anything for an event
+// inside it): the order of a graph's launch is its launcher's.
+template <class F>
+ht_status in_order(ht_sectors *sec, cudaStream_t st, F call)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    SCK(cudaStreamGetCaptureInfo(st, &cs, &id));
+    const bool captured = cs != cudaStreamCaptureStatusNone;
+    if (captured ? sec->cap_id == id : sec->done_pending)
+        SCK(cudaStreamWaitEvent(st, captured ? sec->cap_done : sec->done, 0));
+    const ht_status s = pass_on(sec, call());
+    if (sec->poisoned)
+        return s;
+    SCK(cudaEventRecord(captured ? sec->cap_done : sec->done, st));
+    if (captured)
+        sec->cap_id = id;
+    else
+        sec->done_pending = true;
+    return s;
+}
+
 } // namespace
 
 extern "C" {
@@ -74,7 +103,13 @@ ht_status ht_sectors_destroy(ht_sectors *sec)
         return HT_OK;
     if (sec->stream)
         cudaStreamSynchronize(sec->stream);
+    if (sec->done_pending)
+        cudaEventSynchronize(sec->done);
     ht_destroy(sec->ctx);
+    if (sec->done)
+        cudaEventDestroy(sec->done);
+    if (sec->cap_done)
+        cudaEventDestroy(sec->cap_done);
     if (sec->stream)
         cudaStreamDestroy(sec->stream);
     delete sec;
@@ -113,8 +148,10 @@ ht_status ht_sectors_create(const ht_binning *binning, const ht_ranges *ranges, 
         ht_sectors_destroy(sec);
         return hte::report(s, msg);
     }
-    const cudaError_t e = cudaStreamCreateWithFlags(&sec->stream, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
+    cudaError_t e;
+    if ((e = cudaStreamCreateWithFlags(&sec->stream, cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&sec->done, cudaEventDisableTiming)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&sec->cap_done, cudaEventDisableTiming)) != cudaSuccess) {
         cudaGetLastError();
         ht_sectors_destroy(sec);
         return hte::report(HT_E_CUDA, std::string("sector setup: ") + cudaGetErrorString(e));
@@ -136,7 +173,8 @@ ht_status ht_sectors_fill(ht_sectors *sec, const float *x, const float *y, const
         return hte::report(HT_E_INVAL, "hit arrays must not be NULL");
     if (n_hits > sec->max_hits)
         return hte::report(HT_E_INVAL, "more hits than max_hits");
-    return pass_on(sec, ht_fill(sec->ctx, x, y, z, n_hits, flags, stream ? stream : sec->stream));
+    cudaStream_t st = stream ? (cudaStream_t)stream : sec->stream;
+    return in_order(sec, st, [&] { return ht_fill(sec->ctx, x, y, z, n_hits, flags, st); });
 }
 
 ht_status ht_sectors_find_maxima(ht_sectors *sec, ht_peak *out, uint32_t capacity, uint32_t *n_found,
@@ -150,7 +188,8 @@ ht_status ht_sectors_find_maxima(ht_sectors *sec, ht_peak *out, uint32_t capacit
         return hte::report(HT_E_INVAL, "unknown flag");
     if (!n_found || (capacity && !out))
         return hte::report(HT_E_INVAL, "out (capacity > 0) and n_found must not be NULL");
-    return pass_on(sec, ht_find_maxima(sec->ctx, out, capacity, n_found, flags, stream ? stream : sec->stream));
+    cudaStream_t st = stream ? (cudaStream_t)stream : sec->stream;
+    return in_order(sec, st, [&] { return ht_find_maxima(sec->ctx, out, capacity, n_found, flags, st); });
 }
 
 ht_status ht_sectors_copy_matrix(ht_sectors *sec, uint32_t sector, uint32_t *dst, uint64_t n_cells)
@@ -164,7 +203,8 @@ ht_status ht_sectors_copy_matrix(ht_sectors *sec, uint32_t sector, uint32_t *dst
     const uint64_t slice = (uint64_t)E.geom.na * E.geom.nb, part = sec->m * slice;   // cells of a slice, of a theta row
     if (!dst || n_cells != E.geom.nt * part)
         return hte::report(HT_E_INVAL, "dst must hold exactly n_theta*n_phi*n_a*n_b cells");
-    SCK(cudaDeviceSynchronize());   // the fill may have run on any stream
+    if (sec->done_pending)
+        SCK(cudaStreamWaitEvent(sec->stream, sec->done, 0));   // the fill may have run on any stream
     for (uint32_t t = 0; t < E.geom.nt; ++t)
         SCK(cudaMemcpyAsync(dst + t * part, E.d_M + ((uint64_t)t * E.geom.np + (uint64_t)sector * sec->m) * slice,
                             part * 4, cudaMemcpyDeviceToHost, sec->stream));

@@ -97,3 +97,82 @@ def test_sectors_reject_bad_arguments(ht):
             sec.fill(*[np.zeros(17, np.float32)] * 3)
         with pytest.raises(ht.HTError):
             sec.matrix(4)
+
+
+def test_sectors_order_across_streams(ht):
+    """A step waits for the step before it whatever stream that took: a fill of
+    4 GiB on one stream, its peaks asked for on another or on the object's own
+    at once, the next fill on a third."""
+    import torch
+    b, r, T = ht.Binning(8, 32, 2048, 2048), ht.Ranges(), 10
+    evs = [[torch.from_numpy(a).cuda() for a in (ev.x, ev.y, ev.z)]
+           for ev in (synth.make_event(*synth.split_hits(n), seed=n) for n in (50000, 21000, 37000))]
+    ref = []
+    with ht.Context(b, r, threshold=T, max_hits=50000) as ctx:
+        for ev in evs:
+            ctx.fill(*ev)
+            ref.append(ctx.find_maxima(capacity=1 << 16))
+        M_last = ctx.matrix()[:, 8:16]
+    assert len({n for _, n in ref}) == 3
+    sts = [torch.cuda.Stream() for _ in range(4)]
+    torch.cuda.synchronize()
+    with ht.Sectors(b, r, threshold=T, n_sectors=4, max_hits=50000) as sec:
+        outs = [torch.zeros(1 << 16, 8, dtype=torch.int32, device="cuda") for _ in range(9)]
+        cnts = [torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(9)]
+        torch.cuda.synchronize()
+        for k in range(9):
+            sec.fill(*evs[k % 3], stream=sts[k % 4])
+            sec.find_maxima(capacity=1 << 16, out=outs[k], count=cnts[k], stream=sts[(k + 1) % 4])
+        torch.cuda.synchronize()
+        for k in range(9):
+            pk, n = ref[k % 3]
+            assert int(cnts[k].item()) == n
+            assert_peaks_equal(outs[k].cpu().numpy().view(ht.PEAK_DTYPE).reshape(-1)[:n], pk)
+        for k in range(3):   # host memory, on the object's own stream
+            sec.fill(*evs[k], stream=sts[k])
+            pk, n = sec.find_maxima(capacity=1 << 16)
+            assert n == ref[k][1]
+            assert_peaks_equal(pk, ref[k][0])
+        sec.fill(*evs[1], stream=sts[0])
+        sec.fill(*evs[2], stream=sts[1])
+        assert np.array_equal(sec.matrix(1), M_last)
+
+
+def test_sectors_capture_between_eager_calls(ht, paper11):
+    """Captured steps and eager ones: neither waits for the other's events, and
+    inside a capture the order holds across its streams."""
+    import torch
+    ev, M_ref, pk_ref, n_ref = paper11
+    b, r = ht.Binning(*synth.PAPER_BINNING), ht.Ranges()
+    with ht.Sectors(b, r, threshold=10, n_sectors=4, max_hits=ev.n_hits) as sec:
+        d = [torch.from_numpy(a).cuda() for a in (ev.x, ev.y, ev.z)]
+        out = torch.zeros(n_ref, 8, dtype=torch.int32, device="cuda")
+        cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+        st, other, eager = (torch.cuda.Stream() for _ in range(3))
+        torch.cuda.synchronize()
+
+        def check_out():
+            torch.cuda.synchronize()
+            assert int(cnt.item()) == n_ref
+            assert_peaks_equal(out.cpu().numpy().view(ht.PEAK_DTYPE).reshape(-1), pk_ref)
+            out.zero_()
+            cnt.zero_()
+            torch.cuda.synchronize()
+
+        def steps(s0, s1):
+            sec.fill(*d, stream=s0)
+            sec.find_maxima(capacity=n_ref, out=out, count=cnt, stream=s1)
+
+        steps(eager, eager)
+        check_out()
+        for _ in range(2):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=st):
+                other.wait_stream(st)
+                steps(st, other)
+                st.wait_stream(other)
+            for _ in range(2):
+                g.replay()
+                check_out()
+            steps(st, eager)
+            check_out()
