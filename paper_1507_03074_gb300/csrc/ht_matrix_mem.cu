@@ -112,19 +112,27 @@ bool map_compressible(MatrixMem &m, size_t bytes, int device)
 cudaError_t matrix_alloc(MatrixMem &m, size_t bytes, int device, bool compressible)
 {
     m = MatrixMem{};
-    if (compressible && bytes >= kCompressMin && map_compressible(m, bytes, device))
-        return cudaSuccess;
+    if (compressible && bytes >= kCompressMin) {
+        if (cudaMalloc(&m.guard, 16) == cudaSuccess && map_compressible(m, bytes, device))
+            return cudaSuccess;
+        cudaGetLastError();
+        cudaFree(m.guard);
+        m = MatrixMem{};
+    }
     return cudaMalloc(reinterpret_cast<void **>(&m.p), bytes);
 }
 
 void matrix_free(MatrixMem &m)
 {
     if (m.mapped) {
-        cudaDeviceSynchronize();   // as cudaFree: no kernel or copy still uses the memory
+        // Freeing the guard waits for every kernel and copy of the device that owns
+        // it, whichever device is current, and may run beside another thread's
+        // stream capture, which a device synchronisation would break.  Where it
+        // fails the memory stays mapped: something may still use it.
         const DriverCalls &d = driver();
         const CUdeviceptr va = reinterpret_cast<CUdeviceptr>(m.p);
-        d.unmap(va, m.mapped);
-        d.unreserve(va, m.mapped);
+        if (cudaFree(m.guard) == cudaSuccess && d.unmap(va, m.mapped) == CUDA_SUCCESS)
+            d.unreserve(va, m.mapped);
     } else {
         cudaFree(m.p);
     }

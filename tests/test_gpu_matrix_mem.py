@@ -63,3 +63,44 @@ def test_matrix_into_device_memory(ht, bins, shift):
         got = buf.cpu().numpy()
         assert np.array_equal(got[shift:shift + b.n_cells].view(np.uint32), ctx.matrix().ravel())
         assert np.all(got[:shift] == -1) and np.all(got[shift + b.n_cells:] == -1)
+
+
+@pytest.mark.parametrize("n_a", [64, 2048], ids=["ordinary", "compressible"])
+def test_destroyed_beside_a_capture(ht, n_a):
+    """A context is destroyed by one thread while another captures a stream: the
+    capture stays valid, and the context's memory is given back."""
+    import threading
+
+    import torch
+    b, r, T = ht.Binning(1, 2, n_a, 2048), ht.Ranges(), 3
+    x, y, z = random_hits(600, n_a)
+    dev = [torch.from_numpy(a).cuda() for a in (x, y, z)]
+    M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+    pk_ref, n_ref = oracle.find_maxima(_ob(b), _orr(r), M_ref, T)
+    out = torch.zeros(n_ref, 8, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    st = torch.cuda.Stream()
+    with ht.Context(b, r, threshold=T, max_hits=600) as ctx:
+        ctx.fill(*dev, stream=st)
+        ctx.find_maxima(capacity=n_ref, out=out, count=cnt, stream=st)
+        ctx.sync(stream=st)
+        out.zero_()
+        cnt.zero_()
+        other = ht.Context(b, r, threshold=T, max_hits=600)
+        other.fill(*dev)
+        other.sync()
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st, capture_error_mode="thread_local"):
+            ctx.fill(*dev, stream=st)
+            t = threading.Thread(target=other.close)
+            t.start()
+            t.join()
+            ctx.find_maxima(capacity=n_ref, out=out, count=cnt, stream=st)
+        g.replay()
+        torch.cuda.synchronize()
+        assert int(cnt.item()) == n_ref
+        assert_peaks_equal(out.cpu().numpy().view(ht.PEAK_DTYPE).reshape(-1), pk_ref)
+        if n_a == 2048:
+            assert torch.cuda.mem_get_info()[0] >= free + b.n_cells * 4
