@@ -7,6 +7,7 @@
 #include "ht_geom.h"
 #include "ht_trace.h"
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -28,16 +29,20 @@ struct ht_ctx {
     hte::Engine E;
     cudaStream_t stream = nullptr;
     float *d_in = nullptr;        // 3 * max_hits device staging
-    float *h_in = nullptr;        // 3 * max_hits mapped pinned staging
+    // mapped pinned staging: max_hits hits, or two places of place_hits that fills
+    // read in place take in turn
+    float *h_in = nullptr;
     float *h_in_dev = nullptr;    // its device address
+    uint32_t place_hits = 0;
     uint32_t *h_small = nullptr;  // mapped pinned: [0] count (written by the order kernel), [1] status
     uint32_t *h_small_dev = nullptr;  // its device address
     uint32_t *d_small = nullptr;  // device: [2] the 4-D scan's 2-D count
     htk::Peak *h_peaks = nullptr;     // mapped pinned peaks of host-mode ht_find_maxima
     htk::Peak *h_peaks_dev = nullptr; // their device address
     uint32_t peaks_cap = 0;
-    cudaEvent_t ev_in = nullptr;
-    bool ev_in_pending = false;
+    cudaEvent_t ev_in[2] = {};    // per place: its hits have been read
+    bool ev_in_pending[2] = {};
+    uint32_t next_place = 0;
     uint32_t acc_hits = 0;
     bool last_peaks_only = false;  // the last fill left M_H as it was
     htk::Peak *d_p2 = nullptr;     // the 2-D peak list of 4-D scans (E.scan.entries_cap entries)
@@ -56,7 +61,9 @@ Engine &ctx_engine(ht_ctx *c) { return c->E; }
 // the host, instead of being copied to the device first: the copy's hand-over
 // to the kernel costs more than the reads (blocking round trips, in place /
 // copied: 120 hits 32.0 / 33.2 us, 4990 hits 70.3 / 72.4 us, 16000 hits 136 / 139
-// us).
+// us).  The staging of such a fill is read while its kernels run, so there are two
+// places for it: the next fill's hits go to the other one, and a caller who only
+// enqueues is one fill ahead of the GPU.
 static constexpr uint32_t kReadInPlace = 16384;
 
 static ht_status cuda_fail(ht_ctx *c, cudaError_t e, const char *what)
@@ -157,13 +164,16 @@ ht_status ht_create(const ht_binning *binning, const ht_ranges *ranges, uint32_t
         delete ctx;
         return set_err(s, why);
     }
+    ctx->place_hits = std::min(max_hits, kReadInPlace);
+    const size_t in_bytes = (size_t)std::max(max_hits, 2 * ctx->place_hits) * 12 + 64;
     cudaError_t e;
     if ((e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&ctx->ev_in, cudaEventDisableTiming)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&ctx->ev_in[0], cudaEventDisableTiming)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&ctx->ev_in[1], cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaMalloc(&ctx->d_in, (size_t)max_hits * 12 + 64)) != cudaSuccess ||
         (e = cudaMalloc(&ctx->d_small, 16)) != cudaSuccess ||
         (p2_bytes(ctx) <= kSmallP2 && (e = alloc_p2(ctx)) != cudaSuccess) ||
-        (e = cudaHostAlloc(&ctx->h_in, (size_t)max_hits * 12 + 64, cudaHostAllocMapped)) != cudaSuccess ||
+        (e = cudaHostAlloc(&ctx->h_in, in_bytes, cudaHostAllocMapped)) != cudaSuccess ||
         (e = cudaHostGetDevicePointer((void **)&ctx->h_in_dev, ctx->h_in, 0)) != cudaSuccess ||
         (e = cudaHostAlloc(&ctx->h_small, 16, cudaHostAllocMapped)) != cudaSuccess ||
         (e = cudaHostGetDevicePointer((void **)&ctx->h_small_dev, ctx->h_small, 0)) != cudaSuccess) {
@@ -188,8 +198,9 @@ ht_status ht_destroy(ht_ctx *ctx)
     cudaFree(ctx->d_p2);
     cudaFreeHost(ctx->h_in);
     cudaFreeHost(ctx->h_small);
-    if (ctx->ev_in)
-        cudaEventDestroy(ctx->ev_in);
+    for (cudaEvent_t ev : ctx->ev_in)
+        if (ev)
+            cudaEventDestroy(ev);
     if (ctx->stream)
         cudaStreamDestroy(ctx->stream);
     delete ctx;
@@ -216,27 +227,37 @@ ht_status ht_fill(ht_ctx *ctx, const float *x, const float *y, const float *z, u
     cudaStream_t st = stream ? (cudaStream_t)stream : ctx->stream;
 
     const float *px = x, *py = y, *pz = z;
-    if (!(flags & HT_MEM_DEVICE) && n_hits) {
-        if (ctx->ev_in_pending)
-            CK(cudaEventSynchronize(ctx->ev_in));       // staging free again
-        const size_t bytes = (size_t)n_hits * 4;
-        std::memcpy(ctx->h_in, x, bytes);
-        std::memcpy(ctx->h_in + n_hits, y, bytes);
-        std::memcpy(ctx->h_in + 2 * (size_t)n_hits, z, bytes);
-        px = ctx->h_in_dev;
-        if (n_hits > kReadInPlace) {
-            CK(cudaMemcpyAsync(ctx->d_in, ctx->h_in, 3 * bytes, cudaMemcpyHostToDevice, st));
-            CK(cudaEventRecord(ctx->ev_in, st));
-            ctx->ev_in_pending = true;
+    const bool host = !(flags & HT_MEM_DEVICE) && n_hits, in_place = host && n_hits <= kReadInPlace;
+    const uint32_t place = in_place ? ctx->next_place : 0u;
+    if (host) {
+        for (uint32_t k = 0; k < 2; ++k)   // a copied fill takes the whole staging
+            if (ctx->ev_in_pending[k] && (!in_place || k == place)) {
+                CK(cudaEventSynchronize(ctx->ev_in[k]));
+                ctx->ev_in_pending[k] = false;
+            }
+        const size_t bytes = (size_t)n_hits * 4, at = (size_t)place * 3 * ctx->place_hits;
+        float *h = ctx->h_in + at;
+        std::memcpy(h, x, bytes);
+        std::memcpy(h + n_hits, y, bytes);
+        std::memcpy(h + 2 * (size_t)n_hits, z, bytes);
+        if (in_place) {
+            px = ctx->h_in_dev + at;
+        } else {
+            CK(cudaMemcpyAsync(ctx->d_in, h, 3 * bytes, cudaMemcpyHostToDevice, st));
+            for (uint32_t k = 0; k < 2; ++k) {
+                CK(cudaEventRecord(ctx->ev_in[k], st));
+                ctx->ev_in_pending[k] = true;
+            }
             px = ctx->d_in;
         }
         py = px + n_hits;
         pz = px + 2 * (size_t)n_hits;
     }
     CK(hte::engine_fill(ctx->E, px, py, pz, nullptr, n_hits, 1, n_hits, flags & ~(uint32_t)HT_MEM_DEVICE, st));
-    if (px == ctx->h_in_dev && n_hits) {
-        CK(cudaEventRecord(ctx->ev_in, st));
-        ctx->ev_in_pending = true;
+    if (in_place) {
+        CK(cudaEventRecord(ctx->ev_in[place], st));
+        ctx->ev_in_pending[place] = true;
+        ctx->next_place ^= 1u;
     }
     ctx->acc_hits = (uint32_t)acc;
     ctx->last_peaks_only = (flags & HT_PEAKS_ONLY) != 0;
