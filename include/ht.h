@@ -228,8 +228,10 @@ uint64_t ht_launch_count(const ht_ctx *ctx);
  * then on, records a pair of CUDA events on the launching stream around
  * every kernel launch of the context; ht_profile(ctx, 0) stops recording.
  * ht_profile_read waits for the recorded events and writes up to cap
- * entries (one per kernel kind that has run: k_bin_cluster, k_fill_tma,
- * k_order and so on) with their launch count and summed duration. */
+ * entries, one per kernel kind (k_bin_cluster, k_fill_tma, k_order and so on;
+ * k_fill_peaks is the tile fill without the writing), with their launch count
+ * (0 for the kinds that have not run) and summed duration; *n receives the
+ * number of kinds.  out may be NULL when cap is 0. */
 typedef struct {
     char name[32];
     uint64_t launches;

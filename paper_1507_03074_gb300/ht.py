@@ -379,6 +379,16 @@ def _cached_autotune(path, key: str, run, apply):
     return tun, us
 
 
+def _profile(read, h) -> dict:
+    """{kernel: (launches, total_ms)} from a *_profile_read function: the number
+    of kernel kinds first, then that many entries."""
+    n = ctypes.c_uint32()
+    check(read(h, None, 0, ctypes.byref(n)))
+    arr = (c_kernel_time * n.value)()
+    check(read(h, ctypes.cast(arr, ctypes.c_void_p), n.value, ctypes.byref(n)))
+    return {k.name.decode(): (int(k.launches), float(k.total_ms)) for k in arr}
+
+
 class Context:
     """One event at a time (ht_create / ht_fill / ht_find_maxima).  A context
     owns its stream, staging, M_H and counters, so several contexts fed
@@ -442,12 +452,9 @@ class Context:
         check(lib().ht_profile(self._h, 1 if enable else 0))
 
     def profile_read(self) -> dict:
-        """ht_profile_read: {kernel: (launches, total_ms)} (synchronises)."""
-        arr = (c_kernel_time * 16)()
-        n = ctypes.c_uint32()
-        check(lib().ht_profile_read(self._h, ctypes.cast(arr, ctypes.c_void_p), 16, ctypes.byref(n)))
-        return {arr[i].name.decode(): (int(arr[i].launches), float(arr[i].total_ms))
-                for i in range(min(n.value, 16))}
+        """ht_profile_read: {kernel: (launches, total_ms)} of every kernel kind
+        (synchronises)."""
+        return _profile(lib().ht_profile_read, self._h)
 
     def fill(self, x, y, z, accumulate: bool = False, naive: bool = False, peaks_only: bool = False, stream=None):
         n = int(x.numel() if _is_torch(x) else np.asarray(x).size)
@@ -692,11 +699,7 @@ class Batch:
         check(lib().ht_batch_profile(self._h, 1 if enable else 0))
 
     def profile_read(self) -> dict:
-        arr = (c_kernel_time * 16)()
-        n = ctypes.c_uint32()
-        check(lib().ht_batch_profile_read(self._h, ctypes.cast(arr, ctypes.c_void_p), 16, ctypes.byref(n)))
-        return {arr[i].name.decode(): (int(arr[i].launches), float(arr[i].total_ms))
-                for i in range(min(n.value, 16))}
+        return _profile(lib().ht_batch_profile_read, self._h)
 
 
 class Server:
