@@ -115,7 +115,8 @@ uint64_t matrix_bytes(const Key &k)
 }
 
 // Device memory of a lane with `events` events: matrices, hit workspace and
-// staging, the peak scratch (bounded like the engine bounds it) and a margin
+// staging (32 bytes a hit, and 24 per slice that it can enter: its record and its
+// vote line), the peak scratch (bounded like the engine bounds it) and a margin
 // for the bookkeeping.
 uint64_t lane_estimate(const ht_server_cfg &, const Key &k, uint32_t events, uint32_t max_hits)
 {
@@ -123,7 +124,8 @@ uint64_t lane_estimate(const ht_server_cfg &, const Key &k, uint32_t events, uin
     const uint64_t admit = (2ull * b.win_theta + 1) * (2ull * b.win_phi + 1);
     const uint64_t by_votes = (uint64_t)max_hits * admit * b.n_a / k.threshold + 1;
     const uint64_t by_space = (uint64_t)b.n_theta * b.n_phi * ((b.n_a + 1) / 2) * ((b.n_b + 1) / 2) * events;
-    return matrix_bytes(k) * events + (uint64_t)max_hits * 64 + std::min(by_votes, by_space) * 16 + (32ull << 20);
+    const uint64_t per_hit = std::max<uint64_t>(64, 32 + 24ull * htg::max_admit(b));
+    return matrix_bytes(k) * events + max_hits * per_hit + std::min(by_votes, by_space) * 16 + (32ull << 20);
 }
 
 uint32_t lane_hits(const ht_server_cfg &c, uint32_t events)

@@ -210,3 +210,27 @@ def test_serving_mix_matches_oracle(ht, serving_mix, cfg):
                 assert np.array_equal(pk[f], want[f]), (k, f)
         st = S.stats()
         assert st["completed"] == len(tickets) and st["lanes"] >= 2
+
+
+def test_server_budget_covers_the_hit_lists(ht):
+    """Lanes whose device memory is their hits' more than their matrices': with
+    admission windows a hit is listed nine times, and a micro-batch of 64 events
+    has room for 384000 hits.  The lane stays within the budget."""
+    b, r, T = ht.Binning(3, 16, 1, 5000, 1, 1), ht.Ranges(), 10
+    ob = oracle.Binning(3, 16, 1, 5000, 1, 1)
+    rng = np.random.default_rng(8)
+    evs = []
+    for _ in range(70):
+        rad, ph, z = rng.uniform(50, 900, 40), rng.uniform(-np.pi, np.pi, 40), rng.uniform(-900, 900, 40)
+        evs.append(tuple(np.repeat(a.astype(np.float32), 12) for a in (rad * np.cos(ph), rad * np.sin(ph), z)))
+    budget = 130 << 20
+    with ht.Server(hbm_budget_bytes=budget, n_streams=1, max_batch=64, max_hits_per_event=6000) as S:
+        tickets = [S.submit(b, r, T, *ev) for ev in evs]
+        for ev, t in zip(evs, tickets):
+            status, pk, n = _wait(S, t)
+            M, _ = oracle.fill(ob, oracle.Ranges(), *ev)
+            want, n_want = oracle.find_maxima(ob, oracle.Ranges(), M, T)
+            assert n == n_want > 0
+            for f in PEAK_FIELDS[:-1]:
+                assert np.array_equal(pk[f], want[f]), f
+        assert 0 < S.stats()["lane_bytes"] <= budget
