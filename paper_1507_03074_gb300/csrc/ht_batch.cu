@@ -30,7 +30,7 @@ struct ht_batch {
 
 namespace hte {
 
-static constexpr size_t kMaxGraphs = 8;
+static constexpr size_t kMaxGraphs = 16;
 
 ht_status runner_create(Runner &R, const ht_binning *b, const ht_ranges *r, uint32_t threshold, uint32_t max_events,
                         uint32_t max_hits, uint32_t capacity, std::string *why)
@@ -86,37 +86,41 @@ void runner_destroy(Runner &R)
 }
 
 // The kernels of one run (also what a graph captures).
-static cudaError_t enqueue_compute(Runner &R, uint32_t n_events, bool to_host, uint32_t fill_flags, cudaStream_t st)
+static cudaError_t enqueue_compute(Runner &R, uint32_t n_events, uint32_t n_hits, bool to_host, uint32_t fill_flags,
+                                   cudaStream_t st)
 {
     Engine &E = R.E;
     const uint32_t mh = E.max_hits;
     // offsets clamped to the staging size; n_total = max_hits: nothing the
-    // kernels take as arguments depends on the run
+    // kernels take as arguments depends on the run; n_hits only chooses whether
+    // k_edges follows the fill (part of the graph's key)
     cudaError_t e = engine_fill(E, R.d_xyz, R.d_xyz + mh, R.d_xyz + 2 * (size_t)mh, R.d_off, mh, n_events, mh,
-                                fill_flags, st);
+                                fill_flags, st, n_hits);
     if (e != cudaSuccess)
         return e;
     return engine_scan(E, n_events, to_host ? R.h_out_dev : R.d_out, R.capacity, to_host ? R.h_counts_dev : R.d_counts,
                        st, true, to_host ? R.h_counts_dev + E.max_events : nullptr);
 }
 
-// Replay the graph for (n_events, to_host), or run directly and capture one
-// for the next run with that shape.
-static cudaError_t run_compute(Runner &R, uint32_t n_events, bool to_host, uint32_t fill_flags, cudaStream_t st)
+// Replay the graph for this kind of run, or run directly and capture one for
+// the next run of the kind.
+static cudaError_t run_compute(Runner &R, uint32_t n_events, uint32_t n_hits, bool to_host, uint32_t fill_flags,
+                               cudaStream_t st)
 {
     if (R.E.prof.on || !R.graphs_ok)
-        return enqueue_compute(R, n_events, to_host, fill_flags, st);
+        return enqueue_compute(R, n_events, n_hits, to_host, fill_flags, st);
+    const bool edges = engine_edges_later(R.E, n_hits, n_events, fill_flags);
     for (auto &g : R.graphs)
-        if (g.n_events == n_events && g.to_host == to_host && g.fill_flags == fill_flags)
+        if (g.n_events == n_events && g.to_host == to_host && g.fill_flags == fill_flags && g.edges == edges)
             return cudaGraphLaunch(g.exec, st);
-    cudaError_t e = enqueue_compute(R, n_events, to_host, fill_flags, st);
+    cudaError_t e = enqueue_compute(R, n_events, n_hits, to_host, fill_flags, st);
     if (e != cudaSuccess)
         return e;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        const cudaError_t ec = enqueue_compute(R, n_events, to_host, fill_flags, st);
+        const cudaError_t ec = enqueue_compute(R, n_events, n_hits, to_host, fill_flags, st);
         e = cudaStreamEndCapture(st, &graph);
         if (ec != cudaSuccess)
             e = ec;
@@ -135,7 +139,7 @@ static cudaError_t run_compute(Runner &R, uint32_t n_events, bool to_host, uint3
         cudaGraphExecDestroy(R.graphs.front().exec);
         R.graphs.erase(R.graphs.begin());
     }
-    R.graphs.push_back({n_events, to_host, fill_flags, exec});
+    R.graphs.push_back({n_events, to_host, fill_flags, edges, exec});
     return cudaSuccess;
 }
 
@@ -156,8 +160,9 @@ cudaError_t runner_enqueue(Runner &R, uint32_t n_events, uint32_t n_hits, bool h
             cudaSuccess)
             return e;
     }
-    if ((e = run_compute(R, n_events, to_host, fill_flags, st)) != cudaSuccess)
+    if ((e = run_compute(R, n_events, n_hits, to_host, fill_flags, st)) != cudaSuccess)
         return e;
+    E.binned = n_hits;
     E.last_hit_off = R.d_off;         // what a later autotune re-times (also after a replay)
     E.last_n_hits0 = (uint32_t)mh;
     E.last_n_events = n_events;

@@ -692,12 +692,18 @@ static VoteKind vote_kind(const Engine &E, uint32_t flags)
     return E.use_tma && !E.use_ws ? TILES_MH : OTHER_FILL;
 }
 
+bool engine_edges_later(const Engine &E, uint32_t n_hits, uint32_t n_events, uint32_t flags)
+{
+    return vote_kind(E, flags) == TILES_MH &&
+           (double)n_hits * E.max_admit >= (double)htk::kEdgeHits * E.geom.n_slices * n_events;
+}
+
 cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *z,
                         const uint32_t *d_hit_off, uint32_t n_hits0, uint32_t n_events,
-                        uint32_t n_total, uint32_t flags, cudaStream_t st)
+                        uint32_t n_total, uint32_t flags, cudaStream_t st, uint32_t n_known)
 {
     E.fused_valid = false;
-    E.binned = n_total;
+    E.binned = std::min(n_total, n_known);
     // one binning launch ahead of a tile fill that has the SMs to itself
     const VoteKind kind = vote_kind(E, flags);
     const bool capped = kind == TILES_PEAKS ? E.po_capped : E.tma_capped;
@@ -794,8 +800,7 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     if (kind != OTHER_FILL) {
         const bool store = kind == TILES_MH;
         htk::TileCfg c = store ? E.tile : E.po_tile;
-        c.edges_later = store && (double)E.binned * E.max_admit >=
-                                     (double)htk::kEdgeHits * E.geom.n_slices * n_events;
+        c.edges_later = engine_edges_later(E, E.binned, n_events, flags);
         const uint64_t passes = htk::tile_passes(E.geom, c, n_events);
         const uint32_t grid = (uint32_t)std::max<uint64_t>(
             1, std::min<uint64_t>(store ? E.tma_grid : E.po_grid, (passes + c.warps - 1) / c.warps));

@@ -114,7 +114,7 @@ struct Engine {
     const uint32_t *last_hit_off = nullptr;   // what the last fill binned
     uint32_t last_n_hits0 = 0, last_n_events = 0;
     bool last_accumulate = false;
-    uint32_t binned = 0;         // hits the last binning was given
+    uint32_t binned = 0;         // hits of the last fill
 
     float *d_edges = nullptr;
     MatrixMem M;
@@ -148,12 +148,17 @@ ht_status engine_configure(Engine &E, std::string *why);
 
 // Step 1 for n_events events whose hits (device pointers) are concatenated;
 // d_hit_off (device, n_events + 1) or nullptr for one event of n_hits0 hits.
-// n_total (host) is the total hit count; it sizes the binning grid.  Unless
+// n_total (host) is the total hit count; it sizes the binning grid.  Where it is
+// only a bound (a graph that serves several runs), n_known is this run's count:
+// with it the tile fill decides on k_edges (engine_edges_later).  Unless
 // HT_ACCUMULATE or HT_FILL_NAIVE is set (or the tuning turns it off), the
 // fused kernel also finds the peaks, which engine_scan then only orders.
 cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *z,
                         const uint32_t *d_hit_off, uint32_t n_hits0, uint32_t n_events,
-                        uint32_t n_total, uint32_t flags, cudaStream_t st);
+                        uint32_t n_total, uint32_t flags, cudaStream_t st, uint32_t n_known = ~0u);
+
+// Whether a fill of n_hits hits leaves the comparisons across passes to k_edges.
+bool engine_edges_later(const Engine &E, uint32_t n_hits, uint32_t n_events, uint32_t flags);
 
 // M_H to dst, device memory: the GPU's own, 32-byte aligned, by a kernel, else by
 // cudaMemcpyAsync.

@@ -4,8 +4,8 @@
 // A runner owns an Engine for up to max_events events, fixed staging for
 // max_hits hits (x | y | z) and max_events + 1 hit offsets, and the peak
 // outputs.  One run: hit copies into the staging, the kernels of steps 1
-// and 2 (replayed from a CUDA graph captured per event count and output
-// place), then the results: either into device buffers, or written by the
+// and 2 (replayed from a CUDA graph captured per event count, output place and
+// kind of fill), then the results: either into device buffers, or written by the
 // order kernel straight into mapped pinned host memory (no copy back).
 #pragma once
 
@@ -33,6 +33,7 @@ struct Runner {
         uint32_t n_events;
         bool to_host;
         uint32_t fill_flags;         // HT_PEAKS_ONLY, HT_FILL_NAIVE or 0
+        bool edges;                  // the fill is followed by k_edges
         cudaGraphExec_t exec;
     };
     std::vector<Graph> graphs;

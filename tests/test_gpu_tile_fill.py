@@ -128,3 +128,31 @@ def test_crowded_passes(ht, n_b, rows):
                         assert np.all(pk[at:at + n_ref]["event"] == e)
                         assert_peaks_equal(pk[at:at + n_ref], pk_ref)
                         at += n_ref
+
+
+def test_edges_follow_the_runs_hits(ht):
+    """A batch with room for many more hits than a run has: whether the rows
+    where two passes meet are compared after the fill goes by the run's own hits
+    (192 admissions per slice on average), directly and in the captured graphs,
+    crowded and sparse runs in turn."""
+    b, r, T = ht.Binning(2, 3, 53, 96), ht.Ranges(), 3
+    runs = {}
+    for n in (100, 2303, 2304, 9000):     # two events of 6 slices: from 2304 hits on
+        evs = [random_hits(n // 3, n, rmax=700.0), random_hits(n - n // 3, n + 1, rmax=700.0)]
+        ref = []
+        for x, y, z in evs:
+            M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+            ref.append((M_ref, *oracle.find_maxima(_ob(b), _orr(r), M_ref, T)))
+        runs[n] = (evs, ref)
+    with ht.Batch(b, r, threshold=T, max_events=2, max_hits=1 << 16, capacity=1 << 16) as B:
+        for rep in range(3):
+            for n in (100, 9000, 2303, 2304):
+                evs, ref = runs[n]
+                B.profile(rep == 0)
+                pk, counts = B.run(*ht.Batch.concat(evs))
+                if rep == 0:
+                    assert B.profile_read()["k_edges"][0] == (n >= 2304), n
+                assert list(counts) == [q[2] for q in ref]
+                assert_peaks_equal(pk, np.concatenate([q[1] for q in ref]))
+                for e in range(2):
+                    assert np.array_equal(B.matrix(e), ref[e][0])
