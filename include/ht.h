@@ -243,7 +243,9 @@ ht_status ht_profile_read(ht_ctx *ctx, ht_kernel_time *out, uint32_t cap, uint32
 
 /* Launch shapes.  Every field 0 means automatic; results (M_H and peaks)
  * are identical for every accepted tuning, only the speed changes.
- *   fill_rows          A rows per shared-memory vote tile (power of two)
+ *   fill_rows          A rows per shared-memory vote tile (power of two); the
+ *                      tile fill takes lower tiles where such high ones would
+ *                      leave an SM fewer than 6 warps
  *   fill_threads       256, 512 or 1024 threads per fill CTA (the tile fill
  *                      runs as many of their warps, up to 12, as their tiles
  *                      fit)
@@ -294,7 +296,7 @@ ht_status ht_profile_read(ht_ctx *ctx, ht_kernel_time *out, uint32_t cap, uint32
  *                      other events), else 2
  * ht_set_tuning waits for the device, re-derives the shapes and returns
  * HT_E_INVAL for an impossible value; ht_get_tuning reports the shapes in
- * effect (0 fields filled in). */
+ * effect (0 fields filled in; fill_rows as asked for). */
 enum { HT_SCAN_AUTO = 0, HT_SCAN_BULK = 1, HT_SCAN_STREAM = 2, HT_SCAN_DIRECT = 3 };
 typedef struct {
     uint32_t fill_rows, fill_threads, fill_hits_staged, fill_blocks_per_sm;

@@ -147,10 +147,9 @@ ht_status engine_configure(Engine &E, std::string *why)
         *why = "fill_rows must be a power of two";
         return HT_E_INVAL;
     }
-    // with the bulk-copy-tile fill (asked for, or automatic where n_b allows
-    // it) fill_rows sizes its tiles; the other fills (accumulating, peaks-only)
-    // keep their own tile height
-    bool tma_mode = (t.fused == 0 || (t.fused == 5 && (b.n_b & 3u) == 0)) && b.n_b <= 4096;
+    // with the tile fill (asked for, or automatic where n_b allows it) fill_rows
+    // sizes its tiles; the other fills (accumulating) keep their own tile height
+    const bool tma_mode = (t.fused == 0 || (t.fused == 5 && (b.n_b & 3u) == 0)) && b.n_b <= 4096;
     // the tile fill's shape at W rows per pass: as many of fill_threads' warps as
     // their tiles fit, twice per SM unless the threads were asked for
     auto tile_shape = [&](uint32_t W) {
@@ -166,8 +165,6 @@ ht_status engine_configure(Engine &E, std::string *why)
         c.run = c.warps;
         return c;
     };
-    if (tma_mode && t.fill_W)   // a requested height that the tile fill cannot hold leaves it to the others
-        tma_mode = t.fill_W <= 64 && htk::tile_smem_bytes(tile_shape(t.fill_W)) <= kSmemMax;
     uint32_t W = tma_mode ? 0u : t.fill_W;
     if (!W) {
         // aim at ~64 KB tiles so that two CTAs share an SM
@@ -280,19 +277,29 @@ ht_status engine_configure(Engine &E, std::string *why)
     // --- the tile fill, and the same without the writing (peaks-only fills) --------
     E.tma_ok = E.tma_capped = E.po_ok = E.po_capped = false;
     auto tile_fit = [&](bool store, uint32_t W, htk::TileCfg &out, uint32_t &grid, bool &capped) {
-        if (!W) {
+        const bool asked = W != 0;
+        if (!asked) {
             W = 64;   // tiles of at most 16 KB, and lower ones while there are fewer passes than warps
             while (W > 2 && ((size_t)W * b.n_b * 4 > 16 * 1024 ||
                              (W > 4 && (uint64_t)E.max_events * g.n_slices * ((b.n_a + W - 1) / W) < 12ull * E.num_sms)))
                 W >>= 1;
         }
-        const htk::TileCfg c = tile_shape(std::min<uint32_t>(W, 64));
-        int occ = 0;
-        if (htk::tile_smem_bytes(c) > kSmemMax || htk::tile_passes(g, c, E.max_events) > 0x7fffffffull ||
-            htk::fill_tma_occupancy(c, store, &occ) != cudaSuccess || occ < 1) {
-            cudaGetLastError();
+        W = std::min<uint32_t>(W, 64);
+        htk::TileCfg c = tile_shape(W);
+        if (t.fused == 5 && htk::tile_smem_bytes(c) > kSmemMax)
             return false;
+        int occ = 0;
+        for (;; c = tile_shape(W >>= 1)) {
+            occ = 0;
+            if (htk::tile_smem_bytes(c) <= kSmemMax && htk::fill_tma_occupancy(c, store, &occ) != cudaSuccess) {
+                cudaGetLastError();
+                occ = 0;
+            }
+            if (!asked || W <= 2 || c.warps * (uint32_t)occ >= htk::kTileMinWarps)
+                break;
         }
+        if (occ < 1 || htk::tile_passes(g, c, E.max_events) > 0x7fffffffull)
+            return false;
         capped = t.fill_blocks_per_sm && (int)t.fill_blocks_per_sm < occ;
         if (t.fill_blocks_per_sm)
             occ = std::min<int>(occ, (int)t.fill_blocks_per_sm);
@@ -1103,7 +1110,7 @@ void engine_get_tuning(const Engine &E, ht_tuning *t)
     t->fill_vote_agg = E.use_tma ? E.tile.vote_agg : 0u;
     t->bin_cluster = E.tune.bin_cluster ? E.tune.bin_cluster : (E.use_tma && !E.tma_capped) ? 1u : 2u;
     if (E.use_tma) {
-        t->fill_rows = E.tile.W;
+        t->fill_rows = E.tune.fill_W ? E.tune.fill_W : E.tile.W;
         t->fill_threads = E.tile.threads;
         t->fill_hits_staged = E.fill.HC;
         t->fill_blocks_per_sm = E.num_sms ? E.tma_grid / (uint32_t)E.num_sms : 0;

@@ -39,6 +39,10 @@ struct TileCfg {
     uint32_t edges_later; // tiles that go to M_H: comparisons across passes are left to k_edges
 };
 constexpr uint32_t kTileWarps = 12;    // most warps of a tile-fill CTA (two such CTAs per SM: 80 registers a thread)
+// An asked-for height (fill_rows) is halved until an SM holds this many warps:
+// with 3 (16 rows of 1024) a peaks-only paper event takes 39.3 us in flight, with
+// 6 26.4 us, with 12 20.2 us; with 1 (32 rows) a paper event takes 121.7 us.
+constexpr uint32_t kTileMinWarps = 6;
 constexpr uint32_t kTileCand = 127;    // cells >= T that a pass lists (more: every cell is looked at)
 constexpr uint32_t kAhead = 4;         // lines per lane loaded ahead
 constexpr uint32_t kHandedOut = 3;     // passes per warp handed out at run time (at least)

@@ -156,3 +156,35 @@ def test_edges_follow_the_runs_hits(ht):
                 assert_peaks_equal(pk, np.concatenate([q[1] for q in ref]))
                 for e in range(2):
                     assert np.array_equal(B.matrix(e), ref[e][0])
+
+
+@pytest.mark.parametrize("peaks_only", [False, True])
+def test_high_tiles_leave_the_sm_its_warps(ht, peaks_only):
+    """Rows of 1024 bins: 16 to 64 rows per tile as asked for would leave an SM
+    three warps, one or none; the fill takes lower ones and is as fast as 8 rows."""
+    import torch
+    from paper_1507_03074_gb300 import synth
+    b, r = ht.Binning(*synth.PAPER_BINNING), ht.Ranges()
+    ev = synth.paper_event(seed=11)
+    d = [torch.from_numpy(a).cuda() for a in (ev.x, ev.y, ev.z)]
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with ht.Context(b, r, threshold=10, max_hits=ev.n_hits) as ctx:
+        ctx.fill(*d)
+        want, n_want = ctx.find_maxima(capacity=1 << 16)
+        times = {}
+        for rows in (8, 16, 32, 64):
+            ctx.set_tuning(fill_rows=rows)
+            assert ctx.get_tuning()["fill_rows"] == rows
+            for n in (20, 100):       # warm, then timed
+                t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                t0.record(st)
+                for _ in range(n):
+                    ctx.fill(*d, peaks_only=peaks_only, stream=st)
+                t1.record(st)
+                st.synchronize()
+                times[rows] = t0.elapsed_time(t1) / n
+            pk, n = ctx.find_maxima(capacity=1 << 16)
+            assert n == n_want
+            assert_peaks_equal(pk, want)
+        assert max(times.values()) < 1.4 * times[8], times
