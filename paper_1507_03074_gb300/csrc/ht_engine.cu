@@ -626,8 +626,7 @@ void engine_destroy(Engine &E)
     for (cudaEvent_t ev : E.prof.pool)
         cudaEventDestroy(ev);
     E.prof.pool.clear();
-    cudaFree(E.d_edges);
-    matrix_free(E.M);
+    matrix_free(E.M, E.d_edges);
     cudaFree(E.d_hits4);
     cudaFree(E.d_codes);
     cudaFree(E.d_slice);

