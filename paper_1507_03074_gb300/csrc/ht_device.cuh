@@ -45,6 +45,9 @@ struct Work {
     const uint32_t *hit_off;    // [n_events + 1] or nullptr: one event, n_hits0 hits
     uint32_t n_hits0;           // with hit_off: the bound every offset is clamped to (staging size)
     uint32_t n_events;
+    // the (event, slice) units u0 .. u0 + nu of this launch (the fills with a range
+    // per CTA); the scans get M at the first of them and count rows from there
+    uint32_t u0, nu;
     float4 *hits4;              // per hit: {x, x^2 + y^2, 2y, event (bits)}
     uint32_t *codes;            // per hit: (itheta << 16) | iphi, or kDropped
     uint32_t *M;                // vote matrices

@@ -111,6 +111,19 @@ static uint32_t chunks_for(uint64_t rows, uint32_t per_row, uint32_t K, uint32_t
     return (uint32_t)std::min<uint64_t>(rows * per_row / (K - per_round) + 2, 1u << 20);
 }
 
+// The vote weight of the fills that keep a candidate list per CTA.  Over more
+// than four windows they split the cells evenly: each window has its own lists,
+// and a list has room for all the cells that a split by cost may give its CTA.
+// (Two windows, upgrade event: 1096 us evenly, 1027 us by cost.  13 windows, a batch
+// of 100 events: by cost the lists alone would take 4.9 GB.)  The warp-specialised
+// fill, which hands nothing out at run time, splits evenly over any windows (16
+// events of 256 MiB in two: 829 us by cost, 745 us evenly).
+static uint32_t list_weight(const Engine &E, bool ws)
+{
+    const uint64_t units = (uint64_t)E.max_events * E.geom.n_slices;
+    return !E.win_units || (!ws && 4ull * E.win_units >= units) ? htk::kVoteWeight : 0u;
+}
+
 ht_status engine_configure(Engine &E, std::string *why)
 {
     const ht_binning &b = E.b;
@@ -372,9 +385,14 @@ ht_status engine_configure(Engine &E, std::string *why)
         occ = std::min<int>(occ, (int)t.scan_blocks_per_sm);
     E.scan_grid_max = (uint32_t)E.num_sms * (uint32_t)occ;
 
-    // --- chunk bookkeeping for the largest launch (max_events events) ---------
-    const uint32_t scan_grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.scan_grid_max, G_max));
-    const uint64_t items_max = (uint64_t)E.max_events * g.n_slices * f.strips;
+    // --- chunk bookkeeping for the largest launch (a window of max_events events) ---
+    const uint64_t units_max = (uint64_t)E.max_events * g.n_slices, slice_bytes = (uint64_t)g.na * g.nb * 4;
+    if (!E.d_M)   // (the matrices' memory is chosen by this, once)
+        E.win_units = E.tma_ok && units_max * slice_bytes > kWindowBytes
+                          ? (uint32_t)std::max<uint64_t>(1, kWindowBytes / slice_bytes) : 0u;
+    const uint64_t win = E.win_units ? E.win_units : units_max, windows = (units_max + win - 1) / win;
+    const uint64_t G_win = win * g.na, items_max = win * f.strips;
+    const uint32_t scan_grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.scan_grid_max, G_win));
     const uint32_t fused_grid = E.fused_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.fused_grid, items_max)) : 0;
     const uint32_t ws_grid = E.ws_ok ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.ws_grid, items_max)) : 0;
     E.max_passes = std::max(E.tma_ok ? htk::tile_passes(g, E.tile, E.max_events) : 0,
@@ -386,23 +404,22 @@ ht_status engine_configure(Engine &E, std::string *why)
         ++E.seg_shift;
     // the fused fill's candidate lists: one per CTA plus one per handed-out item
     const uint32_t fused_lists = fused_grid + (uint32_t)htk::dyn_items(items_max, fused_grid);
-    const uint32_t grid_cap = std::max(std::max(scan_grid, fused_lists), ws_grid);
-    uint32_t seq = chunks_for((G_max + scan_grid - 1) / scan_grid + 1, (g.nb + 1) / 2, s.K, 2 * kScanThreads);
+    const uint32_t grid_cap = (uint32_t)(windows * std::max(std::max(scan_grid, fused_lists), ws_grid));
+    uint32_t seq = chunks_for((G_win + scan_grid - 1) / scan_grid + 1, (g.nb + 1) / 2, s.K, 2 * kScanThreads);
     // the cost-balanced split gives a CTA at most `spread` times the items of
     // an even split (every strip costs at least its n_b-per-row writing share)
-    const double hits_per_unit = (double)std::max<uint32_t>(E.max_hits, 1) * E.max_admit /
-                                 ((double)E.max_events * g.n_slices);
-    const double spread = 1.0 + htk::kVoteWeight * hits_per_unit / g.nb;
-    auto rows_per_cta = [&](uint32_t grid) {
+    const double hits_per_unit = (double)std::max<uint32_t>(E.max_hits, 1) * E.max_admit / (double)win;
+    auto rows_per_cta = [&](uint32_t grid, bool ws) {
+        const double spread = 1.0 + list_weight(E, ws) * hits_per_unit / g.nb;
         return (uint64_t)(std::ceil((double)items_max / grid * spread) + 2) * f.W + 1;
     };
     if (E.fused_ok) {
-        const uint64_t fused_rows = rows_per_cta(fused_grid);
+        const uint64_t fused_rows = rows_per_cta(fused_grid, false);
         seq = std::max(seq, chunks_for(fused_rows, g.nb, E.fused_K,
                                        htk::fused_round(E.fused_fill.threads, E.fused_K)));
     }
     if (E.ws_ok) {
-        const uint64_t ws_rows = rows_per_cta(ws_grid);
+        const uint64_t ws_rows = rows_per_cta(ws_grid, true);
         seq = std::max(seq, chunks_for(ws_rows, g.nb, E.fused_K, htk::fused_round(E.ws_fill.threads, E.fused_K)));
     }
     s.seq_max = seq;
@@ -652,6 +669,7 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
                            const uint32_t *d_hit_off, uint32_t n_hits0, uint32_t n_events)
 {
     htk::Work w{};
+    w.nu = n_events * E.geom.n_slices;
     w.x = x;
     w.y = y;
     w.z = z;
@@ -676,6 +694,29 @@ static htk::Work make_work(Engine &E, const float *x, const float *y, const floa
     w.n_seg = (uint32_t)((E.max_passes / E.max_events * n_events) >> E.seg_shift) + 1u;
     w.seg_shift = E.seg_shift;
     return w;
+}
+
+// The windows of a launch over n_events events (see kWindowBytes): calls
+// f(w) with w.u0, w.nu set to each in turn, until one fails.
+template <class F>
+static cudaError_t each_window(const Engine &E, htk::Work w, F f)
+{
+    const uint32_t units = w.n_events * E.geom.n_slices, win = E.win_units ? E.win_units : units;
+    cudaError_t e = cudaSuccess;
+    for (w.u0 = 0; w.u0 < units && e == cudaSuccess; w.u0 += w.nu) {
+        w.nu = std::min(win, units - w.u0);
+        e = f(w);
+    }
+    return e;
+}
+
+// a with its candidate lists from list number `first` on.
+static htk::ScanArgs lists_from(htk::ScanArgs a, uint32_t first)
+{
+    a.desc += (size_t)first * a.seq_max;
+    a.cta_nseq += first;
+    a.cta_total += first;
+    return a;
 }
 
 // engine_vote's fill for these flags: the tile fill (TILES_MH: writing M_H,
@@ -792,7 +833,6 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     }
     htk::FillCfg f = E.fill;
     f.accumulate = accumulate ? 1u : 0u;
-    const uint64_t items = (uint64_t)n_events * E.geom.n_slices * f.strips;
     const VoteKind kind = vote_kind(E, flags);
     if (!fresh && (e = engine_clear_counts(E, st)) != cudaSuccess)   // voted again (the autotuner)
         return e;
@@ -834,17 +874,18 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
         a.K = E.fused_K;
         htk::FillCfg ff = ws ? E.ws_fill : E.fused_fill;
         ff.accumulate = 0u;
-        ff.vote_weight = htk::kVoteWeight;
-        const uint64_t items_ff = (uint64_t)n_events * E.geom.n_slices * ff.strips;
-        const uint32_t grid = (uint32_t)std::max<uint64_t>(
-            1, std::min<uint64_t>(ws ? E.ws_grid : E.fused_grid, items_ff));
-        const uint32_t lists = grid + (ff.dyn ? (uint32_t)htk::dyn_items(items_ff, grid) : 0u);
-        {
+        ff.vote_weight = list_weight(E, ws);
+        uint32_t lists = 0;
+        e = each_window(E, w, [&](const htk::Work &v) {
+            const uint64_t items = (uint64_t)v.nu * ff.strips;
+            const uint32_t grid = (uint32_t)std::min<uint64_t>(ws ? E.ws_grid : E.fused_grid, items);
+            const htk::ScanArgs l = lists_from(a, lists);
+            lists += grid + (ff.dyn ? (uint32_t)htk::dyn_items(items, grid) : 0u);
+            ++E.launches;
             ProfScope ps(E, ws ? K_FILL_WS : K_FILL_SCAN, st);
-            e = ws ? htk::launch_fill_ws(E.geom, w, ff, a, grid, st)
-               : htk::launch_fill_scan(E.geom, w, ff, a, grid, st);
-        }
-        ++E.launches;
+            return ws ? htk::launch_fill_ws(E.geom, v, ff, l, grid, st)
+                      : htk::launch_fill_scan(E.geom, v, ff, l, grid, st);
+        });
         if (e == cudaSuccess) {
             ProfScope ps(E, K_PEAKS, st);
             e = htk::launch_peaks(E.geom, w, a, lists, st);
@@ -859,11 +900,12 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
         }
         return e;
     }
-    const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(E.fill_grid, items));
-    ProfScope ps(E, K_FILL_PRIV, st);
-    e = htk::launch_fill_priv(E.geom, w, f, grid, st);
-    ++E.launches;
-    return e;
+    return each_window(E, w, [&](const htk::Work &v) {
+        const uint32_t grid = (uint32_t)std::min<uint64_t>(E.fill_grid, (uint64_t)v.nu * f.strips);
+        ++E.launches;
+        ProfScope ps(E, K_FILL_PRIV, st);
+        return htk::launch_fill_priv(E.geom, v, f, grid, st);
+    });
 }
 
 cudaError_t engine_copy_matrix(Engine &E, uint32_t *dst, cudaStream_t st)
@@ -916,15 +958,19 @@ cudaError_t engine_scan(Engine &E, uint32_t n_events, htk::Peak *out, uint32_t c
                 return e;
         }
         E.fused_valid = false;
-        const uint64_t G = (uint64_t)E.geom.n_slices * E.geom.na * n_events;
-        a.grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(a.grid, G));
-        {
+        uint32_t lists = 0;
+        e = each_window(E, w, [&](htk::Work v) {
+            v.M += (uint64_t)v.u0 * E.geom.na * E.geom.nb;
+            htk::ScanArgs l = lists_from(a, lists);
+            l.grid = (uint32_t)std::min<uint64_t>(a.grid, (uint64_t)v.nu * E.geom.na);
+            lists += l.grid;
+            ++E.launches;
             ProfScope ps(E, K_SCAN, st);
-            e = htk::launch_scan(E.geom, w, a, E.scan_kind, st);
-        }
+            return htk::launch_scan(E.geom, v, l, E.scan_kind, st);
+        });
         if (e != cudaSuccess)
             return e;
-        ++E.launches;
+        a.grid = lists;
     }
     {
         ProfScope ps(E, K_ORDER, st);

@@ -54,6 +54,13 @@ struct MatrixMem {
     size_t mapped = 0;           // bytes mapped by the driver calls (0: from cudaMalloc)
 };
 constexpr size_t kCompressMin = (size_t)32 << 20;
+// The fills and scans whose CTAs own a contiguous range each work through
+// compressible matrices window by window of at most this size: with ranges spread
+// over more, compressible memory is slower than ordinary (tiles of 16 KB in 2432
+// ranges, us written / read: 4 GiB 717 / 351, 8 GiB 2149 / 1502, 16 GiB 5209 / 4885;
+// in windows of 2 GiB 537 / 404, 1069 / 805, 2128 / 1612; of 4 GiB 16 GiB take 3200 /
+// 1759; ordinary memory 662 / 617, 1303 / 1231, 2625 / 2449 in any order).
+constexpr size_t kWindowBytes = (size_t)2 << 30;
 cudaError_t matrix_alloc(MatrixMem &m, size_t bytes, int device, bool compressible);
 // Frees guard, a cudaMalloc'd block of the matrix's device, which waits for the
 // device's work, then the matrix.
@@ -82,6 +89,7 @@ struct Engine {
     bool ws_ok = false;          // the warp-specialised fused kernel fits
     htk::FillCfg ws_fill{};      // its shape (threads = one group)
     uint32_t ws_grid = 0;
+    uint32_t win_units = 0;      // (event, slice) units per window (kWindowBytes); 0: all in one
     bool use_ws = false;         // fills run the warp-specialised kernel
     bool tma_ok = false;         // the bulk-copy-tile fused kernel fits
     htk::TileCfg tile{};         // its shape

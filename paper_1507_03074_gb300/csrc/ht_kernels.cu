@@ -623,11 +623,11 @@ __device__ __forceinline__ void vote_pass(const Geom &g, const Work &w, uint32_t
     }
 }
 
-// The work items [it0, it1) of CTA `cta` of `grid`: the (event, slice,
-// strip) items in order, cut where the estimated cost -- v = c.vote_weight
+// The work items [it0, it1) of CTA `cta` of `grid`, counted from the first of
+// the launch's units: the (event, slice, strip) items in order, cut where the estimated cost -- v = c.vote_weight
 // per (hit, row) vote plus one per cell written -- reaches cta / grid of the
 // total.  A unit u = (event, slice) costs n_a (n_b + v hits(u)), so the cost
-// before unit u is n_a (n_b u + v slice_off[u]); a cut inside a unit falls
+// before unit u0 + u is n_a (n_b u + v (slice_off[u0 + u] - slice_off[u0])); a cut inside a unit falls
 // on a strip boundary.  Every thread of the group calls
 // it and gets the same result; s_res: 2 shared words.
 template <class G = BlockGroup>
@@ -635,9 +635,10 @@ __device__ __forceinline__ void cta_items(const Geom &g, const Work &w, const Fi
                                           uint32_t grid, uint64_t n_static, uint64_t &it0, uint64_t &it1,
                                           unsigned long long *s_res)
 {
-    const uint32_t U = w.n_events * g.n_slices;
+    const uint32_t U = w.nu, off0 = __ldcg(&w.slice_off[w.u0]);
     auto cost = [&](uint32_t u) {
-        return (uint64_t)g.na * ((uint64_t)g.nb * u + (uint64_t)c.vote_weight * __ldcg(&w.slice_off[u]));
+        return (uint64_t)g.na *
+               ((uint64_t)g.nb * u + (uint64_t)c.vote_weight * (__ldcg(&w.slice_off[w.u0 + u]) - off0));
     };
     // the cost of the first n_static items
     const uint32_t us = (uint32_t)(n_static / c.strips), ks = (uint32_t)(n_static % c.strips);
@@ -732,7 +733,7 @@ __global__ void __launch_bounds__(1024) k_fill_priv(Geom g, Work w, FillCfg c)
 
     __shared__ unsigned long long s_rng[2];
     __shared__ uint32_t s_dyn;
-    const uint64_t items = (uint64_t)w.n_events * g.n_slices * c.strips;
+    const uint64_t items = (uint64_t)w.nu * c.strips, first = (uint64_t)w.u0 * c.strips;
     const uint64_t n_dyn = c.dyn ? dyn_items(items, gridDim.x) : 0, n_static = items - n_dyn;
     uint64_t it0, it1;
     cta_items(g, w, c, blockIdx.x, gridDim.x, n_static, it0, it1, s_rng);
@@ -774,12 +775,12 @@ __global__ void __launch_bounds__(1024) k_fill_priv(Geom g, Work w, FillCfg c)
             }
         }
     };
-    ItemCursor cur(g, c, it0);
+    ItemCursor cur(g, c, first + it0);
     for (uint64_t item = it0; item < it1; ++item, cur.next(g, c))
         do_item(cur);
     if (c.dyn)
         for (uint32_t d; (d = next_dyn_item(w, (uint32_t)n_dyn, &s_dyn)) < n_dyn;)
-            do_item(ItemCursor(g, c, n_static + d));
+            do_item(ItemCursor(g, c, first + n_static + d));
 }
 
 // ---------------------------------------------------------------------------
@@ -1049,8 +1050,9 @@ __device__ void scan_rows_slow(const Geom &g, const Work &w, const ScanArgs &a, 
     const uint32_t rounds = (units + bd - 1) / bd;
     for (uint64_t gr = ra; gr < rb; ++gr) {
         const uint32_t i = (uint32_t)(gr % g.na);
-        const uint32_t ev = (uint32_t)(gr / rows_ev);
-        const uint32_t row_lin0 = (uint32_t)((gr - (uint64_t)ev * rows_ev) * nb);
+        const uint64_t row_all = gr + (uint64_t)w.u0 * g.na;   // of all matrices' rows
+        const uint32_t ev = (uint32_t)(row_all / rows_ev);
+        const uint32_t row_lin0 = (uint32_t)((row_all - (uint64_t)ev * rows_ev) * nb);
         const uint32_t *row = base + (gr - b_first) * nb;
         const uint32_t *up = i > 0 ? row - nb : nullptr;
         const uint32_t *dn = i + 1 < g.na ? row + nb : nullptr;
@@ -1093,7 +1095,7 @@ __global__ void __launch_bounds__(256) k_scan_tma(Geom g, Work w, ScanArgs a)
 
     const uint32_t tid = threadIdx.x, bd = blockDim.x;
     const uint32_t nb = g.nb, T = g.threshold;
-    const uint64_t G = (uint64_t)g.n_slices * g.na * w.n_events;
+    const uint64_t G = (uint64_t)g.na * w.nu;
     const uint64_t g0 = G * blockIdx.x / gridDim.x, g1 = G * (blockIdx.x + 1) / gridDim.x;
     const uint32_t R = a.R, S = a.S;
     const uint64_t n_stages = (g1 - g0 + R - 1) / R;
@@ -1175,7 +1177,7 @@ __global__ void __launch_bounds__(256) k_scan_direct(Geom g, Work w, ScanArgs a)
     uint4 *pbuf = sm4 + 16;
     const uint32_t tid = threadIdx.x, bd = blockDim.x;
     const uint32_t nb = g.nb, T = g.threshold;
-    const uint64_t G = (uint64_t)g.n_slices * g.na * w.n_events;
+    const uint64_t G = (uint64_t)g.na * w.nu;
     const uint64_t g0 = G * blockIdx.x / gridDim.x, g1 = G * (blockIdx.x + 1) / gridDim.x;
     const uint32_t R = a.R;
     uint32_t buf_n = 0, nseq = 0, total = 0;
@@ -1424,7 +1426,7 @@ __device__ __forceinline__ void fill_scan_body(const Geom &g, const Work &w, con
 
     __shared__ unsigned long long s_rng[2];
     __shared__ uint32_t s_dyn;
-    const uint64_t items = (uint64_t)w.n_events * g.n_slices * c.strips;
+    const uint64_t items = (uint64_t)w.nu * c.strips, first = (uint64_t)w.u0 * c.strips;
     const uint64_t n_dyn = c.dyn ? dyn_items(items, gridDim.x) : 0, n_static = items - n_dyn;
     uint64_t it0, it1;
     cta_items(g, w, c, cta, gridDim.x, n_static, it0, it1, s_rng);
@@ -1478,7 +1480,7 @@ __device__ __forceinline__ void fill_scan_body(const Geom &g, const Work &w, con
             }
         }
     };
-    ItemCursor cur(g, c, it0);
+    ItemCursor cur(g, c, first + it0);
     for (uint64_t item = it0; item < it1; ++item, cur.next(g, c))
         do_item(cur);
     finish_candidates<BlockGroup>(w, a, ss, pbuf, buf_n, nseq, total, inner, cta);
@@ -1488,7 +1490,7 @@ __device__ __forceinline__ void fill_scan_body(const Geom &g, const Work &w, con
             const uint32_t list = gridDim.x + d;
             inner = interior_list(a, list);
             buf_n = nseq = total = 0;
-            do_item(ItemCursor(g, c, n_static + d));
+            do_item(ItemCursor(g, c, first + n_static + d));
             finish_candidates<BlockGroup>(w, a, ss, pbuf, buf_n, nseq, total, inner, list);
         }
     }
@@ -1578,11 +1580,10 @@ __global__ void __launch_bounds__(1024, 1) k_fill_ws(Geom g, Work w, FillCfg c, 
         // ---------------- vote group ----------------
         const uint32_t vr = VoteGroup::rank();
         uint64_t it0, it1;
-        cta_items<VoteGroup>(g, w, c, cta, gridDim.x, (uint64_t)w.n_events * g.n_slices * c.strips, it0, it1,
-                             s_rng[0]);
+        cta_items<VoteGroup>(g, w, c, cta, gridDim.x, (uint64_t)w.nu * c.strips, it0, it1, s_rng[0]);
         uint64_t cached_es = ~0ull;
         uint32_t cached_n = 0, p = 0;
-        ItemCursor cur(g, c, it0);
+        ItemCursor cur(g, c, (uint64_t)w.u0 * c.strips + it0);
         for (uint64_t item = it0; item < it1; ++item, cur.next(g, c)) {
             const ItemInfo t = item_info(g, w, c, cur);
             const uint32_t r = vr % t.rpass, hl = vr / t.rpass, hstride = VoteGroup::size() / t.rpass;
@@ -1610,12 +1611,11 @@ __global__ void __launch_bounds__(1024, 1) k_fill_ws(Geom g, Work w, FillCfg c, 
     // ---------------- flush + emit group ----------------
     const uint32_t fr = FlushGroup::rank();
     uint64_t it0, it1;
-    cta_items<FlushGroup>(g, w, c, cta, gridDim.x, (uint64_t)w.n_events * g.n_slices * c.strips, it0, it1,
-                          s_rng[1]);
+    cta_items<FlushGroup>(g, w, c, cta, gridDim.x, (uint64_t)w.nu * c.strips, it0, it1, s_rng[1]);
     const ChunkList inner = interior_list(a, cta);
     uint32_t buf_n = 0, nseq = 0, total = 0, p = 0;
     bool alive = true;
-    ItemCursor cur(g, c, it0);
+    ItemCursor cur(g, c, (uint64_t)w.u0 * c.strips + it0);
     for (uint64_t item = it0; item < it1 && alive; ++item, cur.next(g, c)) {
         const ItemInfo t = item_info(g, w, c, cur);
         const uint32_t slice_lin0 = t.s * g.na * nb;
@@ -1748,12 +1748,13 @@ __device__ void test_candidates(const Geom &g, const Work &w, const ScanArgs &a,
             const uint64_t gr = g0 + idx / nb;
             const uint32_t j = idx % nb;
             const uint32_t i = (uint32_t)(gr % g.na);
-            const uint32_t ev = (uint32_t)(gr / rows_ev);
+            const uint64_t row_all = gr + (uint64_t)w.u0 * g.na;   // of all matrices' rows
+            const uint32_t ev = (uint32_t)(row_all / rows_ev);
             const uint32_t *row = w.M + gr * nb;
             const uint32_t v = row[j];
             if (is_peak(row, i > 0 ? row - nb : nullptr, i + 1 < g.na ? row + nb : nullptr, j, nb, v)) {
                 has = 1;
-                ent = make_uint4((uint32_t)((gr - (uint64_t)ev * rows_ev) * nb) + j, ev, v, 0u);
+                ent = make_uint4((uint32_t)((row_all - (uint64_t)ev * rows_ev) * nb) + j, ev, v, 0u);
             }
         }
         if (__syncthreads_or(has)) {
@@ -1777,7 +1778,7 @@ __global__ void __launch_bounds__(256) k_scan_ldg(Geom g, Work w, ScanArgs a)
     uint4 *pbuf = sm4 + 16;
     const uint32_t tid = threadIdx.x, bd = blockDim.x;
     const uint32_t nb = g.nb, nb4 = nb >> 2, T = g.threshold;
-    const uint64_t G = (uint64_t)g.n_slices * g.na * w.n_events;
+    const uint64_t G = (uint64_t)g.na * w.nu;
     const uint64_t g0 = G * blockIdx.x / gridDim.x, g1 = G * (blockIdx.x + 1) / gridDim.x;
     const uint32_t RC = a.R;
     uint32_t buf_n = 0, nseq = 0, total = 0;

@@ -146,6 +146,7 @@ extern "C" ht_status ht_find_maxima_noalloc(const ht_binning *binning, const ht_
     uint32_t *ctr = reinterpret_cast<uint32_t *>(base + kOffCtr);
     htk::Work w{};
     w.n_events = n_events;
+    w.nu = n_events * g.n_slices;
     w.M = const_cast<uint32_t *>(M);   // read only
     w.n_cells = (uint64_t)g.n_slices * g.na * g.nb;
     w.status = ctr + htk::CTR_STATUS;
