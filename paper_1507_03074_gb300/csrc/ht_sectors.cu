@@ -31,6 +31,7 @@ struct ht_sectors {
     // capture cap_id): calls run in the order they are made, on whichever streams
     cudaEvent_t done = nullptr, cap_done = nullptr;
     bool done_pending = false;
+    unsigned long long done_id = 0;   // the stream's id (not its handle, which another stream may get)
     unsigned long long cap_id = 0;
     bool poisoned = false;
 };
@@ -80,15 +81,20 @@ ht_status in_order(ht_sectors *sec, cudaStream_t st, F call)
     unsigned long long id = 0;
     SCK(cudaStreamGetCaptureInfo(st, &cs, &id));
     const bool captured = cs != cudaStreamCaptureStatusNone;
-    if (captured ? sec->cap_id == id : sec->done_pending)
-        SCK(cudaStreamWaitEvent(st, captured ? sec->cap_done : sec->done, 0));
+    if (captured) {
+        if (sec->cap_id == id)
+            SCK(cudaStreamWaitEvent(st, sec->cap_done, 0));
+    } else {
+        SCK(cudaStreamGetId(st, &id));
+        if (sec->done_pending && sec->done_id != id)
+            SCK(cudaStreamWaitEvent(st, sec->done, 0));
+    }
     const ht_status s = pass_on(sec, call());
     if (sec->poisoned)
         return s;
     SCK(cudaEventRecord(captured ? sec->cap_done : sec->done, st));
-    if (captured)
-        sec->cap_id = id;
-    else
+    (captured ? sec->cap_id : sec->done_id) = id;
+    if (!captured)
         sec->done_pending = true;
     return s;
 }
