@@ -92,8 +92,8 @@ static cudaError_t enqueue_compute(Runner &R, uint32_t n_events, uint32_t n_hits
     Engine &E = R.E;
     const uint32_t mh = E.max_hits;
     // offsets clamped to the staging size; n_total = max_hits: nothing the
-    // kernels take as arguments depends on the run; n_hits only chooses whether
-    // k_edges follows the fill (part of the graph's key)
+    // kernels take as arguments depends on the run; n_hits only chooses the
+    // fill's launch (engine_fill_kind, part of the graph's key)
     cudaError_t e = engine_fill(E, R.d_xyz, R.d_xyz + mh, R.d_xyz + 2 * (size_t)mh, R.d_off, mh, n_events, mh,
                                 fill_flags, st, n_hits);
     if (e != cudaSuccess)
@@ -109,9 +109,9 @@ static cudaError_t run_compute(Runner &R, uint32_t n_events, uint32_t n_hits, bo
 {
     if (R.E.prof.on || !R.graphs_ok)
         return enqueue_compute(R, n_events, n_hits, to_host, fill_flags, st);
-    const bool edges = engine_edges_later(R.E, n_hits, n_events, fill_flags);
+    const uint32_t how = engine_fill_kind(R.E, n_hits, n_events, fill_flags);
     for (auto &g : R.graphs)
-        if (g.n_events == n_events && g.to_host == to_host && g.fill_flags == fill_flags && g.edges == edges)
+        if (g.n_events == n_events && g.to_host == to_host && g.fill_flags == fill_flags && g.how == how)
             return cudaGraphLaunch(g.exec, st);
     cudaError_t e = enqueue_compute(R, n_events, n_hits, to_host, fill_flags, st);
     if (e != cudaSuccess)
@@ -139,7 +139,7 @@ static cudaError_t run_compute(Runner &R, uint32_t n_events, uint32_t n_hits, bo
         cudaGraphExecDestroy(R.graphs.front().exec);
         R.graphs.erase(R.graphs.begin());
     }
-    R.graphs.push_back({n_events, to_host, fill_flags, edges, exec});
+    R.graphs.push_back({n_events, to_host, fill_flags, how, exec});
     return cudaSuccess;
 }
 

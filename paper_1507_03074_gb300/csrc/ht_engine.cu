@@ -399,7 +399,13 @@ ht_status engine_configure(Engine &E, std::string *why)
                             E.po_ok ? htk::tile_passes(g, E.po_tile, E.max_events) : 0);
     // segments of the passes' peaks (a CTA of k_edges and k_order_passes each):
     // enough to fill the GPU, few enough for each CTA to add up those before it
+    // (smaller ones where few passes hold many peaks: 16 slices of 16 x 1024 bins with
+    // 256 hits each, threshold 3: 29.6 -> 24.2 us)
+    const double per_pass = (double)std::max<uint32_t>(E.max_hits, 1) * E.max_admit * g.na / E.threshold /
+                            std::max<uint64_t>(E.max_passes, 1);   // peaks at most
     E.seg_shift = 5;
+    while (E.seg_shift > 0 && per_pass * (1u << E.seg_shift) > 4.0 * htk::kOrderPasses)
+        --E.seg_shift;
     while ((2u << E.seg_shift) <= htk::kOrderPasses && (E.max_passes >> E.seg_shift) > (uint64_t)E.num_sms)
         ++E.seg_shift;
     // the fused fill's candidate lists: one per CTA plus one per handed-out item
@@ -739,10 +745,34 @@ static VoteKind vote_kind(const Engine &E, uint32_t flags)
     return E.use_tma && !E.use_ws ? TILES_MH : OTHER_FILL;
 }
 
-bool engine_edges_later(const Engine &E, uint32_t n_hits, uint32_t n_events, uint32_t flags)
+uint32_t engine_fill_kind(const Engine &E, uint32_t n_hits, uint32_t n_events, uint32_t flags)
 {
-    return vote_kind(E, flags) == TILES_MH &&
-           (double)n_hits * E.max_admit >= (double)htk::kEdgeHits * E.geom.n_slices * n_events;
+    const VoteKind kind = vote_kind(E, flags);
+    if (kind != TILES_MH && kind != TILES_PEAKS)
+        return 0;
+    const htk::TileCfg &c = kind == TILES_MH ? E.tile : E.po_tile;
+    const double per_unit = (double)n_hits * E.max_admit / ((double)E.geom.n_slices * n_events);   // at most, on average
+    const double warps = (double)c.warps * (kind == TILES_MH ? E.tma_grid : E.po_grid);
+    const double passes = (double)htk::tile_passes(E.geom, c, n_events), cells = (double)E.n_cells * n_events;
+    const bool crowded = per_unit >= htk::kEdgeHits && c.strips > 1;
+    // Whole CTAs may vote passes: where the passes, of many hits each, are fewer
+    // than the warps (the event of 4 slices of 16 x 1024 bins with 4096 hits each
+    // that takes 43 us took 161 us without; close to as many passes, of 1024 hits,
+    // lose: 64 slices of 128 x 64 bins 92 against 73 us); where an SM has few tile
+    // warps, as rows are wide, and the hits are very many; and where most hits may
+    // be in one slice whose passes then outlast the rest: a warp takes about 1 ns per
+    // hit and row, the matrix 1 ns per 1750 cells (42936 hits in one of 96 slices of
+    // 1456 x 93 bins, 3453 us without).  Below 150 us of such votes the larger CTAs
+    // cost more than they save (3131 even hits in 102 slices of 219 x 427 bins: 25.0
+    // against 21.0 us).  Peaks-only fills of crowded slices take the same kernel for
+    // its search, which loads the lines of the rows beyond ahead.
+    const bool many = per_unit >= htk::kTeamHits, very = per_unit >= 4.0 * htk::kTeamHits;
+    const bool few = (many && passes * 2.0 < warps) || (very && passes < warps);
+    const bool wide = very && c.warps <= 4u;
+    const bool one = (double)n_hits * c.W > std::max(1.5e5, cells / 1750.0);
+    const bool teams = few || wide || one || (kind == TILES_PEAKS && many);
+    return (kind == TILES_MH && crowded ? kEdgesLater : 0u) | (teams ? kTeams : 0u) | (few ? kTeamsFew : 0u) |
+           (wide ? kTeamsAll : 0u);
 }
 
 cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *z,
@@ -846,13 +876,19 @@ cudaError_t engine_vote(Engine &E, const uint32_t *d_hit_off, uint32_t n_hits0, 
     if (kind != OTHER_FILL) {
         const bool store = kind == TILES_MH;
         htk::TileCfg c = store ? E.tile : E.po_tile;
-        c.edges_later = engine_edges_later(E, E.binned, n_events, flags);
+        const uint32_t how = engine_fill_kind(E, E.binned, n_events, flags);
+        c.edges_later = how & kEdgesLater;
         const uint64_t passes = htk::tile_passes(E.geom, c, n_events);
-        const uint32_t grid = (uint32_t)std::max<uint64_t>(
-            1, std::min<uint64_t>(store ? E.tma_grid : E.po_grid, (passes + c.warps - 1) / c.warps));
+        uint64_t grid = std::min<uint64_t>(store ? E.tma_grid : E.po_grid, (passes + c.warps - 1) / c.warps);
+        if (how & kTeams) {   // a CTA for every pass
+            // their passes: of all that is voted more than one warp's share, or twice
+            // that of a tile warp where there are plenty of passes, or any
+            c.team_share = how & kTeamsAll ? 1u << 20 : how & kTeamsFew ? htk::kTileWarps : std::max(1u, c.warps / 2u);
+            grid = std::min<uint64_t>({store ? E.tma_grid : E.po_grid, passes, 2u * (uint64_t)E.num_sms});
+        }
         {
             ProfScope ps(E, store ? K_FILL_TMA : K_FILL_PEAKS, st);
-            e = htk::launch_fill_tma(E.geom, w, c, E.scan, grid, store, st);
+            e = htk::launch_fill_tma(E.geom, w, c, E.scan, (uint32_t)std::max<uint64_t>(grid, 1), store, st);
         }
         ++E.launches;
         if (e == cudaSuccess && c.edges_later) {

@@ -159,15 +159,19 @@ ht_status engine_configure(Engine &E, std::string *why);
 // d_hit_off (device, n_events + 1) or nullptr for one event of n_hits0 hits.
 // n_total (host) is the total hit count; it sizes the binning grid.  Where it is
 // only a bound (a graph that serves several runs), n_known is this run's count:
-// with it the tile fill decides on k_edges (engine_edges_later).  Unless
+// with it the tile fill chooses its launch (engine_fill_kind).  Unless
 // HT_ACCUMULATE or HT_FILL_NAIVE is set (or the tuning turns it off), the
 // fused kernel also finds the peaks, which engine_scan then only orders.
 cudaError_t engine_fill(Engine &E, const float *x, const float *y, const float *z,
                         const uint32_t *d_hit_off, uint32_t n_hits0, uint32_t n_events,
                         uint32_t n_total, uint32_t flags, cudaStream_t st, uint32_t n_known = ~0u);
 
-// Whether a fill of n_hits hits leaves the comparisons across passes to k_edges.
-bool engine_edges_later(const Engine &E, uint32_t n_hits, uint32_t n_events, uint32_t flags);
+// What a tile fill's launch takes from the number of hits: kEdgesLater: the
+// comparisons across passes are left to k_edges; kTeams: whole CTAs vote the
+// passes of crowded units; kTeamsFew: as there are few passes; kTeamsAll: even
+// where there are plenty.
+enum : uint32_t { kEdgesLater = 1, kTeams = 2, kTeamsFew = 4, kTeamsAll = 8 };
+uint32_t engine_fill_kind(const Engine &E, uint32_t n_hits, uint32_t n_events, uint32_t flags);
 
 // M_H to dst, device memory: the GPU's own, 32-byte aligned, by a kernel, else by
 // cudaMemcpyAsync.

@@ -36,6 +36,9 @@ struct TileCfg {
     uint32_t run;         // neighbouring passes of a CTA's run (= warps)
     uint32_t threads;     // the tuning's fill_threads (at least 32 * warps)
     uint32_t vote_agg;    // warp-aggregated vote increments (match.any + one add)
+    // > 0: CTAs of kTileWarps warps, which together vote the passes of crowded
+    // units (team_passes): those that are more than 1 / (team_share * CTAs) of all
+    uint32_t team_share;
     uint32_t edges_later; // tiles that go to M_H: comparisons across passes are left to k_edges
 };
 constexpr uint32_t kTileWarps = 12;    // most warps of a tile-fill CTA (two such CTAs per SM: 80 registers a thread)
@@ -45,6 +48,10 @@ constexpr uint32_t kTileWarps = 12;    // most warps of a tile-fill CTA (two suc
 constexpr uint32_t kTileMinWarps = 6;
 constexpr uint32_t kTileCand = 127;    // cells >= T that a pass lists (more: every cell is looked at)
 constexpr uint32_t kAhead = 4;         // lines per lane loaded ahead
+// Fewest hits of a unit whose passes whole CTAs may take: at 192 units of 256 hits
+// lose by it (64 slices of 128 x 1024 bins, threshold 10: 53.7 us against 33.0 us).
+constexpr uint32_t kTeamHits = 512;
+constexpr uint32_t kListHits = 128;    // most hits of a pass that searches its list without a look at the cost
 constexpr uint32_t kHandedOut = 3;     // passes per warp handed out at run time (at least)
 // words of a warp's bits (one per tile cell), of its list (the length and the cells), and of all its shared memory
 __host__ __device__ constexpr uint32_t tile_bit_words(uint32_t tile_words) { return (tile_words / 32u + 4u) & ~3u; }
@@ -170,7 +177,7 @@ size_t scan_smem_bytes(const ScanArgs &a);
 // [6, 6 + n_events) before every fill.
 enum : uint32_t {
     CTR_STATUS = 0, CTR_ENTRIES = 1, CTR_OTICKET = 2, CTR_BTICKET = 3, CTR_DYN = 4, CTR_DYN_DONE = 5,
-    CTR_P4TICKET = 6, CTR_EVENTS = 7
+    CTR_P4TICKET = 6, CTR_TEAM = 7, CTR_EVENTS = 8
 };
 
 // Cost model of the balanced split of (event, slice, strip) work items over

@@ -2055,7 +2055,32 @@ __device__ __forceinline__ void line_bins(const Geom &g, const float2 l, const f
     }
 }
 
-// The votes of a pass into its tile (l: the first 32 * kAhead lines; the next
+// Who works on a pass: a warp (the rule), or all warps of the CTA (team_passes).
+struct WarpCrew {
+    static __device__ __forceinline__ uint32_t rank() { return threadIdx.x & 31u; }
+    static __device__ __forceinline__ uint32_t size() { return 32u; }
+    static __device__ __forceinline__ uint32_t warp() { return 0u; }
+    static __device__ __forceinline__ uint32_t warps() { return 1u; }
+    static __device__ __forceinline__ void sync() { __syncwarp(); }
+};
+struct CtaCrew {
+    static __device__ __forceinline__ uint32_t rank() { return threadIdx.x; }
+    static __device__ __forceinline__ uint32_t size() { return blockDim.x; }
+    static __device__ __forceinline__ uint32_t warp() { return threadIdx.x >> 5; }
+    static __device__ __forceinline__ uint32_t warps() { return blockDim.x >> 5; }
+    static __device__ __forceinline__ void sync() { __syncthreads(); }
+};
+
+// The first 32 * kAhead lines of this warp's share of a pass's n: groups of 32 *
+// kAhead go to the crew's warps in turn.
+template <class C>
+__device__ __forceinline__ void crew_lines(float2 (&l)[kAhead], const float2 *lines, uint32_t n)
+{
+    const uint32_t h = C::warp() * 32u * kAhead;
+    first_lines(l, lines + h, n > h ? n - h : 0u);
+}
+
+// The votes of a pass into its tile (l: crew_lines; the next
 // ones are loaded that far ahead): R rows at a time, a lane holds one hit's
 // line; consecutive lanes hold consecutive hits, whose B columns, and so whose
 // banks, differ.  A vote that lifts its cell from T - 1 to T lists the cell.
@@ -2065,14 +2090,14 @@ __device__ __forceinline__ void line_bins(const Geom &g, const float2 l, const f
 // warp-aggregated increments -- the lanes voting for the same cell find each
 // other (match.any) and their lowest lane adds their number with one atomic;
 // the cell is listed by the add that takes it from below T to T or more.
-template <bool AGG, int R>
+template <bool AGG, int R, class C>
 __device__ __forceinline__ void vote_tile(const Geom &g, uint32_t *tile, const TilePass &P, float2 (&l)[kAhead],
                                           PassList &L, uint32_t spare)
 {
     const uint32_t nb = g.nb, T = g.threshold, lane = threadIdx.x & 31u;
     for (uint32_t r0 = 0; r0 < P.pr; r0 += R) {
         if (r0)
-            first_lines(l, P.lines, P.nc);
+            crew_lines<C>(l, P.lines, P.nc);
         float x[R];
         uint32_t row[R], most[R];   // per row: its first cell, less 1; the largest bin, plus 1 (0 beyond the pass)
 #pragma unroll
@@ -2114,9 +2139,10 @@ __device__ __forceinline__ void vote_tile(const Geom &g, uint32_t *tile, const T
                     }
             }
         };
-        for (uint32_t h0 = 0; h0 < P.nc; h0 += 32u * kAhead) {
+        const uint32_t step = C::warps() * 32u * kAhead;
+        for (uint32_t h0 = C::warp() * 32u * kAhead; h0 < P.nc; h0 += step) {
             float2 ahead[kAhead];
-            const uint32_t h1 = h0 + 32u * kAhead;
+            const uint32_t h1 = h0 + step;
             first_lines(ahead, P.lines + h1, P.nc > h1 ? P.nc - h1 : 0u);
 #pragma unroll
             for (uint32_t k = 0; k < kAhead; ++k) {
@@ -2128,41 +2154,87 @@ __device__ __forceinline__ void vote_tile(const Geom &g, uint32_t *tile, const T
     }
 }
 
-// The votes of A row i into row[0 .. n_b), by one warp.
+// The votes of A row i into row[0 .. n_b).  AHEAD: with kAhead lines per thread
+// loaded ahead (for units of many hits).
+template <class C, bool AHEAD>
 __device__ __forceinline__ void vote_row(const Geom &g, uint32_t *row, const TilePass &P, uint32_t i)
 {
-    __syncwarp();
-    for (uint32_t h = threadIdx.x & 31u; h < P.nc; h += 32u) {
-        const uint32_t j = vote_bin_line(g, __ldg(P.lines + h), i, P.recs + h);
-        if (j < g.nb)
-            atomicAdd(&row[j], 1u);
+    C::sync();
+    if (!AHEAD) {
+        for (uint32_t h = C::rank(); h < P.nc; h += C::size()) {
+            const uint32_t j = vote_bin_line(g, __ldg(P.lines + h), i, P.recs + h);
+            if (j < g.nb)
+                atomicAdd(&row[j], 1u);
+        }
+        C::sync();
+        return;
     }
-    __syncwarp();
+    const uint32_t step = C::size() * kAhead;
+    auto load = [&](float2 (&l)[kAhead], uint32_t h0) {
+#pragma unroll
+        for (uint32_t k = 0; k < kAhead; ++k)
+            l[k] = h0 + k * C::size() < P.nc ? __ldg(P.lines + h0 + k * C::size()) : no_line();
+    };
+    float2 l[kAhead];
+    load(l, C::rank());
+    for (uint32_t h0 = C::rank(); h0 < P.nc; h0 += step) {
+        float2 ahead[kAhead];
+        load(ahead, h0 + step);
+#pragma unroll
+        for (uint32_t k = 0; k < kAhead; ++k) {
+            const uint32_t h = h0 + k * C::size();
+            const uint32_t j = vote_bin_line(g, l[k], i, P.recs + h, h < P.nc);
+            if (j < g.nb)
+                atomicAdd(&row[j], 1u);
+            l[k] = ahead[k];
+        }
+    }
+    C::sync();
 }
 
-// The peaks of pass number `pass` (the warp's own tile and list; bits: one bit
-// per cell of the tile, zero between calls).  reading: a bulk copy may still
-// read the tile.  edges_later: the rows beyond the pass are left to k_edges.
-// Every lane calls it.
-__device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const ScanArgs &a, const TilePass &P,
-                                         uint32_t pass, uint32_t unit, uint32_t *tile, const PassList &L,
-                                         uint32_t *bits, bool reading, bool edges_later)
+// The votes of the rows before (above) and behind (below) a pass into row[0 .. n_b)
+// and row[n_b .. 2 n_b).
+template <class C>
+__device__ __forceinline__ void vote_rows_beyond(const Geom &g, uint32_t *row, const TilePass &P, bool above, bool below)
 {
-    const uint32_t lane = threadIdx.x & 31u, nb = g.nb, n_c = L.n, full = 0xffffffffu, pr = P.pr;
-    const uint32_t e = unit / g.n_slices, s = unit - e * g.n_slices;
-    const uint32_t lin0 = (s * g.na + P.iA) * nb, last = (pr - 1u) * nb;
-    // the pass has a row of the slice before / behind it, which this kernel compares with
-    const bool above = !edges_later && P.iA > 0, below = !edges_later && P.iA + pr < g.na;
-    // the test against the neighbours inside the tile
-    auto inner = [&](uint32_t key, uint32_t v) {
-        const uint32_t r = key / nb, j = key - r * nb;
-        const uint32_t *row = tile + r * nb;
-        return is_peak(row, r > 0 ? row - nb : nullptr, r + 1 < pr ? row + nb : nullptr, j, nb, v);
+    const uint32_t step = C::size() * kAhead, nb = g.nb;
+    const float x[2] = {__int2float_rn((int)P.iA - 1 - g.mid), __int2float_rn((int)(P.iA + P.pr) - g.mid)};
+    auto load = [&](float2 (&l)[kAhead], uint32_t h0) {
+#pragma unroll
+        for (uint32_t k = 0; k < kAhead; ++k)
+            l[k] = h0 + k * C::size() < P.nc ? __ldg(P.lines + h0 + k * C::size()) : no_line();
     };
-    // room for n entries, and the pass's counts
-    auto claim = [&](uint32_t n) {
+    float2 l[kAhead];
+    load(l, C::rank());
+    for (uint32_t h0 = C::rank(); h0 < P.nc; h0 += step) {
+        float2 ahead[kAhead];
+        load(ahead, h0 + step);
+#pragma unroll
+        for (uint32_t k = 0; k < kAhead; ++k) {
+            const uint32_t h = h0 + k * C::size();
+            const float x0[1] = {x[0]}, x1[1] = {x[1]};
+            uint32_t j0[1], j1[1];
+            line_bins<1>(g, l[k], x0, P.iA - 1u, P.recs + h, above && h < P.nc, j0);
+            line_bins<1>(g, l[k], x1, P.iA + P.pr, P.recs + h, below && h < P.nc, j1);
+            if (above && j0[0] - 1u < nb)
+                atomicAdd(&row[j0[0] - 1u], 1u);
+            if (below && j1[0] - 1u < nb)
+                atomicAdd(&row[nb + j1[0] - 1u], 1u);
+            l[k] = ahead[k];
+        }
+    }
+    C::sync();
+}
+
+// Where a pass's peaks go: the pass and segment counts, and the entries.
+struct PassOut {
+    uint32_t e, lin0;   // event, linear index of the pass's first cell
+    uint32_t pass;
+    // room for n entries; a warp calls it
+    __device__ __forceinline__ uint32_t claim(const Work &w, const ScanArgs &a, uint32_t n) const
+    {
         uint32_t base = 0;
-        if (lane == 0) {
+        if ((threadIdx.x & 31u) == 0) {
             if (n) {
                 base = atomicAdd(a.g_count, n);
                 atomicAdd(&w.seg_peaks[pass >> w.seg_shift], n);
@@ -2172,137 +2244,335 @@ __device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const 
             }
             w.pass_peaks[pass] = make_uint2(base, n);
         }
-        return __shfl_sync(full, base, 0);
-    };
-    auto put = [&](uint32_t at, uint32_t key, uint32_t v) {
+        return __shfl_sync(0xffffffffu, base, 0);
+    }
+    __device__ __forceinline__ void put(const ScanArgs &a, uint32_t at, uint32_t key, uint32_t v) const
+    {
         if (at < a.entries_cap)
             a.entries[at] = make_uint4(lin0 + key, e, v, 0u);
-    };
-    // many peaks: a bit per cell that is one, then the bits in order
-    const uint32_t cells = pr * nb, words = (cells + 31u) / 32u;
-    auto put_bits = [&]() {
-        __syncwarp();
-        uint32_t n = 0;
-        for (uint32_t q = lane; q < words; q += 32u)
-            n += (uint32_t)__popc(bits[q]);
-        uint32_t base = claim(__reduce_add_sync(full, n));
-        for (uint32_t q0 = 0; q0 < words; q0 += 32u) {
-            const uint32_t q = q0 + lane;
-            uint32_t m = q < words ? bits[q] : 0u;
-            if (q < words)
-                bits[q] = 0u;
-            const uint32_t c = (uint32_t)__popc(m), incl = warp_incl_scan(c);
-            for (uint32_t at = base + incl - c; m; m &= m - 1u, ++at) {
-                const uint32_t key = 32u * q + (uint32_t)(__ffs(m) - 1);
-                put(at, key, tile[key]);
-            }
-            base += __shfl_sync(full, incl, 31);
-        }
-        __syncwarp();
-    };
-    if (n_c <= kTileCand) {   // one listed cell per lane
-        // the three cells of row i next to the cells j of the lanes in m, counted
-        // hit by hit: the most votes one of them holds, for each lane in m
-        auto beyond = [&](uint32_t m, uint32_t i, uint32_t j) {
-            uint32_t c0 = 0, c1 = 0, c2 = 0;
-            const float x[1] = {__int2float_rn((int)i - g.mid)};
-            float2 l = lane < P.nc ? __ldg(P.lines + lane) : no_line();
-            for (uint32_t h0 = 0; h0 < P.nc; h0 += 32u) {
-                const uint32_t h = h0 + lane;
-                uint32_t b[1];
-                line_bins<1>(g, l, x, i, P.recs + h, h < P.nc, b);
-                const uint32_t j1 = b[0] - 1u < nb ? b[0] : 0x80000000u;   // no cell is next to that
-                l = h + 32u < P.nc ? __ldg(P.lines + h + 32u) : no_line();
-                for (uint32_t k = m; k; k &= k - 1u) {
-                    const uint32_t src = (uint32_t)(__ffs(k) - 1);
-                    const uint32_t d = j1 - __shfl_sync(full, j, src);
-                    const uint32_t b0 = __ballot_sync(full, d == 0u), b1 = __ballot_sync(full, d == 1u),
-                                   b2 = __ballot_sync(full, d == 2u);
-                    if (lane == src) {
-                        c0 += (uint32_t)__popc(b0);
-                        c1 += (uint32_t)__popc(b1);
-                        c2 += (uint32_t)__popc(b2);
-                    }
-                }
-            }
-            return max(c1, max(c0, c2));
-        };
-        for (uint32_t k0 = 0; k0 < n_c; k0 += 32u) {
-            const bool has = k0 + lane < n_c;
-            const uint32_t key = has ? L.cand[k0 + lane] : ~0u;
-            const uint32_t v = has ? tile[key] : 0u;
-            bool keep = has && inner(key, v);
-            uint32_t m = __ballot_sync(full, keep && above && key < nb);
-            if (m) {
-                const uint32_t most = beyond(m, P.iA - 1u, key);
-                if ((m >> lane) & 1u)
-                    keep = v > most;
-            }
-            m = __ballot_sync(full, keep && below && key >= last);
-            if (m) {
-                const uint32_t most = beyond(m, P.iA + pr, key - last);
-                if ((m >> lane) & 1u)
-                    keep = v >= most;
-            }
-            if (n_c > 32u) {
-                if (keep)
-                    atomicOr(&bits[key >> 5], 1u << (key & 31u));
-                continue;
-            }
-            m = __ballot_sync(full, keep);
-            uint32_t rank = 0;
-            const uint32_t n = (uint32_t)__popc(m);
-            for (; m; m &= m - 1u)
-                rank += __shfl_sync(full, key, __ffs(m) - 1) < key;
-            const uint32_t base = claim(n);
-            if (keep)
-                put(base + rank, key, v);
-        }
-        if (n_c > 32u)
-            put_bits();
-        return;
     }
-    // more than the list holds: every cell is looked at
-    for (uint32_t q = 0; q < words; ++q) {
+};
+
+// The test of cell `key` of a tile of pr rows against its neighbours in the tile.
+__device__ __forceinline__ bool peak_in_tile(const uint32_t *tile, uint32_t pr, uint32_t nb, uint32_t key, uint32_t v)
+{
+    const uint32_t r = key / nb, j = key - r * nb;
+    const uint32_t *row = tile + r * nb;
+    return is_peak(row, r > 0 ? row - nb : nullptr, r + 1 < pr ? row + nb : nullptr, j, nb, v);
+}
+
+// Many peaks: the cells that are peaks, a bit each (cleared), go out in order.
+// One warp calls it.
+__device__ __forceinline__ void put_bits(const Work &w, const ScanArgs &a, const PassOut &O, const uint32_t *tile,
+                                         uint32_t *bits, uint32_t words)
+{
+    const uint32_t lane = threadIdx.x & 31u, full = 0xffffffffu;
+    __syncwarp();
+    uint32_t n = 0;
+    for (uint32_t q = lane; q < words; q += 32u)
+        n += (uint32_t)__popc(bits[q]);
+    uint32_t base = O.claim(w, a, __reduce_add_sync(full, n));
+    for (uint32_t q0 = 0; q0 < words; q0 += 32u) {
+        const uint32_t q = q0 + lane;
+        uint32_t m = q < words ? bits[q] : 0u;
+        if (q < words)
+            bits[q] = 0u;
+        const uint32_t c = (uint32_t)__popc(m), incl = warp_incl_scan(c);
+        for (uint32_t at = base + incl - c; m; m &= m - 1u, ++at) {
+            const uint32_t key = 32u * q + (uint32_t)(__ffs(m) - 1);
+            O.put(a, at, key, tile[key]);
+        }
+        base += __shfl_sync(full, incl, 31);
+    }
+    __syncwarp();
+}
+
+// The peaks of a pass by a look at every cell of its tile (bits: one bit per cell,
+// zero between calls).  above, below: the pass has a row before, behind it that
+// its first, last row is compared with: that row is voted into a row of the tile
+// which the test does not need (the tile holds at least two), and that row is
+// voted anew after it; with rows to spare (scratch: two rows, zero between calls)
+// both are voted there, in one go.  reading: a bulk copy of the crew's first
+// thread may still read the tile.
+template <class C, bool AHEAD>
+__device__ __forceinline__ void search_cells(const Geom &g, const Work &w, const ScanArgs &a, const TilePass &P,
+                                             const PassOut &O, uint32_t *tile, uint32_t *bits, bool above, bool below,
+                                             bool reading, uint32_t *scratch)
+{
+    const uint32_t lane = threadIdx.x & 31u, nb = g.nb, pr = P.pr, last = (pr - 1u) * nb;
+    const uint32_t cells = pr * nb, words = (cells + 31u) / 32u;
+    for (uint32_t q = C::warp(); q < words; q += C::warps()) {
         const uint32_t key = 32u * q + lane;
         const uint32_t v = key < cells ? tile[key] : 0u;
-        const uint32_t m = __ballot_sync(full, v >= g.threshold && inner(key, v));
+        const uint32_t m = __ballot_sync(0xffffffffu, v >= g.threshold && peak_in_tile(tile, pr, nb, key, v));
         if (lane == 0)
             bits[q] = m;
     }
-    // the rows beyond, each voted into a row of the tile that the test does
-    // not need (the tile holds at least two rows), which is voted anew after it
-    if ((above || below) && reading) {
-        if (lane == 0)
-            bulk_wait_read<0>();
-        __syncwarp();
-    }
-    auto beyond = [&](uint32_t i, uint32_t key0, uint32_t spare, bool before) {
-        uint32_t *row = tile + spare * nb;
-        auto clear = [&]() {
-            __syncwarp();
-            for (uint32_t j = lane; j < nb; j += 32u)
-                row[j] = 0u;
-        };
-        clear();
-        vote_row(g, row, P, i);
-        for (uint32_t j = lane; j < nb; j += 32u) {
+    if ((above || below) && !scratch && reading && C::rank() == 0)
+        bulk_wait_read<0>();
+    C::sync();
+    // drop the peaks of a row (its first cell: key0) that the row beyond outdoes
+    auto compare = [&](const uint32_t *row, uint32_t key0, bool before) {
+        for (uint32_t j = C::rank(); j < nb; j += C::size()) {
             const uint32_t key = key0 + j, b = 1u << (key & 31u);
             const uint32_t most = max(row[j], max(j ? row[j - 1] : 0u, j + 1 < nb ? row[j + 1] : 0u));
             if ((bits[key >> 5] & b) && !(before ? tile[key] > most : tile[key] >= most))
                 atomicAnd(&bits[key >> 5], ~b);
         }
+    };
+    if (scratch) {
+        if (above || below) {
+            vote_rows_beyond<C>(g, scratch, P, above, below);
+            if (above)
+                compare(scratch, 0u, true);
+            if (below)
+                compare(scratch + nb, last, false);
+            C::sync();
+            for (uint32_t j = C::rank(); j < 2u * nb; j += C::size())
+                scratch[j] = 0u;
+        }
+        if (C::warp() == 0)
+            put_bits(w, a, O, tile, bits, words);
+        C::sync();
+        return;
+    }
+    auto beyond = [&](uint32_t i, uint32_t key0, uint32_t spare, bool before) {
+        uint32_t *row = tile + spare * nb;
+        auto clear = [&]() {
+            C::sync();
+            for (uint32_t j = C::rank(); j < nb; j += C::size())
+                row[j] = 0u;
+        };
+        clear();
+        vote_row<C, AHEAD>(g, row, P, i);
+        compare(row, key0, before);
         clear();
         if (spare < pr)
-            vote_row(g, row, P, P.iA + spare);
-        __syncwarp();
+            vote_row<C, AHEAD>(g, row, P, P.iA + spare);
+        C::sync();
     };
-    __syncwarp();
     if (above)
         beyond(P.iA - 1u, 0u, 1u, true);
     if (below)
         beyond(P.iA + pr, last, pr > 1u ? 0u : 1u, false);
-    put_bits();
+    if (C::warp() == 0)
+        put_bits(w, a, O, tile, bits, words);
+    C::sync();
+}
+
+// The peaks of a warp's pass (its own tile and list; bits as search_cells).
+// reading: a bulk copy may still read the tile.  edges_later: the rows beyond the
+// pass are left to k_edges.  MANY: units may hold many hits.  Every lane calls it.
+template <bool MANY>
+__device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const ScanArgs &a, const TilePass &P,
+                                            const PassOut &O, uint32_t *tile, const PassList &L, uint32_t *bits,
+                                            bool reading, bool edges_later)
+{
+    const uint32_t lane = threadIdx.x & 31u, nb = g.nb, n_c = L.n, full = 0xffffffffu, pr = P.pr;
+    const uint32_t last = (pr - 1u) * nb;
+    const uint32_t cells = pr * nb, words = (cells + 31u) / 32u;
+    // the pass has a row of the slice before / behind it, which this kernel compares with
+    const bool above = !edges_later && P.iA > 0, below = !edges_later && P.iA + pr < g.na;
+    bool list = n_c <= kTileCand;
+    if (MANY && list && P.nc > kListHits && (above || below)) {
+        // many hits: counting them for every listed cell of the first and last row
+        // against voting the rows beyond and looking at every cell
+        uint32_t edge = 0;
+        for (uint32_t k = lane; k < n_c; k += 32u)
+            edge += (above && L.cand[k] < nb) + (below && L.cand[k] >= last);
+        edge = __reduce_add_sync(full, edge);
+        list = (uint64_t)edge * P.nc <= 8u * P.nc + 64u * words;
+    }
+    if (!list) {
+        search_cells<WarpCrew, MANY>(g, w, a, P, O, tile, bits, above, below, reading, nullptr);
+        return;
+    }
+    // one listed cell per lane;
+    // the three cells of row i next to the cells j of the lanes in m, counted
+    // hit by hit: the most votes one of them holds, for each lane in m
+    auto beyond = [&](uint32_t m, uint32_t i, uint32_t j) {
+        uint32_t c0 = 0, c1 = 0, c2 = 0;
+        const float x[1] = {__int2float_rn((int)i - g.mid)};
+        float2 l = lane < P.nc ? __ldg(P.lines + lane) : no_line();
+        for (uint32_t h0 = 0; h0 < P.nc; h0 += 32u) {
+            const uint32_t h = h0 + lane;
+            uint32_t b[1];
+            line_bins<1>(g, l, x, i, P.recs + h, h < P.nc, b);
+            const uint32_t j1 = b[0] - 1u < nb ? b[0] : 0x80000000u;   // no cell is next to that
+            l = h + 32u < P.nc ? __ldg(P.lines + h + 32u) : no_line();
+            for (uint32_t k = m; k; k &= k - 1u) {
+                const uint32_t src = (uint32_t)(__ffs(k) - 1);
+                const uint32_t d = j1 - __shfl_sync(full, j, src);
+                const uint32_t b0 = __ballot_sync(full, d == 0u), b1 = __ballot_sync(full, d == 1u),
+                               b2 = __ballot_sync(full, d == 2u);
+                if (lane == src) {
+                    c0 += (uint32_t)__popc(b0);
+                    c1 += (uint32_t)__popc(b1);
+                    c2 += (uint32_t)__popc(b2);
+                }
+            }
+        }
+        return max(c1, max(c0, c2));
+    };
+    for (uint32_t k0 = 0; k0 < n_c; k0 += 32u) {
+        const bool has = k0 + lane < n_c;
+        const uint32_t key = has ? L.cand[k0 + lane] : ~0u;
+        const uint32_t v = has ? tile[key] : 0u;
+        bool keep = has && peak_in_tile(tile, pr, nb, key, v);
+        uint32_t m = __ballot_sync(full, keep && above && key < nb);
+        if (m) {
+            const uint32_t most = beyond(m, P.iA - 1u, key);
+            if ((m >> lane) & 1u)
+                keep = v > most;
+        }
+        m = __ballot_sync(full, keep && below && key >= last);
+        if (m) {
+            const uint32_t most = beyond(m, P.iA + pr, key - last);
+            if ((m >> lane) & 1u)
+                keep = v >= most;
+        }
+        if (n_c > 32u) {
+            if (keep)
+                atomicOr(&bits[key >> 5], 1u << (key & 31u));
+            continue;
+        }
+        m = __ballot_sync(full, keep);
+        uint32_t rank = 0;
+        const uint32_t n = (uint32_t)__popc(m);
+        for (; m; m &= m - 1u)
+            rank += __shfl_sync(full, key, __ffs(m) - 1) < key;
+        const uint32_t base = O.claim(w, a, n);
+        if (keep)
+            O.put(a, base + rank, key, v);
+    }
+    if (n_c > 32u)
+        put_bits(w, a, O, tile, bits, words);
+}
+
+// A finished tile to M_H: whole 16 bytes as one bulk copy, which the crew's first
+// thread issues, up to three words on either side by hand.
+template <class C>
+__device__ __forceinline__ void send_tile(uint32_t *dst, const uint32_t *tile, uint64_t cell0, uint32_t cells)
+{
+    const uint32_t head = min((uint32_t)(-cell0 & 3u), cells), mid = (cells - head) & ~3u, rank = C::rank();
+    if (rank == 0) {
+        if (mid)
+            bulk_store_evict_first(dst + head, tile + head, mid * 4u);
+        bulk_commit();
+    }
+    if (rank < cells - mid) {
+        const uint32_t k = rank < head ? rank : mid + rank;
+        dst[k] = tile[k];
+    }
+}
+
+// Pass `pass` of unit `unit`, whose hits are the list entries off.x .. off.y.
+__device__ __forceinline__ TilePass tile_pass(const Geom &g, const Work &w, const TileCfg &c, uint32_t pass,
+                                              uint32_t unit, uint2 off)
+{
+    TilePass P;
+    P.iA = (pass - unit * c.strips) * c.W;
+    P.pr = min(c.W, g.na - P.iA);
+    P.lines = w.lines + off.x;
+    P.recs = w.list + off.x;
+    P.nc = off.y - off.x;
+    return P;
+}
+
+__device__ __forceinline__ PassOut pass_out(const Geom &g, const TilePass &P, uint32_t pass, uint32_t unit)
+{
+    const uint32_t e = unit / g.n_slices;
+    return PassOut{e, ((unit - e * g.n_slices) * g.na + P.iA) * g.nb, pass};
+}
+
+// Passes of units with more hits than this are left to whole CTAs (team_passes):
+// such a pass is more than the fair share of one of the grid's warps, so the
+// others would end long before it.
+__device__ __forceinline__ uint32_t team_limit(const Geom &g, const Work &w, const TileCfg &c)
+{
+    const uint64_t total = __ldcg(&w.slice_off[w.n_events * g.n_slices]);
+    const uint64_t share = total * c.strips / (c.team_share * gridDim.x);
+    return (uint32_t)min(max(share, (uint64_t)kTeamHits), (uint64_t)0xffffffffu);
+}
+
+// The passes of units with more than `limit` hits, each by all warps of a CTA in
+// the first warp's tile: the votes, and the look at every cell, are dealt out to
+// the warps.  The passes are numbered over those units in order and handed out by
+// a counter.  Out of line: most launches have none.
+//
+// Crowded slices are bound by one warp's chain of votes, and by its look at the
+// rows beyond the pass, unless they are dealt out so (us per event, one warp per
+// pass / this): 16384 hits in one slice of 128 x 4096 bins, threshold 3, 620 / 73,
+// peaks only, threshold 10, 4568 / 67; 4 slices of 16 x 1024 bins with 4096 hits each,
+// threshold 3, 161 / 43; 64 slices of 128 x 4096 bins with 4096 hits each, peaks only,
+// threshold 10, 3508 / 381.
+template <bool STORE>
+__device__ __noinline__ void team_passes(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a,
+                                         uint32_t limit, uint32_t *tile0, uint32_t spare0, uint32_t *s_word)
+{
+    const uint32_t nb = g.nb, tid = threadIdx.x, U = w.n_events * g.n_slices;
+    uint32_t *bits = tile0 + c.tile_words;
+    PassList &L = *reinterpret_cast<PassList *>(bits + tile_bit_words(c.tile_words));
+    uint32_t *scratch = c.warps > 1u ? tile0 + tile_warp_words(c.tile_words) : nullptr;   // the second warp's tile
+    auto claim = [&]() {
+        __syncthreads();   // the last claim is read, the tile clear
+        if (tid == 0)
+            *s_word = atomicAdd(&w.ctr[CTR_TEAM], 1u);
+        __syncthreads();
+        return *s_word;
+    };
+    auto vote_pass = [&](uint32_t unit, uint32_t strip) {
+        const uint32_t pass = unit * c.strips + strip;
+        const TilePass P = tile_pass(g, w, c, pass, unit,
+                                     make_uint2(__ldcg(&w.slice_off[unit]), __ldcg(&w.slice_off[unit + 1u])));
+        const uint64_t cell0 = (uint64_t)unit * ((uint64_t)g.na * nb) + (uint64_t)P.iA * nb;
+        const uint32_t shift = (uint32_t)(cell0 & 3u);
+        uint32_t *tile = tile0 + shift;
+        float2 l[kAhead];
+        crew_lines<CtaCrew>(l, P.lines, P.nc);
+        if (P.pr > 2u)
+            vote_tile<false, 4, CtaCrew>(g, tile, P, l, L, spare0 - shift);
+        else
+            vote_tile<false, 2, CtaCrew>(g, tile, P, l, L, spare0 - shift);
+        if (STORE)
+            fence_proxy_async_smem();
+        __syncthreads();
+        if (STORE)
+            send_tile<CtaCrew>(w.M + cell0, tile, cell0, P.pr * nb);
+        const bool here = !(STORE && c.edges_later);   // the rows beyond are compared here
+        if (L.n)
+            search_cells<CtaCrew, true>(g, w, a, P, pass_out(g, P, pass, unit), tile, bits, here && P.iA > 0,
+                                        here && P.iA + P.pr < g.na, STORE, scratch);
+        else if (tid == 0)
+            w.pass_peaks[pass] = make_uint2(0u, 0u);
+        if (STORE && tid == 0)
+            bulk_wait_read<0>();
+        __syncthreads();
+        if (tid == 0)
+            L.n = 0u;
+        for (uint32_t q = tid; q < c.tile_words / 4u; q += blockDim.x)
+            reinterpret_cast<uint4 *>(tile0)[q] = make_uint4(0u, 0u, 0u, 0u);
+    };
+    auto crowded = [&](uint32_t u) {
+        return u < U && __ldcg(&w.slice_off[u + 1u]) - __ldcg(&w.slice_off[u]) > limit;
+    };
+    uint32_t mine = ~0u, before = 0;   // the claimed pass; the passes of the crowded units so far
+    for (uint32_t u0 = 0; u0 < U; u0 += 32u) {
+        if (u0 % blockDim.x == 0) {   // a block's width of units at once: mostly none is crowded
+            if (!__syncthreads_or(crowded(u0 + tid))) {
+                u0 += blockDim.x - 32u;
+                continue;
+            }
+            if (mine == ~0u)
+                mine = claim();
+        }
+        uint32_t m = __ballot_sync(0xffffffffu, crowded(u0 + (tid & 31u)));
+        for (; m; m &= m - 1u, before += c.strips)
+            for (; mine - before < c.strips; mine = claim())
+                vote_pass(u0 + (uint32_t)(__ffs(m) - 1), mine - before);
+    }
+    if (STORE && tid == 0)
+        bulk_wait<0>();
 }
 
 // STORE: the tiles go to M_H, else the peaks are all that is wanted (the same
@@ -2311,25 +2581,29 @@ __device__ __forceinline__ void pass_search(const Geom &g, const Work &w, const 
 // went through rows in global memory and k_peaks, 31.8 and 31.5 us).  AGG:
 // warp-aggregated vote increments (vote_tile).  passes: over all events; runs:
 // runs of c.run passes per CTA, the passes behind them being handed out.
-template <bool STORE, bool AGG>
+template <bool STORE, bool AGG, bool TEAM>
 __global__ void __launch_bounds__(kTileWarps * 32, 2) k_fill_tma(const __grid_constant__ Geom g,
-                                                              const __grid_constant__ Work w, const TileCfg c,
+                                                              const __grid_constant__ Work w,
+                                                              const __grid_constant__ TileCfg c,
                                                               const __grid_constant__ ScanArgs a, uint32_t passes,
                                                               uint32_t runs)
 {
     extern __shared__ uint4 sm4[];
-    // layout: per warp a tile, its bits, its list and 32 idle words
-    __shared__ uint32_t s_left;
-    const uint32_t nb = g.nb, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, warps = blockDim.x >> 5;
+    // layout: per tile warp a tile, its bits, its list and 32 idle words.  (TEAM: warps
+    // beyond those only take part in team_passes.)
+    __shared__ uint32_t s_word;   // warps with passes to come; TEAM: team_passes' claim
+    const uint32_t nb = g.nb, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t warps = TEAM ? c.warps : blockDim.x >> 5;
     const uint32_t mine = tile_warp_words(c.tile_words);
-    uint32_t *tile0 = reinterpret_cast<uint32_t *>(sm4) + warp * mine;
+    uint32_t *tile0 = reinterpret_cast<uint32_t *>(sm4) + (TEAM ? warp % warps : warp) * mine;
     uint32_t *bits = tile0 + c.tile_words;
     PassList &L = *reinterpret_cast<PassList *>(bits + tile_bit_words(c.tile_words));
     const uint32_t *idle = reinterpret_cast<uint32_t *>(&L) + tile_list_words() + lane;   // the lane's own word
-    for (uint32_t k = lane; k < mine / 4u; k += 32u)
-        reinterpret_cast<uint4 *>(tile0)[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (!TEAM || warp < warps)
+        for (uint32_t k = lane; k < mine / 4u; k += 32u)
+            reinterpret_cast<uint4 *>(tile0)[k] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0)
-        s_left = warps;
+        s_word = warps;
     __syncthreads();
     grid_dep_wait();   // the unit lists
 
@@ -2356,75 +2630,71 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) k_fill_tma(const __grid_co
     };
     // The next pass's lines are loaded while this one's tile leaves, and the
     // offsets of the one behind it: nothing that a pass begins with is waited for.
-    uint32_t pass = next_pass(), next = next_pass();
+    const bool idler = TEAM && warp >= warps;
+    uint32_t pass = idler ? passes : next_pass(), next = idler ? passes : next_pass();
     uint2 off = offsets(pass), next_off = offsets(next);
+    const uint32_t limit = TEAM ? team_limit(g, w, c) : 0u;
     float2 l[kAhead];
     first_lines(l, w.lines + off.x, off.y - off.x);
     while (pass < passes) {
         const uint32_t unit = pass / c.strips;
-        TilePass P;
-        P.iA = (pass - unit * c.strips) * c.W;
-        P.pr = min(c.W, g.na - P.iA);
-        P.lines = w.lines + off.x;
-        P.recs = w.list + off.x;
-        P.nc = off.y - off.x;
+        const TilePass P = tile_pass(g, w, c, pass, unit, off);
+        const bool team = TEAM && P.nc > limit;   // left to team_passes
         // the pass's first cell lies in the tile as in M_H: at the same address modulo 16 bytes
         const uint64_t cell0 = (uint64_t)unit * ((uint64_t)g.na * nb) + (uint64_t)P.iA * nb;
         uint32_t *tile = tile0 + (uint32_t)(cell0 & 3u);
-        const uint32_t spare = (uint32_t)(idle - tile);
-        if (P.pr > 2u)
-            vote_tile<AGG, 4>(g, tile, P, l, L, spare);
-        else
-            vote_tile<AGG, 2>(g, tile, P, l, L, spare);
-        if (STORE)
-            fence_proxy_async_smem();   // this lane's counts, visible to the copy engine
-        __syncwarp();
-        // ---- the pass leaves: whole 16 bytes as one bulk copy, up to three words on either side by hand
-        if (STORE) {
-            const uint32_t cells = P.pr * nb, head = min((uint32_t)(-cell0 & 3u), cells), mid = (cells - head) & ~3u;
-            uint32_t *dst = w.M + cell0;
-            if (lane == 0) {
-                if (mid)
-                    bulk_store_evict_first(dst + head, tile + head, mid * 4u);
-                bulk_commit();
-            }
-            if (lane < cells - mid) {
-                const uint32_t k = lane < head ? lane : mid + lane;
-                dst[k] = tile[k];
-            }
+        if (!team) {
+            const uint32_t spare = (uint32_t)(idle - tile);
+            if (P.pr > 2u)
+                vote_tile<AGG, 4, WarpCrew>(g, tile, P, l, L, spare);
+            else
+                vote_tile<AGG, 2, WarpCrew>(g, tile, P, l, L, spare);
+            if (STORE)
+                fence_proxy_async_smem();   // this lane's counts, visible to the copy engine
+            __syncwarp();
+            // ---- the pass leaves
+            if (STORE)
+                send_tile<WarpCrew>(w.M + cell0, tile, cell0, P.pr * nb);
         }
         first_lines(l, w.lines + next_off.x, next_off.y - next_off.x);
         const uint32_t next2 = next_pass();
         const uint2 next2_off = offsets(next2);
-        // ---- its peaks
-        if (L.n)
-            pass_search(g, w, a, P, pass, unit, tile, L, bits, STORE, STORE && c.edges_later);
-        else if (lane == 0)
-            w.pass_peaks[pass] = make_uint2(0u, 0u);
-        // ---- the tile is cleared once the copy has read it
-        if (STORE && lane == 0)
-            bulk_wait_read<0>();
-        __syncwarp();
-        if (lane == 0)
-            L.n = 0u;
+        if (!team) {
+            // ---- its peaks
+            if (L.n)
+                pass_search<TEAM>(g, w, a, P, pass_out(g, P, pass, unit), tile, L, bits, STORE, STORE && c.edges_later);
+            else if (lane == 0)
+                w.pass_peaks[pass] = make_uint2(0u, 0u);
+            // ---- the tile is cleared once the copy has read it
+            if (STORE && lane == 0)
+                bulk_wait_read<0>();
+            __syncwarp();
+            if (lane == 0)
+                L.n = 0u;
 #pragma unroll 8
-        for (uint32_t k = lane; k < c.tile_words / 4u; k += 32u)
-            reinterpret_cast<uint4 *>(tile0)[k] = make_uint4(0u, 0u, 0u, 0u);
-        __syncwarp();
+            for (uint32_t k = lane; k < c.tile_words / 4u; k += 32u)
+                reinterpret_cast<uint4 *>(tile0)[k] = make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+        }
         pass = next;
         off = next_off;
         next = next2;
         next_off = next2_off;
     }
-    if (lane == 0) {
-        if (STORE)
-            bulk_wait<0>();   // the warp's copies have written M_H (and read its tile) before the CTA ends
-        if (atomicSub(&s_left, 1u) == 1u) {
-            __threadfence();
-            if (atomicAdd(&w.ctr[CTR_DYN_DONE], 1u) == gridDim.x - 1) {   // nobody claims any more
-                w.ctr[CTR_DYN] = 0u;
-                w.ctr[CTR_DYN_DONE] = 0u;
-            }
+    if (STORE && lane == 0)
+        bulk_wait<0>();   // the warp's copies have written M_H (and read its tile) before the CTA ends
+    if (TEAM) {
+        __syncthreads();
+        team_passes<STORE>(g, w, c, a, limit, reinterpret_cast<uint32_t *>(sm4),
+                           (uint32_t)(idle - reinterpret_cast<uint32_t *>(sm4)), &s_word);
+    }
+    if (TEAM ? tid == 0 : lane == 0 && atomicSub(&s_word, 1u) == 1u) {
+        __threadfence();
+        if (atomicAdd(&w.ctr[CTR_DYN_DONE], 1u) == gridDim.x - 1) {   // nobody claims any more
+            w.ctr[CTR_DYN] = 0u;
+            w.ctr[CTR_DYN_DONE] = 0u;
+            if (TEAM)
+                w.ctr[CTR_TEAM] = 0u;
         }
     }
 }
@@ -2804,8 +3074,10 @@ using TileKernel = void (*)(Geom, Work, TileCfg, ScanArgs, uint32_t, uint32_t);
 static TileKernel tile_kernel(const TileCfg &c, bool store)
 {
     if (!store)
-        return k_fill_tma<false, false>;
-    return c.vote_agg ? k_fill_tma<true, true> : k_fill_tma<true, false>;
+        return c.team_share ? k_fill_tma<false, false, true> : k_fill_tma<false, false, false>;
+    if (c.vote_agg)
+        return c.team_share ? k_fill_tma<true, true, true> : k_fill_tma<true, true, false>;
+    return c.team_share ? k_fill_tma<true, false, true> : k_fill_tma<true, false, false>;
 }
 
 cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, const ScanArgs &a, uint32_t grid,
@@ -2823,7 +3095,7 @@ cudaError_t launch_fill_tma(const Geom &g, const Work &w, const TileCfg &c, cons
     const uint32_t passes = (uint32_t)tile_passes(g, c, w.n_events);
     const uint32_t handed = std::max(kHandedOut * c.warps * grid, passes / 8u);
     const uint32_t runs = passes > handed ? (passes - handed) / (grid * c.run) : 0u;
-    return launch_pdl(k, grid, c.warps * 32u, smem, st, g, w, c, a, passes, runs);
+    return launch_pdl(k, grid, (c.team_share ? kTileWarps : c.warps) * 32u, smem, st, g, w, c, a, passes, runs);
 }
 
 cudaError_t fill_tma_occupancy(const TileCfg &c, bool store, int *blocks_per_sm)

@@ -33,7 +33,7 @@ struct Runner {
         uint32_t n_events;
         bool to_host;
         uint32_t fill_flags;         // HT_PEAKS_ONLY, HT_FILL_NAIVE or 0
-        bool edges;                  // the fill is followed by k_edges
+        uint32_t how;                // engine_fill_kind
         cudaGraphExec_t exec;
     };
     std::vector<Graph> graphs;

@@ -188,3 +188,71 @@ def test_high_tiles_leave_the_sm_its_warps(ht, peaks_only):
             assert n == n_want
             assert_peaks_equal(pk, want)
         assert max(times.values()) < 1.4 * times[8], times
+
+
+def _one_slice(n, seed, phi=0.32):
+    """n hits with one azimuth and one polar angle, as good as."""
+    g = np.random.default_rng(seed)
+    rad, ph, z = g.uniform(20, 1100, n), g.uniform(phi - 0.01, phi + 0.01, n), g.uniform(5, 12, n)
+    return [a.astype(np.float32) for a in (rad * np.cos(ph), rad * np.sin(ph), z)]
+
+
+# (n_theta, n_phi, n_a, n_b), uniform hits, hits in one slice, thresholds
+CROWDED = [
+    ((1, 1, 1, 64), 3000, 0, (2, 60)), ((1, 1, 2, 4096), 5000, 0, (1, 3)), ((1, 1, 3, 7), 2500, 0, (2, 500)),
+    ((1, 2, 5, 1023), 4000, 0, (3, 9)), ((2, 2, 33, 200), 9000, 0, (4, 40)), ((1, 4, 129, 64), 8000, 0, (5, 80)),
+    ((4, 10, 6, 333), 60000, 0, (6, 12)), ((3, 30, 41, 48), 100, 4000, (2, 30)), ((2, 3, 300, 1024), 900, 6000, (3, 5)),
+    ((1, 1, 5, 64), 70000, 0, (40, 1500)), ((1, 64, 4, 96), 0, 513, (2, 9)), ((1, 64, 4, 96), 0, 512, (2, 9)),
+]
+
+
+@pytest.mark.parametrize("rows", [0, 1, 16], ids=lambda r: f"rows{r}")
+@pytest.mark.parametrize("shape", CROWDED, ids=[str(s[:3]) for s in CROWDED])
+def test_units_voted_by_whole_ctas(ht, shape, rows):
+    """Units of so many hits that their passes are the whole CTA's: few rows and
+    many hits, one crowded slice among sparse ones, more than 32 of them, on
+    either side of the number of hits (512) that this begins at."""
+    bins, n, one, thresholds = shape
+    b, r = ht.Binning(*bins), ht.Ranges()
+    parts = [random_hits(n, n + 1, rmax=900.0), _one_slice(one, one + 2)]
+    x, y, z = (np.concatenate(v) for v in zip(*parts))
+    M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+    for T in thresholds:
+        pk_ref, n_ref = oracle.find_maxima(_ob(b), _orr(r), M_ref, T, cap=1 << 18)
+        with ht.Context(b, r, threshold=T, max_hits=x.size) as ctx:
+            ctx.set_tuning(fill_rows=rows)
+            for po in (False, True, False, True):
+                ctx.fill(x, y, z, peaks_only=po)
+                pk, total = ctx.find_maxima(capacity=1 << 18)
+                assert total == n_ref, (T, po)
+                assert_peaks_equal(pk, pk_ref)
+            assert np.array_equal(ctx.matrix(), M_ref)
+            ctx.fill(x[:40], y[:40], z[:40])   # and a sparse fill after them
+            M, _ = oracle.fill(_ob(b), _orr(r), x[:40], y[:40], z[:40])
+            assert np.array_equal(ctx.matrix(), M)
+
+
+def test_crowded_unit_in_a_batch(ht):
+    """The crowded slice is the last event's, the first's, or each one's; sparse
+    and crowded runs take turns on the captured graphs."""
+    b, r, T = ht.Binning(2, 16, 30, 100), ht.Ranges(), 6
+    sparse = [random_hits(40 + 30 * k, 300 + k, rmax=900.0) for k in range(5)]
+    crowd = _one_slice(3000, 4)
+    runs = [sparse, sparse[:4] + [crowd], [crowd] + sparse[:4], [crowd] * 5]
+    refs = []
+    for evs in runs:
+        ref = []
+        for x, y, z in evs:
+            M_ref, _ = oracle.fill(_ob(b), _orr(r), x, y, z)
+            ref.append((M_ref, *oracle.find_maxima(_ob(b), _orr(r), M_ref, T)))
+        refs.append(ref)
+    with ht.Batch(b, r, threshold=T, max_events=5, max_hits=1 << 15, capacity=1 << 17) as B:
+        for rep in range(3):
+            for po in (False, True):
+                for evs, ref in zip(runs, refs):
+                    pk, counts = B.run(*ht.Batch.concat(evs), peaks_only=po)
+                    assert list(counts) == [q[2] for q in ref]
+                    assert_peaks_equal(pk, np.concatenate([q[1] for q in ref]))
+                    if not po:
+                        for e in (0, 4):
+                            assert np.array_equal(B.matrix(e), ref[e][0])
