@@ -272,8 +272,8 @@ ht_status ht_profile_read(ht_ctx *ctx, ht_kernel_time *out, uint32_t cap, uint32
  *                      n_b a multiple of 4); 2: never (a full scan in
  *                      ht_find_maxima); 0: the tile fill for n_b up to 4096
  *                      when it fits (ht_get_tuning then reports 5, or 0 when
- *                      n_b is not a multiple of 4), else 1, when it fits
- *                      (the fused modes only for non-accumulating, non-naive
+ *                      n_b is not a multiple of 4), else 2 (the fused modes
+ *                      only for n_b up to 4096 and non-accumulating, non-naive
  *                      fills)
  *   fill_vote_agg      1: the tile fill of M_H (fill_fused_scan 5)
  *                      aggregates the vote increments of a warp -- lanes

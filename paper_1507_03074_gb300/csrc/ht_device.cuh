@@ -26,7 +26,7 @@ struct Geom {
     uint32_t max_admit;     // slices one hit can enter
     uint32_t threshold;
     float a_min, b_min, da, db, nbf;
-    float inv_db;           // 1 / dB, only to estimate a bin before the exact table test
+    float inv_db;           // 1 / dB, only to estimate a bin before the exact table test (k_fill_naive)
     // the linear model of a hit's votes (see vote_line): -2 dA / dB, -2 A of
     // the A bin mid = n_a / 2, and 1 / dB, each as a sum of two floats, and
     // the bound of the model's error in bins, err_v |v| + 0.5 - err_half
@@ -147,23 +147,6 @@ __device__ __forceinline__ uint32_t bin_code(const Geom &g, const float *et, con
     return (edge_bin(dt, et, g.nt) << 16) | edge_bin(dp, ep, g.np);
 }
 
-// Is slice (ts, ps) among the slices a hit of bin code `code` votes in: its
-// own bin, +-win_theta (clipped), +-win_phi (cyclic on the full circle,
-// clipped otherwise), each slice at most once.
-__device__ __forceinline__ bool admits(const Geom &g, uint32_t code, uint32_t ts, uint32_t ps)
-{
-    if (code == kDropped)
-        return false;
-    const uint32_t it = code >> 16, ip = code & 0xffffu;
-    const uint32_t dt = ts > it ? ts - it : it - ts;
-    if (dt > g.wt)
-        return false;
-    uint32_t dp = ps > ip ? ps - ip : ip - ps;
-    if (g.phi_full && g.np - dp < dp)
-        dp = g.np - dp;
-    return dp <= g.wp;
-}
-
 // Visit every slice id (itheta * n_phi + iphi) a hit of bin code `code` votes in.
 template <class F>
 __device__ __forceinline__ void for_each_slice(const Geom &g, uint32_t code, F &&f)
@@ -233,8 +216,8 @@ __device__ __forceinline__ int bin_from_thresholds(const Geom &g, const float *b
     return j;
 }
 
-// The vote of one (hit, A bin) with the threshold table: B = (r2 - (2A) x) / d
-// by IEEE division, then its bin (or -1).
+// The vote of one (hit, A bin) with the threshold table (k_fill_naive): B = (r2 -
+// (2A) x) / d by IEEE division, then its bin (or -1).
 __device__ __forceinline__ int vote_bin_tab(const Geom &g, const float *beta, float b_lo, float b_hi, float twoA,
                                             float x, float r2, float d)
 {

@@ -13,7 +13,7 @@ static uint32_t round_up(uint32_t v, uint32_t m) { return (v + m - 1) / m * m; }
 
 static const size_t kSmemMax = 227 * 1024;     // per CTA on sm_100-class parts
 static const uint32_t kScanThreads = 256;
-static const uint32_t kPeakBuf = 1024;         // K: entries buffered per scan / seam CTA
+static const uint32_t kPeakBuf = 1024;         // K: entries buffered per scan CTA
 static const uint32_t kFusedPeakBuf = 512;     // K of a fused-fill CTA (at least its block)
 
 const char *const kKernelNames[K_NKINDS] = {"k_bin", "k_scatter", "k_fill_priv", "k_fill_scan", "k_fill_ws",
@@ -208,8 +208,7 @@ ht_status engine_configure(Engine &E, std::string *why)
     E.bin_cluster = htk::bin_cluster_supported(htk::kBinClusterSmem) ? 1 : 0;
 
     // --- fused fill + maxima ---------------------------------------------------
-    // A smaller peak buffer than the scan's (the tile needs the room); k_seam
-    // keeps kPeakBuf in its own launch.
+    // A smaller peak buffer than the scan's (the tile needs the room).
     E.fused_ok = false;
     E.fused_K = std::max<uint32_t>(kFusedPeakBuf, f.threads);
     if (E.fill_priv_ok && t.fused != 2 && W <= 64 && b.n_b <= 4096) {

@@ -12,7 +12,8 @@
 //                 A-rows into a u32 shared-memory tile of its own, laid out as
 //                 M_H's rows, which leaves as one bulk copy; a vote taking a
 //                 cell to T lists it, and the warp tests the listed cells in
-//                 its tile.  k_order_passes puts the peaks in order.
+//                 its tile.  Units of many hits are left to whole CTAs
+//                 (team_passes).  k_order_passes puts the peaks in order.
 //   k_edges       Crowded tile fills: peaks against the rows of other passes.
 //   k_fill_add    Accumulating fills of few hits: a reduction per vote.
 //   k_copy        M_H into the caller's device memory.
@@ -1985,6 +1986,10 @@ __global__ void __launch_bounds__(256) k_order(Geom g, Work w, ScanArgs a, Order
 // the votes of the row beyond are counted from the unit's lines (nothing waits
 // for the warp that owns it), or k_edges compares them later.  Each pass leaves
 // {first entry, count} in pass_peaks, in pass order, for k_order_passes.
+//
+// Where slices may be so crowded that their passes outlast the rest (TEAM, chosen
+// by the host), passes above a share of the votes wait until a CTA's warps have no
+// other pass, and then take all of them (team_passes).
 //
 // Bound: writing M_H where votes are few (paper event, one launch: 42 us for
 // 268 MB, 54 MB of which reach HBM, as M_H is compressed; upgrade event, in
